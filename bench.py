@@ -194,7 +194,7 @@ def kernel_qgemm(args, torch, qpinv):
     gms = st["%s_gemm_ms" % key]
     kname = "k_qgemm_tc"
     if key == "emu":
-        kname = "k_qgemm_emu_pair" if args.emu_pair == "1" else "k_qgemm_emu"
+        kname = "k_qgemm_emu"
     print(json.dumps({"kernel": kname, "n": n, "precision": prec,
                       "split": args.split, "launches_per_product": launches / args.steps, "ms_per_launch": gms / launches,
                       "gemm_ms_per_product": gms / args.steps,

@@ -140,11 +140,9 @@ typedef struct {
                         runs in the GEMM's epilogue, on FP32 masters and, in the FP64 polish
                         steps, on FP64 masters (passes that carry FP64 stop norms excepted);
                         0: separate combine kernel (same arithmetic) */
-  int emu_pair;      /* 1: FP64-accurate exact-slice products with more than 128 rows on pairs of SMs
-                        (256 x 64 tiles, one MMA for both CTAs, half of the B operand staged per SM);
-                        0 or -1 (default): one SM per 128 x 128 tile and component pair, which was
-                        measured faster at every size (5.3 against 7.3 ms at 2048^3, 44.9 against
-                        58.3 ms at 4096^3, 8 slices).  Same arithmetic, bit-identical results */
+  int emu_pair;      /* -1 (default), 0 or 1: accepted for callers that set it, without effect.  It
+                        chose between two exact-slice kernels with bit-identical results; one kernel,
+                        faster than both at every size, has replaced them */
   int tc_broad;      /* BF16-split products with M, N >= 128 and one accumulator on 128-column tiles
                         (one CTA per SM, a 512-column TMEM accumulator) or 64-column tiles (two CTAs
                         per SM): -1 (default) 128 columns for products without a fused combine

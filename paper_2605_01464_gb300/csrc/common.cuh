@@ -42,24 +42,19 @@ struct Split16 {
 // Output specification of the fused combine kernel:
 //   out = cacc * acc + sum_t caux[t] * aux_t + diag * I   (diag on plane s)
 // The master output (and every aux input) has the master type of the pass:
-// float (tensor-core phase) or double (FP64 phase).  BF16 outputs are either
+// float (tensor-core phase) or double (FP64 phase).  BF16 outputs are
 // round-to-nearest splits of the FP32 value (t0 = bf16(v), t1 = bf16(v - t0),
-// ...) or, when exp_a / exp_b are given, exact 7-bit slices of v * 2^-e
-// (e = exponent of the row (A-form) or column (B-form) maximum): slice s is
-// an integer in [-64, 64] ([-128, 128] for s = 0) times 2^(-7(s+1)), which
-// BF16 holds exactly.  Slicing is done in integer arithmetic.
+// ...).
 struct OutSpec {
   void* mp = nullptr;  // master output planes (type of the pass), may be null
   long mld = 0, mps = 0;
   Split16 s16;         // BF16 outputs (a and/or b may be null)
-  const int* exp_a = nullptr;  // per-row exponents: exact slicing of the A-form
-  const int* exp_b = nullptr;  // per-column exponents: exact slicing of the B-form
   double cacc = 0.0;
   double caux[4] = {0, 0, 0, 0};
   double diag = 0.0;
 };
 
-enum { ACC_F32 = 0, ACC_F64 = 1, ACC_I64 = 2 };
+enum { ACC_F32 = 0, ACC_F64 = 1, ACC_Q8 = 2 };
 
 constexpr int kMaxOut = 3;
 
@@ -67,8 +62,11 @@ struct CombineArgs {
   int rows = 0, cols = 0;
   int f64 = 0;                // master type of aux inputs and outputs: 0 float, 1 double
   const void* acc = nullptr;  // accumulator planes, may be null
-  const long long* acc2 = nullptr;  // ACC_I64: a second accumulator of the same layout, summed
-  int acc_kind = ACC_F32;     // ACC_I64: fixed point, value = acc * 2^(erow[i] + ecol[j] - shift)
+  // ACC_Q8: the eight real products of the exact-slice GEMM (qgemm_emu.cu),
+  // int64 planes [set][8], the sets summed; twice a component is an integer
+  // combination q of them, its value q * 2^(erow[i] + ecol[j] - shift)
+  int acc_kind = ACC_F32;
+  int acc_sets = 1;
   long ld_acc = 0, ps_acc = 0;
   const int* acc_erow = nullptr;
   const int* acc_ecol = nullptr;
@@ -105,28 +103,30 @@ cudaError_t launch_antiherm_partials(const Planes<const double>& M, int n, doubl
                                      cudaStream_t st, int* blocks_out);
 cudaError_t launch_init_x0(const Planes<const double>& A, int m, int n, double alpha, const Planes<double>& X,
                            cudaStream_t st);
-// by_col needs `scratch` of COL_SCRATCH(cols) ints
-cudaError_t launch_maxexp_f32(const Planes<const float>& A, int rows, int cols, int by_col, int* e, int* scratch,
-                              cudaStream_t st);
+// Column exponents e (|v| < 2^e over the four planes); `scratch`: COL_SCRATCH(cols) ints
+cudaError_t launch_maxexp(const Planes<const float>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st);
 cudaError_t launch_f64_to_f32(const Planes<const double>& src, int rows, int cols, const Planes<float>& dst,
                               cudaStream_t st);
-cudaError_t launch_maxexp(const Planes<const double>& A, int rows, int cols, int by_col, int* e, int* scratch,
-                          cudaStream_t st);
+cudaError_t launch_maxexp(const Planes<const double>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st);
 cudaError_t launch_f32_to_f64(const Planes<const float>& src, int rows, int cols,
                               const Planes<double>& dst, cudaStream_t st);
 
-// Exact slices (S balanced 7-bit digits of v * 2^-e) of a row-major plane
-// set: A-form rows (row exponents e[i]; dst [S][4][rows][ld]) or the
-// transposed B-form (column exponents e[j]; dst [S][4][cols][ld]); padding
-// up to the next multiple of 8 along the slice rows is written as 0.
-cudaError_t launch_slice_rows(const Planes<const double>& A, int rows, int cols, const int* e, int S, bf16* dst,
-                              long ld, long ps, cudaStream_t st);
-cudaError_t launch_slice_rows(const Planes<const float>& A, int rows, int cols, const int* e, int S, bf16* dst,
-                              long ld, long ps, cudaStream_t st);
-cudaError_t launch_slice_cols(const Planes<const double>& A, int rows, int cols, const int* e, int S, bf16* dst,
-                              long ld, long ps, cudaStream_t st);
-cudaError_t launch_slice_cols(const Planes<const float>& A, int rows, int cols, const int* e, int S, bf16* dst,
-                              long ld, long ps, cudaStream_t st);
+// Exact slices for the eight-product exact-slice GEMM (qgemm_emu.cu): S
+// balanced 7-bit digits of v * 2^-e per component (slice s an integer in
+// [-64, 63], [-128, 128] for s = 0, of weight 2^-7(s+1)), stored as the BF16
+// digit sums of products p0 .. p0 + np - 1: dst [S][np][rows][ld].
+// Rows: A-form with the left combinations; the row exponents are found and
+// written to e.  Cols: the transposed B-form, dst [S][np][cols][ld], with the
+// right combinations and given column exponents (launch_maxexp).  Padding up
+// to the next multiple of 8 along the slice rows is written as 0.
+cudaError_t launch_slice_rows(const Planes<const double>& A, int rows, int cols, int* e, int S, int p0, int np,
+                              bf16* dst, long ld, long ps, cudaStream_t st);
+cudaError_t launch_slice_rows(const Planes<const float>& A, int rows, int cols, int* e, int S, int p0, int np,
+                              bf16* dst, long ld, long ps, cudaStream_t st);
+cudaError_t launch_slice_cols(const Planes<const double>& A, int rows, int cols, const int* e, int S, int p0, int np,
+                              bf16* dst, long ld, long ps, cudaStream_t st);
+cudaError_t launch_slice_cols(const Planes<const float>& A, int rows, int cols, const int* e, int S, int p0, int np,
+                              bf16* dst, long ld, long ps, cudaStream_t st);
 
 cudaError_t launch_qgemm_f64(int M, int K, int N, const Planes<const double>& A,
                              const Planes<const double>& B, const Planes<double>& C,
@@ -166,17 +166,11 @@ int tc_partial_blocks(int M, int N, int broad);
 // the listed (i, j) term pairs of A_i * B_j, restricted to k in [k0, k1).
 struct TcGemmArgs {
   int M = 0, N = 0, K = 0;
-  // Output: FP32 store into C, or (C64 != null) int64 fixed-point
-  // accumulation C64 += rint(acc * 2^shift).
-  long long* C64 = nullptr;
-  long ld64 = 0, ps64 = 0;
-  int shift = 0;
   int k0 = 0, k1 = 0;
   const Split16* A = nullptr;  // uses the A-form
   const Split16* B = nullptr;  // uses the B-form
   int npairs = 0;
   int pair_i[16] = {0}, pair_j[16] = {0};
-  int pair_acc[16] = {0};  // TMEM accumulator of each pair (1 only with C64: the two are summed)
   Planes<float> C;  // FP32 output
   EpiArgs epi;      // epi.nout > 0: fused combine instead of the plain store (FP32 output only)
   int broad = -1;   // one-accumulator products with N >= 128 on 128-column tiles (one CTA per SM):
@@ -186,29 +180,25 @@ struct TcGemmArgs {
 cudaError_t launch_qgemm_tc(const TcGemmArgs& a, cudaStream_t st);
 
 // FP64-accurate product from S exact slices per operand in one launch
-// (qgemm_emu.cu): C64 (+ C64b) = sum over levels d < S of the level-d slice
-// products, in 64-bit fixed point (value * 2^shift); the accumulators are
-// written, not added to (no clearing needed).  kc[d] = K chunk of level d
-// (multiple of 32, or >= K), short enough that every FP32 partial sum of the
-// level is exact.  emu_fused_ok(K, S) says whether K is small enough for the
-// kernel's int32 per-level sums.
+// (qgemm_emu.cu).  emu_plan chooses the tile width, the split of an item's
+// levels and K range into parts, and the fixed point; the launch writes the
+// int64 planes C64 [nparts][8][M][ld64] of products p0 .. p0 + np - 1 (units
+// 2^-F; written, not added to).  ld64 and ps64 are multiples of 4.
+struct EmuPlan {
+  int bn = 128, ngroups = 1, nk = 1, nparts = 1;
+  int F = 0;
+};
+EmuPlan emu_plan(int M, int N, int K, int S);
 struct EmuGemmArgs {
   int M = 0, N = 0, K = 0;
-  const Split16* A = nullptr;  // A-form slices (levels >= S)
-  const Split16* B = nullptr;  // B-form slices (levels >= S)
-  int S = 0;
-  int kc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  const Split16* A = nullptr;  // A-form slices of np combinations (levels >= S)
+  const Split16* B = nullptr;  // B-form slices
+  int S = 0, p0 = 0, np = 8;
   long long* C64 = nullptr;
-  long long* C64b = nullptr;  // non-null: a second accumulator (same layout) for half of the levels
   long ld64 = 0, ps64 = 0;
-  int shift = 0;
   int* err = nullptr;
 };
-bool emu_fused_ok(int K, int S);
-cudaError_t launch_qgemm_emu(const EmuGemmArgs& a, cudaStream_t st);
-// The same product on pairs of SMs (qgemm_emu_pair.cu: 256 x 64 tiles,
-// tcgen05 cta_group::2); same arguments and result.
-cudaError_t launch_qgemm_emu_pair(const EmuGemmArgs& a, cudaStream_t st);
+cudaError_t launch_qgemm_emu(const EmuGemmArgs& a, const EmuPlan& plan, cudaStream_t st);
 bool tc_supported();
 
 // Batched solver (batched_impl.cuh: host side in batched.cu, kernels in batched_tile<t>.cu).

@@ -13,6 +13,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace qp {
 
@@ -89,20 +90,6 @@ __device__ __forceinline__ int exp_of(float v) {
   return ex == 0 ? -100000 : ex - 126;
 }
 
-// Exact slices of v * 2^-e (|v| < 2^e): F = round(v * 2^(7S - e)) written in
-// balanced base 128, least significant digit first; slice s = digit_s * 2^-(7(s+1)).
-template <typename T>
-__device__ __forceinline__ void slice_store(bf16* base, long idx, long lstride, int S, T v, int e) {
-  long long F = to_fixed(v, 7 * S - e);
-  for (int l = S - 1; l >= 1; l--) {
-    int d = (int)(F & 127);
-    if (d >= 64) d -= 128;
-    F = (F - d) >> 7;
-    base[l * lstride + idx] = __float2bfloat16_rn(ldexpf((float)d, -7 * (l + 1)));
-  }
-  base[idx] = __float2bfloat16_rn(ldexpf((float)F, -7));
-}
-
 // q 2^e as a double, rounded to nearest (ties to even) from the integer bits:
 // the same value as ldexp((double)q, e), without FP64 arithmetic (GB300's
 // FP64 rate is a small fraction of its integer rate).  Results below the
@@ -126,17 +113,47 @@ __device__ __forceinline__ double i64_scaled(long long q, int e) {
   return __longlong_as_double((long long)(sgn | ((unsigned long long)biased << 52) | (m & 0xFFFFFFFFFFFFFull)));
 }
 
+// Twice the four components from the eight real products of the exact-slice
+// GEMM (see qgemm_emu.cu).  Wrapping arithmetic: a doubled component is below
+// 2^63 in modulus, the partial sums need not be.
+__device__ __forceinline__ void quad_of(const unsigned long long* p, long long* q) {
+  const unsigned long long a = p[4] + p[5], b = p[4] - p[5], c = p[6] + p[7], d = p[6] - p[7];
+  q[0] = (long long)(2 * p[1] - a + c);
+  q[1] = (long long)(2 * p[0] - a - c);
+  q[2] = (long long)(2 * p[2] + b + d);
+  q[3] = (long long)(2 * p[3] + b - d);
+}
 template <typename T>
-__device__ __forceinline__ T acc_value(const CombineArgs& a, int c, int i, int j) {
-  const long off = c * a.ps_acc + (long)i * a.ld_acc + j;
-  if (a.acc_kind == ACC_F64) return (T)((const double*)a.acc)[off];
-  if (a.acc_kind == ACC_I64) {
-    const long long q = ((const long long*)a.acc)[off] + (a.acc2 ? a.acc2[off] : 0LL);
+__device__ __forceinline__ T q8_value(long long q, int e) {
+  if (sizeof(T) == 4) return (T)ldexpf((float)q, e);
+  return (T)i64_scaled(q, e);
+}
+
+// The accumulator's four components at (i, j).
+template <typename T>
+__device__ __forceinline__ void acc_values(const CombineArgs& a, int i, int j, T* v) {
+  const long off = (long)i * a.ld_acc + j;
+  if (a.acc_kind == ACC_Q8) {
+    unsigned long long p[8];
+    const unsigned long long* src = (const unsigned long long*)a.acc + off;
+#pragma unroll
+    for (int t = 0; t < 8; t++) p[t] = src[t * a.ps_acc];
+    for (int s = 1; s < a.acc_sets; s++) {
+      src += 8 * a.ps_acc;
+#pragma unroll
+      for (int t = 0; t < 8; t++) p[t] += src[t * a.ps_acc];
+    }
+    long long q[4];
+    quad_of(p, q);
     const int e = a.acc_erow[i] + a.acc_ecol[j] - a.acc_shift;
-    if (sizeof(T) == 4) return (T)ldexpf((float)q, e);
-    return (T)i64_scaled(q, e);
+#pragma unroll
+    for (int c = 0; c < 4; c++) v[c] = q8_value<T>(q[c], e);
+    return;
   }
-  return (T)((const float*)a.acc)[off];
+#pragma unroll
+  for (int c = 0; c < 4; c++)
+    v[c] = a.acc_kind == ACC_F64 ? (T)((const double*)a.acc)[c * a.ps_acc + off]
+                                 : (T)((const float*)a.acc)[c * a.ps_acc + off];
 }
 
 // cacc x for cacc = +-1 without arithmetic (a sign flip), else the product.
@@ -164,8 +181,10 @@ __global__ void __launch_bounds__(256) k_combine(CombineArgs a) {
       const int i = r0 + ty + q * TROWS, j = c0 + tx;
       T v[4] = {0, 0, 0, 0};
       if (i < a.rows && j < a.cols) {
-        if (a.acc && O.cacc != 0.0)
-          for (int c = 0; c < 4; c++) v[c] = times_coef<T>(acc_value<T>(a, c, i, j), cacc);
+        if (a.acc && O.cacc != 0.0) {
+          acc_values<T>(a, i, j, v);
+          for (int c = 0; c < 4; c++) v[c] = times_coef<T>(v[c], cacc);
+        }
         for (int t = 0; t < 4; t++) {
           if (!a.aux[t] || O.caux[t] == 0.0) continue;
           const T* ap = (const T*)a.aux[t];
@@ -189,8 +208,7 @@ __global__ void __launch_bounds__(256) k_combine(CombineArgs a) {
         if (O.s16.a) {
           for (int c = 0; c < 4; c++) {
             const long idx = c * O.s16.psa + (long)i * O.s16.lda + j;
-            if (O.exp_a) slice_store<T>(O.s16.a, idx, 4 * O.s16.psa, O.s16.levels, v[c], O.exp_a[i]);
-            else split_store(O.s16.a, idx, 4 * O.s16.psa, O.s16.levels, (float)v[c]);
+            split_store(O.s16.a, idx, 4 * O.s16.psa, O.s16.levels, (float)v[c]);
           }
         }
       }
@@ -205,8 +223,7 @@ __global__ void __launch_bounds__(256) k_combine(CombineArgs a) {
           for (int c = 0; c < 4; c++) {
             const long idx = c * O.s16.psb + (long)jj * O.s16.ldb + ii;
             const T val = stage[c][tx][ty + q * TROWS];
-            if (O.exp_b) slice_store<T>(O.s16.b, idx, 4 * O.s16.psb, O.s16.levels, val, O.exp_b[jj]);
-            else split_store(O.s16.b, idx, 4 * O.s16.psb, O.s16.levels, (float)val);
+            split_store(O.s16.b, idx, 4 * O.s16.psb, O.s16.levels, (float)val);
           }
         }
       }
@@ -242,30 +259,57 @@ __device__ __forceinline__ void split_store2(bf16* base, long idx, long lstride,
   }
 }
 
-__device__ __forceinline__ void acc_pair(const CombineArgs& a, int c, int i, int j, bool two, float& x, float& y) {
-  const long off = c * a.ps_acc + (long)i * a.ld_acc + j;
+// The accumulator's four components at (i, j) and (i, j + 1).
+__device__ __forceinline__ void acc_pairs(const CombineArgs& a, int i, int j, bool two, float (*v)[2]) {
+  const long off = (long)i * a.ld_acc + j;
   if (a.acc_kind == ACC_F32) {
-    if (two) {
-      const float2 t = *reinterpret_cast<const float2*>((const float*)a.acc + off);
-      x = t.x;
-      y = t.y;
-    } else {
-      x = ((const float*)a.acc)[off];
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const float* p = (const float*)a.acc + c * a.ps_acc + off;
+      if (two) {
+        const float2 t = *reinterpret_cast<const float2*>(p);
+        v[c][0] = t.x;
+        v[c][1] = t.y;
+      } else {
+        v[c][0] = p[0];
+      }
     }
   } else if (a.acc_kind == ACC_F64) {
-    const double* p = (const double*)a.acc + off;
-    x = (float)p[0];
-    if (two) y = (float)p[1];
-  } else {
-    const long long* p = (const long long*)a.acc + off;
-    long long q0 = p[0], q1 = two ? p[1] : 0;
-    if (a.acc2) {
-      q0 += a.acc2[off];
-      if (two) q1 += a.acc2[off + 1];
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const double* p = (const double*)a.acc + c * a.ps_acc + off;
+      v[c][0] = (float)p[0];
+      if (two) v[c][1] = (float)p[1];
     }
+  } else {
+    // the planes' rows are padded to a multiple of 4: the pair load stays inside
+    unsigned long long p0[8], p1[8];
+    const unsigned long long* src = (const unsigned long long*)a.acc + off;
+#pragma unroll
+    for (int t = 0; t < 8; t++) {
+      const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(src + t * a.ps_acc);
+      p0[t] = u.x;
+      p1[t] = u.y;
+    }
+    for (int s = 1; s < a.acc_sets; s++) {
+      src += 8 * a.ps_acc;
+#pragma unroll
+      for (int t = 0; t < 8; t++) {
+        const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(src + t * a.ps_acc);
+        p0[t] += u.x;
+        p1[t] += u.y;
+      }
+    }
+    long long q0[4], q1[4];
+    quad_of(p0, q0);
+    quad_of(p1, q1);
     const int er = a.acc_erow[i] - a.acc_shift;
-    x = ldexpf((float)q0, er + a.acc_ecol[j]);
-    if (two) y = ldexpf((float)q1, er + a.acc_ecol[j + 1]);
+    const int e0 = er + a.acc_ecol[j], e1 = two ? er + a.acc_ecol[j + 1] : 0;
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      v[c][0] = ldexpf((float)q0[c], e0);
+      if (two) v[c][1] = ldexpf((float)q1[c], e1);
+    }
   }
 }
 
@@ -286,13 +330,14 @@ __global__ void __launch_bounds__(256) k_combine_f2(CombineArgs a) {
       float v[4][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
       const bool in0 = i < a.rows && j < a.cols, two = in0 && j + 1 < a.cols;
       if (in0) {
-        if (a.acc && O.cacc != 0.0)
+        if (a.acc && O.cacc != 0.0) {
+          acc_pairs(a, i, j, two, v);
+#pragma unroll
           for (int c = 0; c < 4; c++) {
-            float x = 0.f, y = 0.f;
-            acc_pair(a, c, i, j, two, x, y);
-            v[c][0] = cacc * x;
-            v[c][1] = cacc * y;
+            v[c][0] *= cacc;
+            v[c][1] *= cacc;
           }
+        }
         for (int t = 0; t < 4; t++) {
           if (!a.aux[t] || O.caux[t] == 0.0) continue;
           const float* ap = (const float*)a.aux[t];
@@ -329,10 +374,7 @@ __global__ void __launch_bounds__(256) k_combine_f2(CombineArgs a) {
         if (O.s16.a)
           for (int c = 0; c < 4; c++) {
             const long idx = c * O.s16.psa + (long)i * O.s16.lda + j;
-            if (O.exp_a) {
-              slice_store<float>(O.s16.a, idx, 4 * O.s16.psa, O.s16.levels, v[c][0], O.exp_a[i]);
-              if (two) slice_store<float>(O.s16.a, idx + 1, 4 * O.s16.psa, O.s16.levels, v[c][1], O.exp_a[i]);
-            } else if (two) {
+            if (two) {
               split_store2(O.s16.a, idx, 4 * O.s16.psa, O.s16.levels, v[c][0], v[c][1]);
             } else {
               split_store(O.s16.a, idx, 4 * O.s16.psa, O.s16.levels, v[c][0]);
@@ -357,10 +399,7 @@ __global__ void __launch_bounds__(256) k_combine_f2(CombineArgs a) {
           for (int c = 0; c < 4; c++) {
             const long idx = c * O.s16.psb + (long)jj * O.s16.ldb + ii;
             const float x = stage[c][jl][2 * p], y = stage[c][jl][2 * p + 1];
-            if (O.exp_b) {
-              slice_store<float>(O.s16.b, idx, 4 * O.s16.psb, O.s16.levels, x, O.exp_b[jj]);
-              if (pair) slice_store<float>(O.s16.b, idx + 1, 4 * O.s16.psb, O.s16.levels, y, O.exp_b[jj]);
-            } else if (pair) {
+            if (pair) {
               split_store2(O.s16.b, idx, 4 * O.s16.psb, O.s16.levels, x, y);
             } else {
               split_store(O.s16.b, idx, 4 * O.s16.psb, O.s16.levels, x);
@@ -390,7 +429,7 @@ static bool combine_pairs_ok(const CombineArgs& a) {
   if (a.f64) return false;
   auto even = [](long x) { return (x & 1) == 0; };
   auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  if (a.acc && (!even(a.ld_acc) || !even(a.ps_acc) || !al(a.acc) || (a.acc2 && !al(a.acc2)))) return false;
+  if (a.acc && (!even(a.ld_acc) || !even(a.ps_acc) || !al(a.acc))) return false;
   for (int t = 0; t < 4; t++)
     if (a.aux[t] && (!even(a.ld_aux[t]) || !even(a.ps_aux[t]) || !al(a.aux[t]))) return false;
   for (int o = 0; o < a.nout; o++) {
@@ -403,79 +442,144 @@ static bool combine_pairs_ok(const CombineArgs& a) {
 }
 
 // ---------------------------------------------------------------- exact slicing
-// S exact slices (slice_store's digits) of 8 consecutive entries that share
-// one exponent, written as one 16-byte store per slice plane.
+// The exact-slice GEMM computes a quaternion product as eight real products
+// of digit sums (qgemm_emu.cu).  A thread takes 8 consecutive entries along
+// the slice row: its four components become 64-bit integers F = round(v
+// 2^(7S - e)), biased so that every balanced 7-bit digit is a plain bit field
+// (F + 64 (1 + 2^7 + ... + 2^(7(S-2))): field - 64 in [-64, 63]; the top digit
+// is what is left above them), and each slice writes one 16-byte store per
+// product.  Digits become floats by inserting the field into the mantissa of
+// 2^23, so the sums and the conversion are FP32 adds and packed BF16
+// conversions (exact: the sums are integers of at most 8 bits).
+// Bound: HBM writes, 16 S bytes per entry (double the four-plane form's; the
+// product it feeds does half the tensor work).
 template <typename T>
-__device__ __forceinline__ void slice8_store(bf16* base, long lstride, int S, const T* v, int e) {
-  long long F[8];
+__device__ __forceinline__ void slice_bias(const T* v, int S, int e, long long* G) {
+  long long bias = 0;
+  for (int q = 0; q < S - 1; q++) bias = (bias << 7) + 64;
 #pragma unroll
-  for (int q = 0; q < 8; q++) F[q] = to_fixed(v[q], 7 * S - e);
-  for (int l = S - 1; l >= 0; l--) {
-    uint32_t pk[4];
+  for (int t = 0; t < 8; t++) G[t] = to_fixed(v[t], 7 * S - e) + bias;
+}
+__device__ __forceinline__ float digit_of(long long G, int sh, bool top) {
+  if (top) return (float)(int)(G >> sh);
+  return __uint_as_float(0x4B000000u | ((unsigned)(G >> sh) & 127u)) - 8388672.0f;
+}
+// LEFT: w+x, z-y, w-x, y+z, x+z, x-z, w+y, w-y; right: w+x, y-z, y+z, w-x, x+y, x-y, w-z, w+z.
+template <bool LEFT>
+__device__ __forceinline__ void digit_sums(float w, float x, float y, float z, float* c) {
+  if (LEFT) {
+    c[0] = w + x; c[1] = z - y; c[2] = w - x; c[3] = y + z;
+    c[4] = x + z; c[5] = x - z; c[6] = w + y; c[7] = w - y;
+  } else {
+    c[0] = w + x; c[1] = y - z; c[2] = y + z; c[3] = w - x;
+    c[4] = x + y; c[5] = x - y; c[6] = w - z; c[7] = w + z;
+  }
+}
+// dst: the entries' place in slice 0, product p0; planes ps apart, slices np ps apart.
+template <bool LEFT>
+__device__ __forceinline__ void slices_store(bf16* dst, long ps, int S, int p0, int np, const long long (*G)[8]) {
+  for (int l = 0; l < S; l++) {
+    const int sh = 7 * (S - 1 - l);
+    uint32_t pk[8][4];
 #pragma unroll
-    for (int q = 0; q < 8; q += 2) {
-      float x[2];
+    for (int t = 0; t < 8; t += 2) {
+      float a[8], b[8];
+      digit_sums<LEFT>(digit_of(G[0][t], sh, l == 0), digit_of(G[1][t], sh, l == 0), digit_of(G[2][t], sh, l == 0),
+                       digit_of(G[3][t], sh, l == 0), a);
+      digit_sums<LEFT>(digit_of(G[0][t + 1], sh, l == 0), digit_of(G[1][t + 1], sh, l == 0),
+                       digit_of(G[2][t + 1], sh, l == 0), digit_of(G[3][t + 1], sh, l == 0), b);
 #pragma unroll
-      for (int h = 0; h < 2; h++) {
-        if (l > 0) {
-          int d = (int)(F[q + h] & 127);
-          if (d >= 64) d -= 128;
-          F[q + h] = (F[q + h] - d) >> 7;
-          x[h] = ldexpf((float)d, -7 * (l + 1));
-        } else {
-          x[h] = ldexpf((float)F[q + h], -7);
-        }
+      for (int p = 0; p < 8; p++) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(a[p], b[p]);
+        pk[p][t >> 1] = *reinterpret_cast<const uint32_t*>(&h);
       }
-      pk[q >> 1] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x[0])) |
-                   ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x[1])) << 16);
     }
-    *reinterpret_cast<uint4*>(base + l * lstride) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-  }
-}
-
-// A-form slices of a row-major plane set (row exponents e[i]): one thread per
-// (plane, row, 8 columns), columns past `cols` up to the padded pitch as 0.
-template <typename T>
-__global__ void __launch_bounds__(256) k_slice_rows(Planes<const T> A, int rows, int cols, const int* __restrict__ e,
-                                                    int S, bf16* dst, long ld, long ps) {
-  const int g8 = (cols + 7) / 8;
-  const long total = 4L * rows * g8;
-  for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-    const int g = (int)(t % g8);
-    const long ci = t / g8;
-    const int i = (int)(ci % rows), c = (int)(ci / rows);
-    const T* src = A.p + c * A.ps + (long)i * A.ld + 8 * g;
-    T v[8];
+    bf16* dl = dst + (long)l * np * ps;
 #pragma unroll
-    for (int q = 0; q < 8; q++) v[q] = 8 * g + q < cols ? src[q] : (T)0;
-    slice8_store<T>(dst + c * ps + (long)i * ld + 8 * g, 4 * ps, S, v, e[i]);
+    for (int p = 0; p < 8; p++)
+      if (p >= p0 && p < p0 + np)
+        *reinterpret_cast<uint4*>(dl + (p - p0) * ps) = make_uint4(pk[p][0], pk[p][1], pk[p][2], pk[p][3]);
   }
 }
 
-// B-form slices (the plane-wise transpose; column exponents e[j]): a block
-// takes 32 rows x 64 columns of one plane through shared memory, then each
-// thread writes 8 consecutive rows of one column, rows past `rows` up to the
-// padded pitch as 0.
+// A-form: WPR warps per row find the row's exponent (one read of the row),
+// then slice it (the second read hits L1 / L2: a row is at most a few
+// hundred KB), so no separate exponent pass is needed.
+template <typename T, int WPR>
+__global__ void __launch_bounds__(256) k_slice_rows(Planes<const T> A, int rows, int cols, int* __restrict__ e_out,
+                                                    int S, int p0, int np, bf16* dst, long ld, long ps) {
+  __shared__ int sh[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = blockIdx.x * (8 / WPR) + warp / WPR, tr = (warp % WPR) * 32 + lane;
+  const bool ok = i < rows;
+  const T* row = A.p + (long)(ok ? i : 0) * A.ld;
+  int mx = -100000;
+  if (ok) {
+#pragma unroll 4
+    for (int j = tr; j < cols; j += 32 * WPR)
+#pragma unroll
+      for (int c = 0; c < 4; c++) mx = max(mx, exp_of(row[c * A.ps + j]));
+  }
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (WPR > 1) {
+    if (lane == 0) sh[warp] = mx;
+    __syncthreads();
+    const int w0 = warp / WPR * WPR;
+#pragma unroll
+    for (int q = 0; q < WPR; q++) mx = max(mx, sh[w0 + q]);
+  }
+  if (!ok) return;
+  const int e = mx == -100000 ? 0 : mx;
+  if (tr == 0) e_out[i] = e;
+  const int g8 = (cols + 7) / 8;
+  for (int g = tr; g < g8; g += 32 * WPR) {
+    long long G[4][8];
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const T* src = row + c * A.ps + 8 * g;
+      T v[8];
+#pragma unroll
+      for (int q = 0; q < 8; q++) v[q] = 8 * g + q < cols ? src[q] : (T)0;
+      slice_bias<T>(v, S, e, G[c]);
+    }
+    slices_store<true>(dst + (long)i * ld + 8 * g, ps, S, p0, np, G);
+  }
+}
+
+// B-form (the plane-wise transpose; column exponents e[j]): a block takes 64
+// rows x 32 columns of the four planes through shared memory, then each
+// thread slices 8 consecutive rows of one column (a warp's stores cover 128
+// bytes of each of 4 slice rows).  Rows past `rows` up to the padded pitch are 0.
+constexpr int SC_ROWS = 64, SC_COLS = 32;
 template <typename T>
 __global__ void __launch_bounds__(256) k_slice_cols(Planes<const T> A, int rows, int cols, const int* __restrict__ e,
-                                                    int S, bf16* dst, long ld, long ps) {
-  __shared__ T tile[64][33];
-  const int c = blockIdx.z, i0 = blockIdx.y * 32, j0 = blockIdx.x * 64;
+                                                    int S, int p0, int np, bf16* dst, long ld, long ps) {
+  extern __shared__ __align__(16) unsigned char sc_smem[];
+  T(*tile)[SC_COLS][SC_ROWS + 1] = reinterpret_cast<T(*)[SC_COLS][SC_ROWS + 1]>(sc_smem);
+  const int i0 = blockIdx.y * SC_ROWS, j0 = blockIdx.x * SC_COLS;
   {
-    const int il = threadIdx.x >> 3, j8 = (threadIdx.x & 7) * 8;  // 32 rows x 8 groups of 8 columns
-    const T* src = A.p + c * A.ps + (long)(i0 + il) * A.ld + j0 + j8;
+    const int jl = threadIdx.x & 31;
+#pragma unroll 2
+    for (int il = threadIdx.x >> 5; il < SC_ROWS; il += 8) {
+      const bool in = i0 + il < rows && j0 + jl < cols;
 #pragma unroll
-    for (int q = 0; q < 8; q++)
-      tile[j8 + q][il] = (i0 + il < rows && j0 + j8 + q < cols) ? src[q] : (T)0;
+      for (int c = 0; c < 4; c++) tile[c][jl][il] = in ? A.p[c * A.ps + (long)(i0 + il) * A.ld + j0 + jl] : (T)0;
+    }
   }
   __syncthreads();
-  const int jl = threadIdx.x >> 2, ig = (threadIdx.x & 3) * 8;  // 64 columns x 4 groups of 8 rows
+  const int jl = threadIdx.x >> 3, ig = (threadIdx.x & 7) * 8;
   const int j = j0 + jl;
   if (j < cols && i0 + ig < ((rows + 7) / 8) * 8) {
-    T v[8];
+    const int ej = e[j];
+    long long G[4][8];
 #pragma unroll
-    for (int q = 0; q < 8; q++) v[q] = tile[jl][ig + q];
-    slice8_store<T>(dst + c * ps + (long)j * ld + i0 + ig, 4 * ps, S, v, e[j]);
+    for (int c = 0; c < 4; c++) {
+      T v[8];
+#pragma unroll
+      for (int q = 0; q < 8; q++) v[q] = tile[c][jl][ig + q];
+      slice_bias<T>(v, S, ej, G[c]);
+    }
+    slices_store<false>(dst + (long)j * ld + i0 + ig, ps, S, p0, np, G);
   }
 }
 
@@ -655,19 +759,8 @@ __global__ void __launch_bounds__(256) k_init_x0(Planes<const double> A, int m, 
   }
 }
 
-// Exponent e with |v| < 2^e for every v of a row (A-operand scaling) or a
-// column (B-operand scaling), over all four planes; integer ops on the bits.
-template <typename T>
-__global__ void k_row_maxexp(Planes<const T> A, int rows, int cols, int* e) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= rows) return;
-  int mx = -100000;
-  for (int j = lane; j < cols; j += 32)
-    for (int c = 0; c < 4; c++) mx = max(mx, exp_of(A.p[c * A.ps + (long)warp * A.ld + j]));
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0) e[warp] = mx == -100000 ? 0 : mx;
-}
-
+// Exponent e with |v| < 2^e for every v of a column, over all four planes;
+// integer ops on the bits.
 template <typename T>
 __global__ void k_col_maxexp_part(Planes<const T> A, int rows, int cols, int chunk_rows, int* part) {
   __shared__ int sh[CR_ROWS][CR_COLS];
@@ -806,34 +899,20 @@ cudaError_t launch_init_x0(const Planes<const double>& A, int m, int n, double a
   return cudaGetLastError();
 }
 
-cudaError_t launch_maxexp(const Planes<const double>& A, int rows, int cols, int by_col, int* e, int* scratch,
-                          cudaStream_t st) {
-  if (by_col) {
-    const int ch = col_chunks(rows, cols), chunk_rows = (rows + ch - 1) / ch;
-    k_col_maxexp_part<double><<<dim3((cols + CR_COLS - 1) / CR_COLS, ch), dim3(CR_COLS, CR_ROWS), 0, st>>>(
-        A, rows, cols, chunk_rows, scratch);
-    k_col_maxexp_finish<<<(cols + 255) / 256, 256, 0, st>>>(scratch, ch, cols, e);
-    g_kernel_launches += 2;
-  } else {
-    k_row_maxexp<double><<<(rows + 7) / 8, 256, 0, st>>>(A, rows, cols, e);
-    ++g_kernel_launches;
-  }
+template <typename T>
+static cudaError_t maxexp_t(const Planes<const T>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st) {
+  const int ch = col_chunks(rows, cols), chunk_rows = (rows + ch - 1) / ch;
+  k_col_maxexp_part<T><<<dim3((cols + CR_COLS - 1) / CR_COLS, ch), dim3(CR_COLS, CR_ROWS), 0, st>>>(
+      A, rows, cols, chunk_rows, scratch);
+  k_col_maxexp_finish<<<(cols + 255) / 256, 256, 0, st>>>(scratch, ch, cols, e);
+  g_kernel_launches += 2;
   return cudaGetLastError();
 }
-
-cudaError_t launch_maxexp_f32(const Planes<const float>& A, int rows, int cols, int by_col, int* e, int* scratch,
-                              cudaStream_t st) {
-  if (by_col) {
-    const int ch = col_chunks(rows, cols), chunk_rows = (rows + ch - 1) / ch;
-    k_col_maxexp_part<float><<<dim3((cols + CR_COLS - 1) / CR_COLS, ch), dim3(CR_COLS, CR_ROWS), 0, st>>>(
-        A, rows, cols, chunk_rows, scratch);
-    k_col_maxexp_finish<<<(cols + 255) / 256, 256, 0, st>>>(scratch, ch, cols, e);
-    g_kernel_launches += 2;
-  } else {
-    k_row_maxexp<float><<<(rows + 7) / 8, 256, 0, st>>>(A, rows, cols, e);
-    ++g_kernel_launches;
-  }
-  return cudaGetLastError();
+cudaError_t launch_maxexp(const Planes<const double>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st) {
+  return maxexp_t<double>(A, rows, cols, e, scratch, st);
+}
+cudaError_t launch_maxexp(const Planes<const float>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st) {
+  return maxexp_t<float>(A, rows, cols, e, scratch, st);
 }
 
 cudaError_t launch_f32_to_f64(const Planes<const float>& src, int rows, int cols, const Planes<double>& dst,
@@ -852,43 +931,48 @@ cudaError_t launch_f64_to_f32(const Planes<const double>& src, int rows, int col
 
 
 template <typename T>
-static cudaError_t slice_rows_t(const Planes<const T>& A, int rows, int cols, const int* e, int S, bf16* dst,
+static cudaError_t slice_rows_t(const Planes<const T>& A, int rows, int cols, int* e, int S, int p0, int np, bf16* dst,
                                 long ld, long ps, cudaStream_t st) {
   if (rows <= 0 || cols <= 0) return cudaSuccess;
   if ((ld & 7) || (ps & 7) || (reinterpret_cast<uintptr_t>(dst) & 15) || ld < ((cols + 7) / 8) * 8)
     return cudaErrorInvalidValue;
-  const long total = 4L * rows * ((cols + 7) / 8);
-  const int blocks = (int)std::min<long>((total + 255) / 256, 152L * 16);
-  k_slice_rows<T><<<blocks, 256, 0, st>>>(A, rows, cols, e, S, dst, ld, ps);
+  // four warps per row once a row is more than two iterations of one warp
+  if (cols > 512)
+    k_slice_rows<T, 4><<<(rows + 1) / 2, 256, 0, st>>>(A, rows, cols, e, S, p0, np, dst, ld, ps);
+  else
+    k_slice_rows<T, 1><<<(rows + 7) / 8, 256, 0, st>>>(A, rows, cols, e, S, p0, np, dst, ld, ps);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
 template <typename T>
-static cudaError_t slice_cols_t(const Planes<const T>& A, int rows, int cols, const int* e, int S, bf16* dst,
-                                long ld, long ps, cudaStream_t st) {
+static cudaError_t slice_cols_t(const Planes<const T>& A, int rows, int cols, const int* e, int S, int p0, int np,
+                                bf16* dst, long ld, long ps, cudaStream_t st) {
   if (rows <= 0 || cols <= 0) return cudaSuccess;
   if ((ld & 7) || (ps & 7) || (reinterpret_cast<uintptr_t>(dst) & 15) || ld < ((rows + 7) / 8) * 8)
     return cudaErrorInvalidValue;
-  dim3 grid((cols + 63) / 64, (rows + 31) / 32, 4);
-  k_slice_cols<T><<<grid, 256, 0, st>>>(A, rows, cols, e, S, dst, ld, ps);
+  constexpr int smem = (int)sizeof(T) * 4 * SC_COLS * (SC_ROWS + 1);
+  static std::atomic<unsigned long long> attr_done{0};
+  if (cudaError_t err = ensure_smem_attr(k_slice_cols<T>, smem, attr_done)) return err;
+  dim3 grid((cols + SC_COLS - 1) / SC_COLS, (rows + SC_ROWS - 1) / SC_ROWS);
+  k_slice_cols<T><<<grid, 256, smem, st>>>(A, rows, cols, e, S, p0, np, dst, ld, ps);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
-cudaError_t launch_slice_rows(const Planes<const double>& A, int rows, int cols, const int* e, int S, bf16* dst,
-                              long ld, long ps, cudaStream_t st) {
-  return slice_rows_t<double>(A, rows, cols, e, S, dst, ld, ps, st);
+cudaError_t launch_slice_rows(const Planes<const double>& A, int rows, int cols, int* e, int S, int p0, int np,
+                              bf16* dst, long ld, long ps, cudaStream_t st) {
+  return slice_rows_t<double>(A, rows, cols, e, S, p0, np, dst, ld, ps, st);
 }
-cudaError_t launch_slice_rows(const Planes<const float>& A, int rows, int cols, const int* e, int S, bf16* dst,
-                              long ld, long ps, cudaStream_t st) {
-  return slice_rows_t<float>(A, rows, cols, e, S, dst, ld, ps, st);
+cudaError_t launch_slice_rows(const Planes<const float>& A, int rows, int cols, int* e, int S, int p0, int np,
+                              bf16* dst, long ld, long ps, cudaStream_t st) {
+  return slice_rows_t<float>(A, rows, cols, e, S, p0, np, dst, ld, ps, st);
 }
-cudaError_t launch_slice_cols(const Planes<const double>& A, int rows, int cols, const int* e, int S, bf16* dst,
-                              long ld, long ps, cudaStream_t st) {
-  return slice_cols_t<double>(A, rows, cols, e, S, dst, ld, ps, st);
+cudaError_t launch_slice_cols(const Planes<const double>& A, int rows, int cols, const int* e, int S, int p0, int np,
+                              bf16* dst, long ld, long ps, cudaStream_t st) {
+  return slice_cols_t<double>(A, rows, cols, e, S, p0, np, dst, ld, ps, st);
 }
-cudaError_t launch_slice_cols(const Planes<const float>& A, int rows, int cols, const int* e, int S, bf16* dst,
-                              long ld, long ps, cudaStream_t st) {
-  return slice_cols_t<float>(A, rows, cols, e, S, dst, ld, ps, st);
+cudaError_t launch_slice_cols(const Planes<const float>& A, int rows, int cols, const int* e, int S, int p0, int np,
+                              bf16* dst, long ld, long ps, cudaStream_t st) {
+  return slice_cols_t<float>(A, rows, cols, e, S, p0, np, dst, ld, ps, st);
 }
 
 }  // namespace qp

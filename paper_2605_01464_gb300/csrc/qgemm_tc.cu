@@ -9,8 +9,7 @@
 //   r=2 -B2   +B3    +B0    -B1
 //   r=3 -B3   -B2    +B1    +B0
 // M(B) is never formed: per K step the kernel stages the four A planes and
-// the four B planes of a tile in shared memory (TMA; 64-byte swizzle for the
-// two-CTA-per-SM shape, 128-byte for the two-accumulator shape) and
+// the four B planes of a tile in shared memory (TMA, 64-byte swizzle) and
 // issues the 16 (r, c) products as separate tcgen05.mma instructions, each
 // reading plane r xor c of B and taking its sign from the instruction
 // descriptor's negate-A bit.  The four output components accumulate in FP32
@@ -42,9 +41,7 @@ constexpr int GROUP_M = 16;       // CTA rasterization: 16 row tiles per group s
 
 // Stage shape.  BK BF16 K-elements per stage = one swizzle row of 2*BK bytes.
 //   Wide: BK = 32 (64-byte swizzle), 48 KB per stage, two CTAs per SM, so one
-//         CTA's epilogue overlaps the other's main loop (one accumulator).
-//   Deep: BK = 64 (128-byte swizzle), 96 KB per stage, one CTA per SM (two
-//         accumulators take all 512 TMEM columns).
+//         CTA's epilogue overlaps the other's main loop.
 //   Broad: BK = 32, 128 columns per CTA (a 512-column accumulator), three
 //         64 KB stages, one CTA per SM: twice the MMA work per operand tile
 //         read of the wide shape.
@@ -65,10 +62,8 @@ struct Cfg {
                                     ((uint32_t)(BM >> 4) << 24);
 };
 using CfgWide = Cfg<32, 64, 2>;
-using CfgDeep = Cfg<64, 128, 1>;
 using CfgBroad = Cfg<32, 64, 1, 128, 3>;
 static_assert(CfgWide::SMEM * 2 <= 227 * 1024, "two wide CTAs per SM");
-static_assert(CfgDeep::SMEM * 2 > 228 * 1024, "one deep CTA per SM");
 static_assert(CfgBroad::SMEM <= 227 * 1024 && CfgBroad::ACC == 512, "one broad CTA per SM, all TMEM columns");
 constexpr int THREADS = 192;
 
@@ -81,14 +76,8 @@ struct KParams {
   int kb0, kb1;  // K blocks [kb0, kb1) of BK elements
   int npairs;
   int pi[16], pj[16];
-  int pacc[16];   // accumulator (0 or 1) of each pair
-  int pfirst[16]; // 1 if the pair is the first of its accumulator
-  int nacc;       // 1 or 2 accumulators (2 only with int64 output)
   Planes<float> C;
   EpiArgs E;       // E.nout > 0: fused combine epilogue (FP32 output only)
-  long long* C64;  // non-null: int64 fixed-point accumulation
-  long ld64, ps64;
-  float scale;     // 2^shift
   int* err;
 };
 
@@ -258,7 +247,7 @@ __global__ void __launch_bounds__(THREADS, C::MINB)
   const int gm = min(GROUP_M, P.Mt - group * GROUP_M);
   const int m0 = (group * GROUP_M + local % gm) * BM, n0 = (local / gm) * BN;
   const int nunits = (P.kb1 - P.kb0) * P.npairs;
-  const uint32_t tmem_cols = P.nacc == 2 ? 2 * ACC_COLS : ACC_COLS;
+  constexpr uint32_t tmem_cols = ACC_COLS;
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -312,12 +301,10 @@ __global__ void __launch_bounds__(THREADS, C::MINB)
         uint8_t* st = smem + (size_t)s * STAGE_BYTES;
         const uint64_t ad0 = smem_desc_sw<C::SWB>(smem_u32(st)),
                        bd0 = smem_desc_sw<C::SWB>(smem_u32(st + 4 * A_PLANE_BYTES));
-        const int pr = u % P.npairs;
-        const uint32_t dacc = tmem + (uint32_t)(P.pacc[pr] * ACC_COLS);
-        const bool fresh = u < P.npairs && P.pfirst[pr];  // first K block of this accumulator
+        const bool fresh = u == 0;
 #pragma unroll
         for (int kk = 0; kk < BK / 16; kk++)
-          qmma_k16<A_PLANE_BYTES, B_PLANE_BYTES>(dacc, BN, ad0 + kk * 2, bd0 + kk * 2, C::IDESC, fresh && kk == 0);
+          qmma_k16<A_PLANE_BYTES, B_PLANE_BYTES>(tmem, BN, ad0 + kk * 2, bd0 + kk * 2, C::IDESC, fresh && kk == 0);
         mma_commit(smem_u32(&bar_empty[s]));
         if (u == nunits - 1) mma_commit(smem_u32(&bar_acc));
       }
@@ -376,44 +363,26 @@ __global__ void __launch_bounds__(THREADS, C::MINB)
         }
       }
     } else if (have) {
-      long long* st64 = reinterpret_cast<long long*>(smem) + (warp - 2) * (32 * 33);
-      float* st32 = reinterpret_cast<float*>(st64);
+      float* st32 = reinterpret_cast<float*>(smem) + (warp - 2) * (32 * 33);
 #pragma unroll 1
       for (int c = 0; c < 4; c++) {
 #pragma unroll 1
         for (int ch = 0; ch < BN / 32; ch++) {
-          float v[32], v2[32];
+          float v[32];
           if (nunits > 0) {
             tmem_ld32(tbase + c * BN + ch * 32, v);
-            if (P.nacc == 2) tmem_ld32(tbase + ACC_COLS + c * BN + ch * 32, v2);
           } else {
 #pragma unroll
-            for (int t = 0; t < 32; t++) v[t] = v2[t] = 0.f;
+            for (int t = 0; t < 32; t++) v[t] = 0.f;
           }
           const int col = n0 + ch * 32 + lane;
           const int nrow = min(32, P.M - row0);
-          if (P.C64) {
-            if (P.nacc == 2) {
 #pragma unroll
-              for (int t = 0; t < 32; t++)
-                st64[lane * 33 + t] = __float2ll_rn(v[t] * P.scale) + __float2ll_rn(v2[t] * P.scale);
-            } else {
-#pragma unroll
-              for (int t = 0; t < 32; t++) st64[lane * 33 + t] = __float2ll_rn(v[t] * P.scale);
-            }
-            __syncwarp();
-            if (col < P.N) {
-              long long* dst = P.C64 + c * P.ps64 + (long)row0 * P.ld64 + col;
-              rmw_rows64(dst, P.ld64, nrow, st64 + lane);
-            }
-          } else {
-#pragma unroll
-            for (int t = 0; t < 32; t++) st32[lane * 33 + t] = v[t];
-            __syncwarp();
-            if (col < P.N) {
-              float* dst = P.C.p + c * P.C.ps + (long)row0 * P.C.ld + col;
-              store_rows32(dst, P.C.ld, nrow, st32 + lane);
-            }
+          for (int t = 0; t < 32; t++) st32[lane * 33 + t] = v[t];
+          __syncwarp();
+          if (col < P.N) {
+            float* dst = P.C.p + c * P.C.ps + (long)row0 * P.C.ld + col;
+            store_rows32(dst, P.C.ld, nrow, st32 + lane);
           }
           __syncwarp();
         }
@@ -563,7 +532,7 @@ __global__ void __launch_bounds__(CP_THREADS, 1)
           fence_after();
           uint8_t* st = smem + (size_t)s * CP_STAGE;
           const uint64_t ad0 = smem_desc_sw<64>(smem_u32(st)), bd0 = smem_desc_sw<64>(smem_u32(st + 4 * CP_A_PLANE));
-          const bool fresh = x < P.npairs && P.pfirst[x % P.npairs];  // first K block of the accumulator
+          const bool fresh = x == 0;
 #pragma unroll
           for (int kk = 0; kk < CP_BK / 16; kk++) {
             qmma_k16_one(dacc, c0, ad0 + kk * 2, bd0 + kk * 2, fresh && kk == 0);
@@ -732,40 +701,21 @@ cudaError_t launch_qgemm_tc(const TcGemmArgs& a, cudaStream_t st) {
   if (a.M <= 0 || a.N <= 0) return cudaSuccess;
   if (a.npairs < 1 || a.npairs > 16 || !a.A || !a.B || !a.A->a || !a.B->b) return cudaErrorInvalidValue;
   if ((a.A->lda % 8) || (a.A->psa % 8) || (a.B->ldb % 8) || (a.B->psb % 8)) return cudaErrorInvalidValue;
-  int nacc = 1;
-  for (int p = 0; p < a.npairs; p++) {
-    if (a.pair_i[p] < 0 || a.pair_i[p] >= a.A->levels || a.pair_j[p] < 0 || a.pair_j[p] >= a.B->levels ||
-        a.pair_acc[p] < 0 || a.pair_acc[p] > 1)
+  for (int p = 0; p < a.npairs; p++)
+    if (a.pair_i[p] < 0 || a.pair_i[p] >= a.A->levels || a.pair_j[p] < 0 || a.pair_j[p] >= a.B->levels)
       return cudaErrorInvalidValue;
-    if (a.pair_acc[p] == 1) nacc = 2;
-  }
-  if (nacc == 2 && !a.C64) return cudaErrorInvalidValue;  // two accumulators only sum into int64
   KParams P;
   P.M = a.M;
   P.N = a.N;
   P.npairs = a.npairs;
-  bool seen[2] = {false, false};
   for (int p = 0; p < 16; p++) {
     P.pi[p] = p < a.npairs ? a.pair_i[p] : 0;
     P.pj[p] = p < a.npairs ? a.pair_j[p] : 0;
-    P.pacc[p] = p < a.npairs ? a.pair_acc[p] : 0;
-    P.pfirst[p] = 0;
-    if (p < a.npairs && !seen[P.pacc[p]]) {
-      P.pfirst[p] = 1;
-      seen[P.pacc[p]] = true;
-    }
   }
-  P.nacc = nacc;
   P.C = a.C;
   P.E = a.epi;
-  if (P.E.nout < 0 || P.E.nout > kMaxOut || (P.E.nout > 0 && (a.C64 || nacc == 2)) || (P.E.f64 && P.E.partials))
-    return cudaErrorInvalidValue;
-  P.C64 = a.C64;
-  P.ld64 = a.ld64;
-  P.ps64 = a.ps64;
-  P.scale = ldexpf(1.0f, a.shift);
+  if (P.E.nout < 0 || P.E.nout > kMaxOut || (P.E.f64 && P.E.partials)) return cudaErrorInvalidValue;
   P.err = a.err;
-  if (nacc == 2) return launch_cfg<CfgDeep>(a, P, st);
   switch (tc_shape(a.broad, P.E.nout > 0, a.M, a.N)) {
     case SHAPE_PAIRS: return launch_pairs(a, P, st);
     case SHAPE_BROAD: return launch_cfg<CfgBroad>(a, P, st);

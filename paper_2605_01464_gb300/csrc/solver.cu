@@ -313,7 +313,7 @@ struct Solver {
     const int* erow;
     const int* ecol;
     int shift;
-    const long long* p2 = nullptr;  // ACC_I64: second accumulator of the same layout, summed
+    int sets = 1;  // ACC_Q8: plane sets, summed
   };
 
   // acc(rows x cols) = P (rows x K) * Q (K x cols) in one of three modes:
@@ -380,7 +380,7 @@ struct Solver {
     a.acc_erow = acc.erow;
     a.acc_ecol = acc.ecol;
     a.acc_shift = acc.shift;
-    a.acc2 = acc.p2;
+    a.acc_sets = acc.sets;
   }
 
   // Whether the combine pass `a` (no accumulator set yet) can run in the
@@ -392,7 +392,6 @@ struct Solver {
     if (a.f64 != (dbl ? 1 : 0) || (dbl && with_partials)) return false;
     for (int o = 0; o < a.nout; o++) {
       const OutSpec& O = a.out[o];
-      if (O.exp_a || O.exp_b) return false;
       if ((O.s16.a || O.s16.b) && O.s16.levels < 1) return false;
       const void* forms[4] = {P.s16.a, P.s16.b, Q.s16.a, Q.s16.b};
       for (const void* f : forms)
@@ -458,142 +457,75 @@ struct Solver {
     run(a, with_partials, red_slot);
   }
 
+  // Exact-slice product (qgemm_emu.cu): slices of the eight digit
+  // combinations of both operands, one GEMM launch, eight int64 product
+  // planes that the combine pass sums.
   Acc prod_emu(const QMat& P, const QMat& Q, int S, double flops) {
     const int M = P.rows, K = P.cols, N = Q.cols;
     // A as an operand: its exponents and slices come from (or go to) the cache
     const bool pA = &P == &A, qA = &Q == &A;
-    const bool pA_hit = pA && acache_form == 0 && acache_S == S && acache_dbl == dbl;
-    const bool qA_hit = qA && acache_form == 1 && acache_S == S && acache_dbl == dbl;
     int* eP = (int*)buf(c, pA ? "emu.cacheA.e" : "emu.eP", sizeof(int) * (size_t)M + 64);
     int* eQ = (int*)buf(c, qA ? "emu.cacheA.e" : "emu.eQ", sizeof(int) * (size_t)N + 64);
     int* eS = (int*)buf(c, "emu.eS", sizeof(int) * (size_t)COL_SCRATCH(N) + 64);
-    if (dbl) {
-      if (!pA_hit)
-        timed(c, EV_EW, 0, 0, 32.0 * M * K, [&] { return launch_maxexp(dview(P), M, K, 0, eP, nullptr, c->st); });
-      if (!qA_hit)
-        timed(c, EV_EW, 0, 0, 32.0 * K * N, [&] { return launch_maxexp(dview(Q), K, N, 1, eQ, eS, c->st); });
-    } else {
-      if (!pA_hit)
-        timed(c, EV_EW, 0, 0, 16.0 * M * K,
-              [&] { return launch_maxexp_f32(fview(P), M, K, 0, eP, nullptr, c->st); });
-      if (!qA_hit)
-        timed(c, EV_EW, 0, 0, 16.0 * K * N, [&] { return launch_maxexp_f32(fview(Q), K, N, 1, eQ, eS, c->st); });
-    }
+    const char* zname[2] = {pA ? "emu.cacheA.z" : "emu.za", qA ? "emu.cacheA.z" : "emu.zb"};
+    EmuGemmArgs g;
+    g.M = M;
+    g.N = N;
+    g.K = K;
+    g.S = S;
+    g.err = c->d_err;
+    const EmuPlan plan = emu_plan(M, N, K, S);
+    g.ld64 = (N + 3) / 4 * 4;
+    g.ps64 = (long)M * g.ld64;
+    g.C64 = (long long*)buf(c, "emu.acc", sizeof(long long) * 8 * (size_t)plan.nparts * g.ps64 + 64);
     Split16 za, zb;
     za.levels = zb.levels = S;
-    za.lda = rup64(K);
+    za.lda = zb.ldb = rup64(K);
     za.psa = (long)M * za.lda;
-    za.a = (bf16*)buf(c, pA ? "emu.cacheA.z" : "emu.za", sizeof(bf16) * 4 * S * (size_t)za.psa + 64);
-    zb.ldb = rup64(K);
     zb.psb = (long)N * zb.ldb;
-    zb.b = (bf16*)buf(c, qA ? "emu.cacheA.z" : "emu.zb", sizeof(bf16) * 4 * S * (size_t)zb.psb + 64);
-    // the slices: P's rows (A-form), Q's columns (B-form, transposed)
-    const double sbytes = 2.0 * S * 4;
-    if (dbl) {
-      if (!pA_hit)
-        timed(c, EV_EW, 0, 0, (32.0 + sbytes) * M * K,
-              [&] { return launch_slice_rows(dview(P), M, K, eP, S, za.a, za.lda, za.psa, c->st); });
-      if (!qA_hit)
-        timed(c, EV_EW, 0, 0, (32.0 + sbytes) * K * N,
-              [&] { return launch_slice_cols(dview(Q), K, N, eQ, S, zb.b, zb.ldb, zb.psb, c->st); });
-    } else {
-      if (!pA_hit)
-        timed(c, EV_EW, 0, 0, (16.0 + sbytes) * M * K,
-              [&] { return launch_slice_rows(fview(P), M, K, eP, S, za.a, za.lda, za.psa, c->st); });
-      if (!qA_hit)
-        timed(c, EV_EW, 0, 0, (16.0 + sbytes) * K * N,
-              [&] { return launch_slice_cols(fview(Q), K, N, eQ, S, zb.b, zb.ldb, zb.psb, c->st); });
+    // all eight combinations at once; four at a time when they do not fit
+    int np = 8;
+    try {
+      za.a = (bf16*)buf(c, zname[0], sizeof(bf16) * 8 * S * (size_t)za.psa + 64);
+      zb.b = (bf16*)buf(c, zname[1], sizeof(bf16) * 8 * S * (size_t)zb.psb + 64);
+    } catch (const QpError&) {
+      np = 4;
+      acache_form = -1;
+      za.a = (bf16*)buf(c, zname[0], sizeof(bf16) * 4 * S * (size_t)za.psa + 64);
+      zb.b = (bf16*)buf(c, zname[1], sizeof(bf16) * 4 * S * (size_t)zb.psb + 64);
+    }
+    const bool hit = np == 8 && (pA || qA) && acache_form == (pA ? 0 : 1) && acache_S == S && acache_dbl == dbl;
+    const bool skipP = pA && hit, skipQ = qA && hit;
+    g.A = &za;
+    g.B = &zb;
+    g.np = np;
+    const double ms = dbl ? 32.0 : 16.0, sbytes = 2.0 * S * np;
+    if (!skipQ)
+      timed(c, EV_EW, 0, 0, ms * K * N, [&] {
+        return dbl ? launch_maxexp(dview(Q), K, N, eQ, eS, c->st) : launch_maxexp(fview(Q), K, N, eQ, eS, c->st);
+      });
+    for (int p0 = 0; p0 < 8; p0 += np) {
+      g.p0 = p0;
+      if (!skipP)
+        timed(c, EV_EW, 0, 0, (ms + sbytes) * M * K, [&] {
+          return dbl ? launch_slice_rows(dview(P), M, K, eP, S, p0, np, za.a, za.lda, za.psa, c->st)
+                     : launch_slice_rows(fview(P), M, K, eP, S, p0, np, za.a, za.lda, za.psa, c->st);
+        });
+      if (!skipQ)
+        timed(c, EV_EW, 0, 0, (ms + sbytes) * K * N, [&] {
+          return dbl ? launch_slice_cols(dview(Q), K, N, eQ, S, p0, np, zb.b, zb.ldb, zb.psb, c->st)
+                     : launch_slice_cols(fview(Q), K, N, eQ, S, p0, np, zb.b, zb.ldb, zb.psb, c->st);
+        });
+      // 8 real products of 2 M K N flops per slice pair: half of the 16-product form
+      timed(c, EV_EMU, flops * np / 8, flops * np / 8 * S * (S + 1) / 4, 0,
+            [&] { return launch_qgemm_emu(g, plan, c->st); });
     }
     if (pA || qA) {
-      acache_form = pA ? 0 : 1;
+      acache_form = np == 8 ? (pA ? 0 : 1) : -1;
       acache_S = S;
       acache_dbl = dbl;
     }
-    long long* acc = (long long*)buf(c, "emu.acc", sizeof(long long) * 4 * (size_t)M * N + 64);
-    int lg = 0;
-    while ((1L << lg) < 4L * K) lg++;
-    const int shift = 61 - lg;  // |sum| < 4K in normalized units: no int64 overflow
-    // Levels d = s + t are launched two at a time (two TMEM accumulators
-    // summed by the epilogue), lowest first.  Levels whose FP32 rounding
-    // could matter are summed in K chunks small enough for every partial sum
-    // to be exact: balanced digits are at most 2^7 (slice 0) and 2^6, so one
-    // level-d product term is at most 2^14 (d = 0) or 2^12 (d + 3) over the
-    // pairs (2^13 for (0, d) and (d, 0), 2^12 for the rest); with 4 Kc terms
-    // per output this stays <= 2^24 for Kc <= 256 (d = 0) and 2^10 / (d + 3).
-    // The two lowest levels are summed over the whole K.
-    auto chunk = [&](int d) {
-      if (d > S - 3) return K;
-      const int lim = d == 0 ? 256 : 1024 / (d + 3);
-      return lim >= 64 ? (lim / 64) * 64 : 64;
-    };
-    if (emu_fused_ok(K, S)) {
-      // all levels and chunks in one launch, int32 level sums in TMEM
-      EmuGemmArgs g;
-      g.M = M;
-      g.N = N;
-      g.K = K;
-      g.A = &za;
-      g.B = &zb;
-      g.S = S;
-      for (int d = 0; d < S; d++) {
-        if (d > S - 3) {
-          g.kc[d] = K;
-        } else {
-          const int lim = d == 0 ? 256 : 1024 / (d + 3);
-          g.kc[d] = (lim / 32) * 32;
-        }
-      }
-      // half of the levels go to a second accumulator (see qgemm_emu.cu)
-      // (each group's first level stores: neither accumulator needs clearing)
-      long long* acc2 = (long long*)buf(c, "emu.acc2", sizeof(long long) * 4 * (size_t)M * N + 64);
-      g.C64 = acc;
-      g.C64b = S >= 2 ? acc2 : nullptr;
-      g.ld64 = N;
-      g.ps64 = (long)M * N;
-      g.shift = shift;
-      g.err = c->d_err;
-      const bool pair = M > 128 && c->opt.emu_pair == 1;
-      timed(c, EV_EMU, flops, flops * S * (S + 1) / 2, 0,
-            [&] { return pair ? launch_qgemm_emu_pair(g, c->st) : launch_qgemm_emu(g, c->st); });
-      Acc r{acc, ACC_I64, (long)N, (long)M * N, eP, eQ, shift};
-      r.p2 = g.C64b;
-      return r;
-    }
-    ck(c, cudaMemsetAsync(acc, 0, sizeof(long long) * 4 * (size_t)M * N, c->st), "memset");
-    for (int hi = S - 1; hi >= 0; hi -= 2) {
-      const int lo = hi - 1;  // second level of the launch (-1: none)
-      TcGemmArgs g;
-      g.M = M;
-      g.N = N;
-      g.K = K;
-      g.A = &za;
-      g.B = &zb;
-      g.npairs = 0;
-      for (int t = 0; t <= hi; t++, g.npairs++) {
-        g.pair_i[g.npairs] = t;
-        g.pair_j[g.npairs] = hi - t;
-        g.pair_acc[g.npairs] = 0;
-      }
-      if (lo >= 0)
-        for (int t = 0; t <= lo; t++, g.npairs++) {
-          g.pair_i[g.npairs] = t;
-          g.pair_j[g.npairs] = lo - t;
-          g.pair_acc[g.npairs] = 1;
-        }
-      g.C64 = acc;
-      g.ld64 = N;
-      g.ps64 = (long)M * N;
-      g.shift = shift;
-      g.err = c->d_err;
-      const int kc = lo >= 0 ? std::min(chunk(hi), chunk(lo)) : chunk(hi);
-      for (int k0 = 0; k0 < K; k0 += kc) {
-        g.k0 = k0;
-        g.k1 = k0 + kc < K ? k0 + kc : K;
-        const double part = flops * (double)(g.k1 - g.k0) / K;
-        timed(c, EV_TC, (lo == 0 || hi == 0) ? part : 0.0, part * g.npairs, 0, [&] { return launch_qgemm_tc(g, c->st); });
-      }
-    }
-    return Acc{acc, ACC_I64, (long)N, (long)M * N, eP, eQ, shift};
+    return Acc{g.C64, ACC_Q8, g.ld64, g.ps64, eP, eQ, plan.F + 1, plan.nparts};
   }
 
   // ---------------- combine helpers ----------------
@@ -610,7 +542,7 @@ struct Solver {
       a.acc_erow = acc->erow;
       a.acc_ecol = acc->ecol;
       a.acc_shift = acc->shift;
-      a.acc2 = acc->p2;
+      a.acc_sets = acc->sets;
     }
     return a;
   }
@@ -670,7 +602,7 @@ struct Solver {
     }
     double bytes = 0;
     const double el = (double)a.rows * a.cols * 4, ms = dbl ? 8 : 4;
-    if (a.acc) bytes += el * (a.acc_kind == ACC_F32 ? 4 : 8);
+    if (a.acc) bytes += el * (a.acc_kind == ACC_F32 ? 4 : a.acc_kind == ACC_F64 ? 8 : 16 * a.acc_sets);
     for (int t = 0; t < 4; t++)
       if (a.aux[t]) bytes += el * ms;
     for (int o = 0; o < a.nout; o++) {

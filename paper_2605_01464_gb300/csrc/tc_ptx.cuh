@@ -39,6 +39,22 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// One lane of the converged warp.  The issuing warps walk their loops with
+// all lanes and branch on this: the compiler then keeps the MMA's descriptors
+// in uniform registers.  With a branch on the lane index it moves every
+// operand of every MMA there first, which bounded the tensor core by the
+// issue rate (8-slice 2048^3 exact-slice product: 4.43 ms with the loops
+// inside a single-lane branch, 3.50 with warp-uniform loops and a lane test,
+// 2.92 with elect.sync).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xFFFFFFFF;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r != 0;
+}
 // Bounded wait: false if the abort flag is raised or WAIT_NS elapses (then
 // raises the flag and records `code` in *err).
 __device__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int code) {
@@ -147,28 +163,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   for (int t = 0; t < 32; t++) v[t] = __uint_as_float(r[t]);
 }
 
-__device__ __forceinline__ void tmem_ld32u(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_st32u(uint32_t taddr, const uint32_t* r) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
-        "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
-        "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-      : "memory");
-}
 // 32 lanes x 16 consecutive columns (one row of 16 values per thread).
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   uint32_t r[16];
@@ -190,25 +184,17 @@ __device__ __forceinline__ void tmem_ld16u(uint32_t taddr, uint32_t* r) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
+// 32 lanes x 8 consecutive columns.
+__device__ __forceinline__ void tmem_ld8u(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-// Epilogue row writers: lane j handles column j of up to 32 consecutive rows
+// Epilogue row writer: lane j handles column j of up to 32 consecutive rows
 // (stride ld) of a transposed 32 x 33 shared-memory block `st` (already offset
 // by the lane).  All loads are issued before any store so that the 32 row
 // accesses of a lane are in flight together.
-__device__ __forceinline__ void rmw_rows64(long long* __restrict__ dst, long ld, int nrow,
-                                           const long long* __restrict__ st) {
-#pragma unroll 1
-  for (int h = 0; h < 32; h += 16) {  // 16 rows in flight: bounded register use
-    long long g[16];
-#pragma unroll
-    for (int r = 0; r < 16; r++)
-      if (h + r < nrow) g[r] = dst[(long)(h + r) * ld];
-#pragma unroll
-    for (int r = 0; r < 16; r++)
-      if (h + r < nrow) dst[(long)(h + r) * ld] = g[r] + st[(h + r) * 33];
-  }
-}
 __device__ __forceinline__ void store_rows32(float* __restrict__ dst, long ld, int nrow,
                                              const float* __restrict__ st) {
   float g[32];
