@@ -143,12 +143,10 @@ typedef struct {
   int emu_pair;      /* -1 (default), 0 or 1: accepted for callers that set it, without effect.  It
                         chose between two exact-slice kernels with bit-identical results; one kernel,
                         faster than both at every size, has replaced them */
-  int tc_broad;      /* BF16-split products with M, N >= 128 and one accumulator on 128-column tiles
-                        (one CTA per SM, a 512-column TMEM accumulator) or 64-column tiles (two CTAs
-                        per SM): -1 (default) 128 columns for products without a fused combine
-                        epilogue (measured 10-19 % faster; with the epilogue the one CTA per SM
-                        cancels the gain), 1 always, 0 never.  Same arithmetic, bit-identical
-                        results */
+  int tc_broad;      /* tile shape of BF16-split products: -1 (default) chosen by size (128-column tiles
+                        when they fill the SMs, 64- or 32-column tiles with one output component per
+                        work item below), 1 always 128 columns, 0 always 64.  Same arithmetic,
+                        bit-identical results */
 } qpinv_options;
 
 typedef struct {

@@ -150,17 +150,17 @@ struct EpiOut {
   bf16* b = nullptr;  // B-form splits [level][comp][cols][ldb] (may be null)
   long ldb = 0, psb = 0;
   int levels = 0;
-  double cacc = 0.0, caux[4] = {0, 0, 0, 0}, diag = 0.0;  // rounded to the master type at use
+  double cacc = 0.0, caux[3] = {0, 0, 0}, diag = 0.0;  // rounded to the master type at use
 };
+constexpr int kEpiAux = 3;
 struct EpiArgs {
   int nout = 0;  // 0: plain FP32 store of the product into TcGemmArgs::C
   EpiOut out[kMaxOut];
-  const void* aux[4] = {nullptr, nullptr, nullptr, nullptr};  // planes of the master type
-  long ld_aux[4] = {0, 0, 0, 0}, ps_aux[4] = {0, 0, 0, 0};
-  double* partials = nullptr;  // 3 values per (CTA, epilogue warp): tc_partial_blocks(M, N) blocks (f64 == 0 only)
+  const void* aux[kEpiAux] = {nullptr, nullptr, nullptr};  // planes of the master type
+  long ld_aux[kEpiAux] = {0, 0, 0}, ps_aux[kEpiAux] = {0, 0, 0};
+  double* partials = nullptr;  // 3 values per (CTA, epilogue warp): tc_partial_blocks() blocks (f64 == 0 only)
   int f64 = 0;  // 1: aux inputs and output masters are double planes (FP64 arithmetic in the epilogue)
 };
-int tc_partial_blocks(int M, int N, int broad);
 
 // Tensor-core quaternion GEMM on BF16 split operands.  acc (FP32) = sum over
 // the listed (i, j) term pairs of A_i * B_j, restricted to k in [k0, k1).
@@ -173,11 +173,11 @@ struct TcGemmArgs {
   int pair_i[16] = {0}, pair_j[16] = {0};
   Planes<float> C;  // FP32 output
   EpiArgs epi;      // epi.nout > 0: fused combine instead of the plain store (FP32 output only)
-  int broad = -1;   // one-accumulator products with N >= 128 on 128-column tiles (one CTA per SM):
-                    // 1 always, 0 never, -1 when the epilogue is not fused
+  int broad = -1;   // tile shapes: 1 128 columns, 0 64 columns, -1 chosen by size
   int* err = nullptr;  // device error word (bounded-wait expiry)
 };
 cudaError_t launch_qgemm_tc(const TcGemmArgs& a, cudaStream_t st);
+int tc_partial_blocks(const TcGemmArgs& a);  // blocks of partials a fused launch of these arguments writes
 
 // FP64-accurate product from S exact slices per operand in one launch
 // (qgemm_emu.cu).  emu_plan chooses the tile width, the split of an item's

@@ -151,16 +151,17 @@ QMat mat(qpinv_ctx* c, const std::string& name, int rows, int cols, int masters,
   QMat M;
   M.rows = rows;
   M.cols = cols;
-  const long ps = (long)rows * cols;
   if (masters & MST_D) {
-    M.d.ld = cols;
-    M.d.ps = ps;
-    M.d.p = (double*)buf(c, name + ".d", sizeof(double) * 4 * (size_t)ps + 64);
+    // matrices that also have an FP32 master feed the GEMM epilogues: 16-byte
+    // rows keep their FP64 accesses vectorised too
+    M.d.ld = (masters & MST_F) ? (cols + 1) / 2 * 2 : cols;
+    M.d.ps = (long)rows * M.d.ld;
+    M.d.p = (double*)buf(c, name + ".d", sizeof(double) * 4 * (size_t)M.d.ps + 64);
   }
   if (masters & MST_F) {
-    // 16-byte rows, so that the tensor-core epilogues' FP32 accesses stay
+    // 32-byte rows, so that the tensor-core epilogues' FP32 accesses stay
     // vectorised for any column count
-    M.f.ld = (cols + 3) / 4 * 4;
+    M.f.ld = (cols + 7) / 8 * 8;
     M.f.ps = (long)rows * M.f.ld;
     M.f.p = (float*)buf(c, name + ".f", sizeof(float) * 4 * (size_t)M.f.ps + 64);
   }
@@ -388,7 +389,7 @@ struct Solver {
   // output that overwrites an operand form the product is still reading, and
   // in the FP64 phase no stop-test partials (those norms stay FP64 sums).
   bool epi_fusable(const CombineArgs& a, const QMat& P, const QMat& Q, bool with_partials) const {
-    if (!c->opt.fuse_epilogue || a.acc || a.nout < 1 || a.nout > kMaxOut) return false;
+    if (!c->opt.fuse_epilogue || a.acc || a.nout < 1 || a.nout > kMaxOut || a.aux[kEpiAux]) return false;
     if (a.f64 != (dbl ? 1 : 0) || (dbl && with_partials)) return false;
     for (int o = 0; o < a.nout; o++) {
       const OutSpec& O = a.out[o];
@@ -426,16 +427,16 @@ struct Solver {
         d.psb = O.s16.psb;
         d.levels = O.s16.levels;
         d.cacc = O.cacc;
-        for (int t = 0; t < 4; t++) d.caux[t] = O.caux[t];
+        for (int t = 0; t < kEpiAux; t++) d.caux[t] = O.caux[t];
         d.diag = O.diag;
       }
       e.f64 = a.f64;
-      for (int t = 0; t < 4; t++) {
+      for (int t = 0; t < kEpiAux; t++) {
         e.aux[t] = a.aux[t];
         e.ld_aux[t] = a.ld_aux[t];
         e.ps_aux[t] = a.ps_aux[t];
       }
-      const int blocks = tc_partial_blocks(M, N, c->opt.tc_broad);
+      const int blocks = tc_partial_blocks(g);
       if (with_partials) {
         if (blocks > partial_cap) {
           partials = (double*)buf(c, "partials", sizeof(double) * 3 * (size_t)blocks + 64);

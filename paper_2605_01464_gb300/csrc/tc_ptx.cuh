@@ -190,6 +190,30 @@ __device__ __forceinline__ void tmem_ld8u(uint32_t taddr, uint32_t* r) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(taddr));
 }
+// 16 lanes x 16 columns as two 16x256b fragments: value e of a lane is at row
+// lane / 4 + 8 ((e >> 1) & 1), column 8 (e >> 2) + 2 (lane % 4) + (e & 1).
+__device__ __forceinline__ void tmem_ld_16x16(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+// Four 8 x 8 BF16 matrices in that fragment layout to shared memory, as they
+// are or transposed; lane L gives the address of row L % 8 of matrix L / 8.
+__device__ __forceinline__ void st_matrix(uint32_t addr, const uint32_t* h) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(h[0]), "r"(h[1]),
+               "r"(h[2]), "r"(h[3])
+               : "memory");
+}
+__device__ __forceinline__ void st_matrix_trans(uint32_t addr, const uint32_t* h) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(h[0]),
+               "r"(h[1]), "r"(h[2]), "r"(h[3])
+               : "memory");
+}
+__device__ __forceinline__ uint4 ld_shared16(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // Epilogue row writer: lane j handles column j of up to 32 consecutive rows
 // (stride ld) of a transposed 32 x 33 shared-memory block `st` (already offset
