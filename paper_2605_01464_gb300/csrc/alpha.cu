@@ -137,54 +137,66 @@ __global__ void k_lanczos_next(const float* w, float* q, float* qprev, const dou
 }
 // One power-iteration step: y = M v with v = yprev / ||yprev|| (v = yprev on
 // the first step, d2prev null; 0 when the norm vanishes), and d2[0] = ||y||^2.
-// One warp per row; each block writes the sum of its rows' squares to
-// part[blockIdx.x], and the last block to finish (counted in *count, which it
-// resets) adds the block sums in a fixed order, so the result does not
-// depend on the blocks' timing.
-constexpr int PW_ROWS = 8;
-__global__ void __launch_bounds__(32 * PW_ROWS) k_power_step(Planes<const float> M, int s, const float* yprev,
-                                                             const double* d2prev, float* y, double* part,
-                                                             unsigned int* count, double* d2) {
-  __shared__ double wsum[PW_ROWS];
+// PW_WARPS warps per row, four adjacent entries per lane and step (16-byte
+// loads; rows are padded to 32 bytes): a 2048^2 step took 38 us with one warp
+// per row, too few loads in flight for a 67 MB matrix.  Each block writes the
+// sum of its rows' squares to part[blockIdx.x], and the last block to finish
+// (counted in *count, which it resets) adds the block sums in a fixed order, so
+// the result does not depend on the blocks' timing.
+constexpr int PW_ROWS = 2, PW_WARPS = 4;
+__global__ void __launch_bounds__(32 * PW_ROWS * PW_WARPS) k_power_step(Planes<const float> M, int s,
+                                                                        const float* yprev, const double* d2prev,
+                                                                        float* y, double* part, unsigned int* count,
+                                                                        double* d2) {
+  __shared__ double wsum[PW_ROWS * PW_WARPS];
+  __shared__ float racc[PW_ROWS * PW_WARPS][4];
   __shared__ int last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int row = blockIdx.x * PW_ROWS + warp;
+  const int rl = warp / PW_WARPS, row = blockIdx.x * PW_ROWS + rl;
   float inv = 1.f;
   if (d2prev) {
     const double b2 = d2prev[0];
     inv = b2 > 1e-60 ? (float)(1.0 / sqrt(b2)) : 0.f;
   }
-  double rs = 0.0;
+  float acc[4] = {0, 0, 0, 0};
   if (row < s) {
-    float acc[4] = {0, 0, 0, 0};
     const float* mr = M.p + (long)row * M.ld;
-#pragma unroll 4
-    for (int j = lane; j < s; j += 32) {
-      float a[4], b[4];
+#pragma unroll 2
+    for (int j = 4 * (lane + 32 * (warp % PW_WARPS)); j < s; j += 128 * PW_WARPS) {
+      float a[4][4];
 #pragma unroll
-      for (int c = 0; c < 4; c++) {
-        a[c] = mr[c * M.ps + j];
-        b[c] = yprev[4 * j + c] * inv;
+      for (int c = 0; c < 4; c++) *reinterpret_cast<float4*>(a[c]) = *reinterpret_cast<const float4*>(mr + c * M.ps + j);
+#pragma unroll
+      for (int t = 0; t < 4; t++) {
+        if (j + t >= s) break;
+        const float4 v = *reinterpret_cast<const float4*>(yprev + 4 * (j + t));
+        const float b0 = v.x * inv, b1 = v.y * inv, b2 = v.z * inv, b3 = v.w * inv;
+        acc[0] += a[0][t] * b0 - a[1][t] * b1 - a[2][t] * b2 - a[3][t] * b3;
+        acc[1] += a[0][t] * b1 + a[1][t] * b0 + a[2][t] * b3 - a[3][t] * b2;
+        acc[2] += a[0][t] * b2 - a[1][t] * b3 + a[2][t] * b0 + a[3][t] * b1;
+        acc[3] += a[0][t] * b3 + a[1][t] * b2 - a[2][t] * b1 + a[3][t] * b0;
       }
-      acc[0] += a[0] * b[0] - a[1] * b[1] - a[2] * b[2] - a[3] * b[3];
-      acc[1] += a[0] * b[1] + a[1] * b[0] + a[2] * b[3] - a[3] * b[2];
-      acc[2] += a[0] * b[2] - a[1] * b[3] + a[2] * b[0] + a[3] * b[1];
-      acc[3] += a[0] * b[3] + a[1] * b[2] - a[2] * b[1] + a[3] * b[0];
     }
-#pragma unroll
-    for (int c = 0; c < 4; c++)
-      for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
-    if (lane == 0)
-      for (int c = 0; c < 4; c++) {
-        y[4 * row + c] = acc[c];
-        rs += (double)acc[c] * acc[c];
-      }
   }
+#pragma unroll
+  for (int c = 0; c < 4; c++)
+    for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+  if (lane == 0)
+    for (int c = 0; c < 4; c++) racc[warp][c] = acc[c];
+  __syncthreads();
+  double rs = 0.0;
+  if (row < s && lane == 0 && warp % PW_WARPS == 0)
+    for (int c = 0; c < 4; c++) {
+      float t = racc[warp][c];
+      for (int w = 1; w < PW_WARPS; w++) t += racc[warp + w][c];
+      y[4 * row + c] = t;
+      rs += (double)t * t;
+    }
   if (lane == 0) wsum[warp] = rs;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
-    for (int w = 0; w < PW_ROWS; w++) t += wsum[w];
+    for (int w = 0; w < PW_ROWS * PW_WARPS; w++) t += wsum[w];
     part[blockIdx.x] = t;
     __threadfence();
     last = atomicAdd(count, 1u) == gridDim.x - 1;
@@ -199,7 +211,7 @@ __global__ void __launch_bounds__(32 * PW_ROWS) k_power_step(Planes<const float>
     __syncthreads();
     if (threadIdx.x == 0) {
       double r = 0.0;
-      for (int w = 0; w < PW_ROWS; w++) r += wsum[w];
+      for (int w = 0; w < PW_ROWS * PW_WARPS; w++) r += wsum[w];
       d2[0] = r;
       *count = 0;
     }
@@ -462,7 +474,7 @@ cudaError_t power_radius(const Planes<const float>& M, int s, int steps, float* 
   if ((e = cudaMemsetAsync(count, 0, sizeof(unsigned int), st)) != cudaSuccess) return e;
   float* buf2[2] = {v, y};
   for (int k = 0; k < steps; k++)
-    k_power_step<<<blocks, 32 * PW_ROWS, 0, st>>>(M, s, buf2[k & 1], k ? dscratch + k - 1 : nullptr,
+    k_power_step<<<blocks, 32 * PW_ROWS * PW_WARPS, 0, st>>>(M, s, buf2[k & 1], k ? dscratch + k - 1 : nullptr,
                                                     buf2[(k + 1) & 1], part, count, dscratch + k);
   g_kernel_launches += steps;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -39,6 +39,100 @@ struct Split16 {
   int levels = 0;
 };
 
+// A coefficient as the kernels read it: GB300's FP64 pipe does two operations
+// per clock and SM, so even a comparison of a double with 0 or 1 costs as much
+// as the arithmetic it saves; the host decides the kind once per launch.
+enum { CK_ZERO = 0, CK_ONE = 1, CK_MINUS = 2, CK_GENERAL = 3 };
+struct Coef {
+  double d = 0.0;
+  float f = 0.f;
+  int kind = CK_ZERO;
+  void set(double x) {
+    d = x;
+    f = (float)x;
+    kind = x == 0.0 ? CK_ZERO : x == 1.0 ? CK_ONE : x == -1.0 ? CK_MINUS : CK_GENERAL;
+  }
+};
+template <typename T>
+__device__ __forceinline__ T coef(const Coef& c);
+template <>
+__device__ __forceinline__ float coef<float>(const Coef& c) { return c.f; }
+template <>
+__device__ __forceinline__ double coef<double>(const Coef& c) { return c.d; }
+
+// FP32 <-> FP64 conversions from the bits, on the integer pipe (64 operations
+// per clock and SM) instead of the FP64 pipe's.  Zeros, subnormals, infinities
+// and NaN take the instruction.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x);
+  if (((b >> 23) & 0xFFu) - 1u >= 254u) return (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ float narrow(double x) {  // round to nearest even, as the cast
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t ex = (hi >> 20) & 0x7FFu;
+  if (ex - 897u >= 253u) return (float)x;  // below the FP32 normal range, or near overflow
+  const uint32_t m = ((ex - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
+  const uint32_t rem = lo & 0x1FFFFFFFu;
+  const uint32_t up = (rem > 0x10000000u || (rem == 0x10000000u && (m & 1u))) ? 1u : 0u;
+  return __uint_as_float((hi & 0x80000000u) | (m + up));
+}
+__device__ __forceinline__ float flip_sign(float x) { return -x; }
+__device__ __forceinline__ double flip_sign(double x) {
+  return __hiloint2double((int)((uint32_t)__double2hiint(x) ^ 0x80000000u), __double2loint(x));
+}
+template <typename T>
+__device__ __forceinline__ T to_master(float x);
+template <>
+__device__ __forceinline__ float to_master<float>(float x) { return x; }
+template <>
+__device__ __forceinline__ double to_master<double>(float x) { return widen(x); }
+__device__ __forceinline__ float to_float(float x) { return x; }
+__device__ __forceinline__ float to_float(double x) { return narrow(x); }
+
+// Block partial sums finished in the kernel that wrote them: the last block
+// to arrive (counted in *count, which it resets) adds the blocks' partials in
+// a fixed order (strided threads, shuffle, warp order), so the result does not
+// depend on the blocks' timing.  A pass with a stop test or a norm is then one
+// launch instead of two (a separate one-block reduction: 4-10 us each, 23 of
+// the 142 launches of a 64 x 48 solve).
+struct Reduce {
+  double* partials = nullptr;  // [block][nvals]
+  double* out = nullptr;       // nvals sums
+  unsigned int* count = nullptr;  // 0 between launches
+};
+// Every thread of the block calls this after its block's partials are
+// written (by any of its threads); sh: 32 doubles of shared memory.
+template <int NVALS>
+__device__ __forceinline__ void reduce_last_block(const Reduce& r, long nblocks, double* sh) {
+  __shared__ int last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned int total = gridDim.x * gridDim.y;
+    last = atomicAdd(r.count, 1u) == total - 1 ? 1 : 0;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+#pragma unroll
+  for (int v = 0; v < NVALS; v++) {
+    double s = 0.0;
+    for (long b = threadIdx.x; b < nblocks; b += blockDim.x) s += __ldcg(r.partials + b * NVALS + v);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) sh[warp] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int w = 0; w < warps; w++) t += sh[w];
+      r.out[v] = t;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) *r.count = 0;
+}
+
 // Output specification of the fused combine kernel:
 //   out = cacc * acc + sum_t caux[t] * aux_t + diag * I   (diag on plane s)
 // The master output (and every aux input) has the master type of the pass:
@@ -52,6 +146,12 @@ struct OutSpec {
   double cacc = 0.0;
   double caux[4] = {0, 0, 0, 0};
   double diag = 0.0;
+  Coef kacc, kaux[4], kdiag;  // set by the launch function
+  void set_coefs() {
+    kacc.set(cacc);
+    for (int t = 0; t < 4; t++) kaux[t].set(caux[t]);
+    kdiag.set(diag);
+  }
 };
 
 enum { ACC_F32 = 0, ACC_F64 = 1, ACC_Q8 = 2 };
@@ -75,7 +175,7 @@ struct CombineArgs {
   long ld_aux[4] = {0, 0, 0, 0}, ps_aux[4] = {0, 0, 0, 0};
   OutSpec out[kMaxOut];
   int nout = 0;
-  double* partials = nullptr;  // per block: ||out0 - aux0||^2, ||out0||^2, non-finite count
+  Reduce red;  // red.partials: sums of ||out0 - aux0||^2, ||out0||^2 and the non-finite count into red.out
 };
 
 }  // namespace qp
@@ -85,22 +185,24 @@ namespace qp {
 
 // blocks (and partials) launch_combine will use for these arguments
 int combine_blocks(const CombineArgs& a);
-cudaError_t launch_combine(const CombineArgs& a, cudaStream_t st, int* blocks_out);
-cudaError_t launch_reduce_partials(const double* partials, int nblocks, int nvals, double* out,
-                                   cudaStream_t st);
+cudaError_t launch_combine(const CombineArgs& a, cudaStream_t st);
 // colsum needs `scratch` of COL_SCRATCH(n) doubles
 cudaError_t launch_abs_sums(const Planes<const double>& A, int m, int n, double* rowsum,
                             double* colsum, double* scratch, cudaStream_t st);
 cudaError_t launch_max(const double* v, int n, double* out, cudaStream_t st);
 // scratch entries of a column reduction over `cols` columns
 inline long COL_SCRATCH(long cols) { return 64 * cols; }
-// Partials (sum of squares, non-finite count of A) of ||scale A + diag I - B||_F^2
-// (B optional; diag on plane s only): 2 doubles per block, *blocks_out blocks.
-cudaError_t launch_fro2_partials(const Planes<const double>& A, const Planes<const double>* B, int m,
-                                 int n, double* partials, cudaStream_t st, int* blocks_out, double scale = 1.0,
-                                 double diag = 0.0);
-cudaError_t launch_antiherm_partials(const Planes<const double>& M, int n, double* partials,
-                                     cudaStream_t st, int* blocks_out);
+// ||A - B||_F^2 (B optional) and the non-finite count of A into r.out[0..1];
+// partials for kFroBlocks blocks.
+constexpr int kFroBlocks = 1024;
+cudaError_t launch_fro2(const Planes<const double>& A, const Planes<const double>* B, int m, int n, const Reduce& r,
+                        cudaStream_t st);
+// The norms of a residual plane set R (n x n, FP64) that the Penrose pass
+// needs, in one read, into r.out[0..3] (partials of penrose_norm_blocks(n)
+// blocks): ||R||_F^2 without its diagonal's s plane, the sum of R_s(i, i)^2,
+// the sum of (sr R_s(i, i) + 1)^2 (sr = +-1), and ||R^H - R||_F^2.
+int penrose_norm_blocks(int n);
+cudaError_t launch_penrose_norms(const Planes<const double>& R, int n, double sr, const Reduce& r, cudaStream_t st);
 cudaError_t launch_init_x0(const Planes<const double>& A, int m, int n, double alpha, const Planes<double>& X,
                            cudaStream_t st);
 // Column exponents e (|v| < 2^e over the four planes); `scratch`: COL_SCRATCH(cols) ints
@@ -138,8 +240,7 @@ cudaError_t launch_qgemm_f64(int M, int K, int N, const Planes<const double>& A,
 // evaluated in the master type (FP32, or FP64 with f64 = 1) and written as a
 // master and/or round-to-nearest BF16 splits of its FP32 rounding (A-form
 // row-major, B-form transposed); in the FP32 case optionally with the
-// stop-test partials of output 0 (||out0 - aux0||^2, ||out0||^2, non-finite
-// count) per (CTA, epilogue warp).
+// stop-test sums of output 0 (||out0 - aux0||^2, ||out0||^2, non-finite count).
 // Outputs must not alias the product's operand forms (other CTAs are still
 // reading them); an output may alias an aux plane (same element, same thread).
 struct EpiOut {
@@ -150,7 +251,7 @@ struct EpiOut {
   bf16* b = nullptr;  // B-form splits [level][comp][cols][ldb] (may be null)
   long ldb = 0, psb = 0;
   int levels = 0;
-  double cacc = 0.0, caux[3] = {0, 0, 0}, diag = 0.0;  // rounded to the master type at use
+  Coef cacc, caux[3], diag;
 };
 constexpr int kEpiAux = 3;
 struct EpiArgs {
@@ -158,7 +259,7 @@ struct EpiArgs {
   EpiOut out[kMaxOut];
   const void* aux[kEpiAux] = {nullptr, nullptr, nullptr};  // planes of the master type
   long ld_aux[kEpiAux] = {0, 0, 0}, ps_aux[kEpiAux] = {0, 0, 0};
-  double* partials = nullptr;  // 3 values per (CTA, epilogue warp): tc_partial_blocks() blocks (f64 == 0 only)
+  Reduce red;  // red.partials: 3 values per (CTA, epilogue warp), tc_partial_blocks() of them (f64 == 0 only)
   int f64 = 0;  // 1: aux inputs and output masters are double planes (FP64 arithmetic in the epilogue)
 };
 

@@ -24,16 +24,32 @@ namespace {
 constexpr int TILE = 32;
 constexpr int TROWS = 8;  // block = 32 x 8 threads, each thread 4 rows of the tile
 
+// Sum over a block of 256 threads, valid in thread 0; sh: 256 doubles.  The
+// first warp adds eight entries per lane and then shuffles: 13 FP64
+// instructions per block (a shuffle tree in every warp takes 48, and GB300's
+// FP64 pipe needs 16 cycles for each).
 __device__ __forceinline__ double block_sum(double v, double* sh) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __syncthreads();
-  if (lane == 0) sh[warp] = v;
+  sh[threadIdx.x] = v;
   __syncthreads();
   double r = 0.0;
+  if (threadIdx.x < 32) {
+    r = sh[threadIdx.x];
+#pragma unroll
+    for (int k = 1; k < 8; k++) r += sh[threadIdx.x + 32 * k];
+    for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  }
+  return r;
+}
+__device__ __forceinline__ double block_count(int v, double* sh) {  // the same for counts
+  __syncthreads();
+  const int w = __reduce_add_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) reinterpret_cast<int*>(sh)[threadIdx.x >> 5] = w;
+  __syncthreads();
+  int r = 0;
   if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x >> 5); w++) r += sh[w];
-  return r;  // valid in thread 0 only
+    for (int k = 0; k < (int)(blockDim.x >> 5); k++) r += reinterpret_cast<int*>(sh)[k];
+  return (double)r;
 }
 
 // Inf / NaN from the exponent bits (integer instructions: GB300's FP64 pipe
@@ -42,16 +58,6 @@ __device__ __forceinline__ int nonfinite_bits(double x) {
   return ((__double_as_longlong(x) >> 52) & 0x7FF) == 0x7FF ? 1 : 0;
 }
 __device__ __forceinline__ int nonfinite_bits(float x) { return ((__float_as_int(x) >> 23) & 0xFF) == 0xFF ? 1 : 0; }
-
-// Round-to-nearest BF16 split of the FP32 value: 3 terms cover all 24 bits.
-__device__ __forceinline__ void split_store(bf16* base, long idx, long lstride, int levels, float v) {
-  float r = v;
-  for (int l = 0; l < levels; l++) {
-    const bf16 t = __float2bfloat16_rn(r);
-    base[l * lstride + idx] = t;
-    r -= __bfloat162float(t);
-  }
-}
 
 // round(v * 2^sh) as an integer, from the bits of v (integer arithmetic only).
 // Requires |v * 2^sh| < 2^62; subnormal inputs count as zero.
@@ -90,27 +96,42 @@ __device__ __forceinline__ int exp_of(float v) {
   return ex == 0 ? -100000 : ex - 126;
 }
 
-// q 2^e as a double, rounded to nearest (ties to even) from the integer bits:
-// the same value as ldexp((double)q, e), without FP64 arithmetic (GB300's
-// FP64 rate is a small fraction of its integer rate).  Results below the
-// normal range or above the finite range take ldexp.
+// q 2^e rounded to nearest (ties to even) as a double or float, from the
+// integer bits: the same value as ldexp((T)q, e) without FP64 arithmetic or
+// 64-bit conversion instructions.  Results outside the normal range take ldexp.
+// The leading one is shifted to bit 63; the kept bits including it are added
+// to the exponent field one too low, so that a rounding carry moves into it.
+__device__ __noinline__ double i64_scaled_slow(long long q, int e) { return ldexp((double)q, e); }
+__device__ __noinline__ float i64_scaledf_slow(long long q, int e) { return ldexpf((float)q, e); }
+__device__ __forceinline__ unsigned long long i64_norm(long long q, uint32_t& sign, int& lz) {
+  sign = (uint32_t)((unsigned long long)q >> 32) & 0x80000000u;
+  const unsigned long long mag = q < 0 ? 0ull - (unsigned long long)q : (unsigned long long)q;
+  lz = __clzll((long long)mag);
+  return mag << (lz & 63);
+}
 __device__ __forceinline__ double i64_scaled(long long q, int e) {
-  if (q == 0) return 0.0;
-  const unsigned long long sgn = q < 0 ? (1ull << 63) : 0ull;
-  unsigned long long mag = q < 0 ? 0ull - (unsigned long long)q : (unsigned long long)q;
-  const int lz = __clzll((long long)mag);
-  mag <<= lz;  // leading one at bit 63
-  unsigned long long m = mag >> 11;  // 53 significant bits
-  const unsigned long long rem = mag & 0x7FFull;
-  if (rem > 0x400ull || (rem == 0x400ull && (m & 1ull))) m++;
-  int ex = 63 - lz + e;  // value = m 2^(ex - 52)
-  if (m >> 53) {
-    m >>= 1;
-    ex++;
-  }
-  const int biased = ex + 1023;
-  if (biased <= 0 || biased >= 2047) return ldexp((double)q, e);
-  return __longlong_as_double((long long)(sgn | ((unsigned long long)biased << 52) | (m & 0xFFFFFFFFFFFFFull)));
+  uint32_t sign;
+  int lz;
+  const unsigned long long mag = i64_norm(q, sign, lz);
+  const int biased = 1023 + 63 - lz + e;
+  if ((unsigned)(biased - 1) >= 2045u) return q == 0 ? 0.0 : i64_scaled_slow(q, e);
+  const unsigned long long m = mag >> 11;
+  const uint32_t up = (((uint32_t)mag & 0x7FFu) + 0x3FFu + ((uint32_t)m & 1u)) >> 11;
+  const unsigned long long b = m + up + ((unsigned long long)(uint32_t)(biased - 1) << 52);
+  return q == 0 ? 0.0 : __longlong_as_double((long long)(b | ((unsigned long long)sign << 32)));
+}
+__device__ __forceinline__ float i64_scaledf(long long q, int e) {
+  uint32_t sign;
+  int lz;
+  const unsigned long long mag = i64_norm(q, sign, lz);
+  const int biased = 127 + 63 - lz + e;
+  if ((unsigned)(biased - 1) >= 253u) return q == 0 ? 0.f : i64_scaledf_slow(q, e);
+  const uint32_t hi = (uint32_t)(mag >> 32), m = hi >> 8;
+  // bits below the last kept one, the low word folded into a sticky bit
+  const uint32_t rest = ((hi & 0xFFu) << 1) | ((uint32_t)mag != 0 ? 1u : 0u);
+  const uint32_t up = (rest + 0xFFu + (m & 1u)) >> 9;
+  const uint32_t b = m + up + ((uint32_t)(biased - 1) << 23);
+  return q == 0 ? 0.f : __uint_as_float(b | sign);
 }
 
 // Twice the four components from the eight real products of the exact-slice
@@ -125,164 +146,48 @@ __device__ __forceinline__ void quad_of(const unsigned long long* p, long long* 
 }
 template <typename T>
 __device__ __forceinline__ T q8_value(long long q, int e) {
-  if (sizeof(T) == 4) return (T)ldexpf((float)q, e);
+  if (sizeof(T) == 4) return (T)i64_scaledf(q, e);
   return (T)i64_scaled(q, e);
 }
 
-// The accumulator's four components at (i, j).
+// Two adjacent values (the second if `two`), one access where the address allows.
+template <typename T2, typename T>
+__device__ __forceinline__ void load_pair(const T* p, bool two, T& x, T& y) {
+  if (two && (reinterpret_cast<uintptr_t>(p) & (sizeof(T2) - 1)) == 0) {
+    const T2 t = *reinterpret_cast<const T2*>(p);
+    x = t.x;
+    y = t.y;
+  } else {
+    x = p[0];
+    y = two ? p[1] : (T)0;
+  }
+}
+__device__ __forceinline__ void ld2(const float* p, bool two, float& x, float& y) { load_pair<float2>(p, two, x, y); }
+__device__ __forceinline__ void ld2(const double* p, bool two, double& x, double& y) {
+  load_pair<double2>(p, two, x, y);
+}
+__device__ __forceinline__ void st2(float* p, bool two, float x, float y) {
+  if (two && (reinterpret_cast<uintptr_t>(p) & 7) == 0) *reinterpret_cast<float2*>(p) = make_float2(x, y);
+  else {
+    p[0] = x;
+    if (two) p[1] = y;
+  }
+}
+__device__ __forceinline__ void st2(double* p, bool two, double x, double y) {
+  if (two && (reinterpret_cast<uintptr_t>(p) & 15) == 0) *reinterpret_cast<double2*>(p) = make_double2(x, y);
+  else {
+    p[0] = x;
+    if (two) p[1] = y;
+  }
+}
+
+// cacc times the accumulator's four components at (i, j) and (i, j + 1);
+// cacc = +-1 is a sign (for the fixed-point planes, of the integer).
 template <typename T>
-__device__ __forceinline__ void acc_values(const CombineArgs& a, int i, int j, T* v) {
+__device__ __forceinline__ void acc_pairs(const CombineArgs& a, const Coef& k, int i, int j, bool two, T (*v)[2]) {
   const long off = (long)i * a.ld_acc + j;
   if (a.acc_kind == ACC_Q8) {
-    unsigned long long p[8];
-    const unsigned long long* src = (const unsigned long long*)a.acc + off;
-#pragma unroll
-    for (int t = 0; t < 8; t++) p[t] = src[t * a.ps_acc];
-    for (int s = 1; s < a.acc_sets; s++) {
-      src += 8 * a.ps_acc;
-#pragma unroll
-      for (int t = 0; t < 8; t++) p[t] += src[t * a.ps_acc];
-    }
-    long long q[4];
-    quad_of(p, q);
-    const int e = a.acc_erow[i] + a.acc_ecol[j] - a.acc_shift;
-#pragma unroll
-    for (int c = 0; c < 4; c++) v[c] = q8_value<T>(q[c], e);
-    return;
-  }
-#pragma unroll
-  for (int c = 0; c < 4; c++)
-    v[c] = a.acc_kind == ACC_F64 ? (T)((const double*)a.acc)[c * a.ps_acc + off]
-                                 : (T)((const float*)a.acc)[c * a.ps_acc + off];
-}
-
-// cacc x for cacc = +-1 without arithmetic (a sign flip), else the product.
-template <typename T>
-__device__ __forceinline__ T times_coef(T x, T cacc) {
-  if (cacc == (T)1) return x;
-  if (cacc == (T)-1) return -x;
-  return cacc * x;
-}
-
-// One 32x32 tile per block; threads (tx, ty), tid = ty * 32 + tx.
-template <typename T>
-__global__ void __launch_bounds__(256) k_combine(CombineArgs a) {
-  __shared__ T stage[4][TILE][TILE + 1];
-  __shared__ double red[8];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int r0 = blockIdx.y * TILE, c0 = blockIdx.x * TILE;
-  T s_dx = 0, s_x = 0;
-  int s_bad = 0;
-
-  for (int o = 0; o < a.nout; o++) {
-    const OutSpec& O = a.out[o];
-    const T cacc = (T)O.cacc, diag = (T)O.diag;
-    for (int q = 0; q < TILE / TROWS; q++) {
-      const int i = r0 + ty + q * TROWS, j = c0 + tx;
-      T v[4] = {0, 0, 0, 0};
-      if (i < a.rows && j < a.cols) {
-        if (a.acc && O.cacc != 0.0) {
-          acc_values<T>(a, i, j, v);
-          for (int c = 0; c < 4; c++) v[c] = times_coef<T>(v[c], cacc);
-        }
-        for (int t = 0; t < 4; t++) {
-          if (!a.aux[t] || O.caux[t] == 0.0) continue;
-          const T* ap = (const T*)a.aux[t];
-          const T ct = (T)O.caux[t];
-          for (int c = 0; c < 4; c++) v[c] += ct * ap[c * a.ps_aux[t] + (long)i * a.ld_aux[t] + j];
-        }
-        if (i == j) v[0] += diag;
-        if (o == 0 && a.partials) {
-          const T* x0p = (const T*)a.aux[0];
-          for (int c = 0; c < 4; c++) {
-            s_x += v[c] * v[c];
-            if (x0p) {
-              const T dx = v[c] - x0p[c * a.ps_aux[0] + (long)i * a.ld_aux[0] + j];
-              s_dx += dx * dx;
-            }
-            s_bad += nonfinite_bits(v[c]);
-          }
-        }
-        if (O.mp)
-          for (int c = 0; c < 4; c++) ((T*)O.mp)[c * O.mps + (long)i * O.mld + j] = v[c];
-        if (O.s16.a) {
-          for (int c = 0; c < 4; c++) {
-            const long idx = c * O.s16.psa + (long)i * O.s16.lda + j;
-            split_store(O.s16.a, idx, 4 * O.s16.psa, O.s16.levels, (float)v[c]);
-          }
-        }
-      }
-      if (O.s16.b)
-        for (int c = 0; c < 4; c++) stage[c][ty + q * TROWS][tx] = v[c];
-    }
-    if (O.s16.b) {
-      __syncthreads();
-      for (int q = 0; q < TILE / TROWS; q++) {
-        const int jj = c0 + ty + q * TROWS, ii = r0 + tx;  // B-form element (jj, ii) = out(ii, jj)
-        if (ii < a.rows && jj < a.cols) {
-          for (int c = 0; c < 4; c++) {
-            const long idx = c * O.s16.psb + (long)jj * O.s16.ldb + ii;
-            const T val = stage[c][tx][ty + q * TROWS];
-            split_store(O.s16.b, idx, 4 * O.s16.psb, O.s16.levels, (float)val);
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
-  if (a.partials) {
-    if (!a.aux[0]) s_dx = s_x;  // ||v - 0||^2
-    const long b = (long)blockIdx.y * gridDim.x + blockIdx.x;
-    const double t0 = block_sum((double)s_dx, red);
-    const double t1 = block_sum((double)s_x, red);
-    const double t2 = block_sum((double)s_bad, red);
-    if (threadIdx.x == 0) {
-      a.partials[3 * b + 0] = t0;
-      a.partials[3 * b + 1] = t1;
-      a.partials[3 * b + 2] = t2;
-    }
-  }
-}
-
-// FP32 passes over column pairs: 32 rows x 64 columns per block, each thread
-// two adjacent columns (8-byte loads and stores, packed BF16 pairs), which
-// halves the index arithmetic and store instructions per element.  Needs even
-// leading dimensions and plane strides for every FP32 / FP64 / int64 plane it
-// touches (combine_pairs_ok); the BF16 forms have ld, ps multiples of 8.
-__device__ __forceinline__ void split_store2(bf16* base, long idx, long lstride, int levels, float x, float y) {
-  float rx = x, ry = y;
-  for (int l = 0; l < levels; l++) {
-    const __nv_bfloat162 t = __floats2bfloat162_rn(rx, ry);
-    *reinterpret_cast<__nv_bfloat162*>(base + l * lstride + idx) = t;
-    rx -= __low2float(t);
-    ry -= __high2float(t);
-  }
-}
-
-// The accumulator's four components at (i, j) and (i, j + 1).
-__device__ __forceinline__ void acc_pairs(const CombineArgs& a, int i, int j, bool two, float (*v)[2]) {
-  const long off = (long)i * a.ld_acc + j;
-  if (a.acc_kind == ACC_F32) {
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-      const float* p = (const float*)a.acc + c * a.ps_acc + off;
-      if (two) {
-        const float2 t = *reinterpret_cast<const float2*>(p);
-        v[c][0] = t.x;
-        v[c][1] = t.y;
-      } else {
-        v[c][0] = p[0];
-      }
-    }
-  } else if (a.acc_kind == ACC_F64) {
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-      const double* p = (const double*)a.acc + c * a.ps_acc + off;
-      v[c][0] = (float)p[0];
-      if (two) v[c][1] = (float)p[1];
-    }
-  } else {
-    // the planes' rows are padded to a multiple of 4: the pair load stays inside
+    // the planes' rows are padded to a multiple of 4: the pair loads stay inside
     unsigned long long p0[8], p1[8];
     const unsigned long long* src = (const unsigned long long*)a.acc + off;
 #pragma unroll
@@ -305,140 +210,172 @@ __device__ __forceinline__ void acc_pairs(const CombineArgs& a, int i, int j, bo
     quad_of(p1, q1);
     const int er = a.acc_erow[i] - a.acc_shift;
     const int e0 = er + a.acc_ecol[j], e1 = two ? er + a.acc_ecol[j + 1] : 0;
+    const bool neg = k.kind == CK_MINUS;
 #pragma unroll
     for (int c = 0; c < 4; c++) {
-      v[c][0] = ldexpf((float)q0[c], e0);
-      if (two) v[c][1] = ldexpf((float)q1[c], e1);
+      v[c][0] = q8_value<T>(neg ? -q0[c] : q0[c], e0);
+      v[c][1] = two ? q8_value<T>(neg ? -q1[c] : q1[c], e1) : (T)0;
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      if (a.acc_kind == ACC_F64) {
+        double x, y;
+        ld2((const double*)a.acc + c * a.ps_acc + off, two, x, y);
+        v[c][0] = (T)x;
+        v[c][1] = (T)y;
+      } else {
+        float x, y;
+        ld2((const float*)a.acc + c * a.ps_acc + off, two, x, y);
+        v[c][0] = to_master<T>(x);
+        v[c][1] = to_master<T>(y);
+      }
+      if (k.kind == CK_MINUS) {
+        v[c][0] = flip_sign(v[c][0]);
+        v[c][1] = flip_sign(v[c][1]);
+      }
+    }
+  }
+  if (k.kind == CK_GENERAL) {
+    const T x = coef<T>(k);
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      v[c][0] *= x;
+      v[c][1] *= x;
     }
   }
 }
 
-__global__ void __launch_bounds__(256) k_combine_f2(CombineArgs a) {
+// Round-to-nearest BF16 splits of two adjacent FP32 values.
+__device__ __forceinline__ void split_store2(bf16* base, long idx, long lstride, int levels, float x, float y) {
+  float rx = x, ry = y;
+  for (int l = 0; l < levels; l++) {
+    const __nv_bfloat162 t = __floats2bfloat162_rn(rx, ry);
+    *reinterpret_cast<__nv_bfloat162*>(base + l * lstride + idx) = t;
+    rx -= __low2float(t);
+    ry -= __high2float(t);
+  }
+}
+
+// Combine pass over column pairs: a block takes 8 `groups` rows x 64 columns,
+// a thread two adjacent columns of one row per group (8- or 16-byte accesses,
+// packed BF16 pairs).  Bound: HBM, once nothing but the pass's own additions
+// runs on the FP64 pipe: coefficients carry a host-side kind (comparing a
+// double with 0 or 1 is FP64 work; it was most of the former kernel's 6 FP64
+// instructions per value), conversions and sign flips are integer operations.
+template <typename T>
+__global__ void __launch_bounds__(256) k_combine(const __grid_constant__ CombineArgs a, int groups) {
   __shared__ float stage[4][2 * TILE][TILE + 1];  // [plane][column][row]
-  __shared__ double red[8];
+  __shared__ double red[256];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int r0 = blockIdx.y * TILE, c0 = blockIdx.x * 2 * TILE;
+  const int rows_b = TROWS * groups, r0 = blockIdx.y * rows_b, c0 = blockIdx.x * 2 * TILE;
   const int j = c0 + 2 * tx;
-  float s_dx = 0.f, s_x = 0.f;
+  T s_dx = 0, s_x = 0;
   int s_bad = 0;
 
   for (int o = 0; o < a.nout; o++) {
     const OutSpec& O = a.out[o];
-    const float cacc = (float)O.cacc, diag = (float)O.diag;
-    for (int q = 0; q < TILE / TROWS; q++) {
+    for (int q = 0; q < groups; q++) {
       const int i = r0 + ty + q * TROWS;
-      float v[4][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+      T v[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
       const bool in0 = i < a.rows && j < a.cols, two = in0 && j + 1 < a.cols;
       if (in0) {
-        if (a.acc && O.cacc != 0.0) {
-          acc_pairs(a, i, j, two, v);
+        if (a.acc && O.kacc.kind != CK_ZERO) acc_pairs<T>(a, O.kacc, i, j, two, v);
+#pragma unroll
+        for (int t = 0; t < 4; t++) {
+          if (!a.aux[t] || O.kaux[t].kind == CK_ZERO) continue;
+          const T* ap = (const T*)a.aux[t] + (long)i * a.ld_aux[t] + j;
+          const T ct = coef<T>(O.kaux[t]);
+          T u[4][2];
+#pragma unroll
+          for (int c = 0; c < 4; c++) ld2(ap + c * a.ps_aux[t], two, u[c][0], u[c][1]);
 #pragma unroll
           for (int c = 0; c < 4; c++) {
-            v[c][0] *= cacc;
-            v[c][1] *= cacc;
+            v[c][0] += ct * u[c][0];
+            v[c][1] += ct * u[c][1];
           }
         }
-        for (int t = 0; t < 4; t++) {
-          if (!a.aux[t] || O.caux[t] == 0.0) continue;
-          const float* ap = (const float*)a.aux[t];
-          const float ct = (float)O.caux[t];
+        if (O.kdiag.kind != CK_ZERO) {
+          if (i == j) v[0][0] += coef<T>(O.kdiag);
+          if (two && i == j + 1) v[0][1] += coef<T>(O.kdiag);
+        }
+        if (o == 0 && a.red.partials) {
+          const T* x0p = (const T*)a.aux[0];
+#pragma unroll
           for (int c = 0; c < 4; c++) {
-            const long off = c * a.ps_aux[t] + (long)i * a.ld_aux[t] + j;
-            if (two) {
-              const float2 u = *reinterpret_cast<const float2*>(ap + off);
-              v[c][0] += ct * u.x;
-              v[c][1] += ct * u.y;
-            } else {
-              v[c][0] += ct * ap[off];
-            }
-          }
-        }
-        if (i == j) v[0][0] += diag;
-        if (two && i == j + 1) v[0][1] += diag;
-        if (o == 0 && a.partials) {
-          const float* x0p = (const float*)a.aux[0];
-          for (int c = 0; c < 4; c++)
-            for (int h = 0; h < (two ? 2 : 1); h++) {
-              const float x0 = x0p ? x0p[c * a.ps_aux[0] + (long)i * a.ld_aux[0] + j + h] : 0.f;
-              s_dx += (v[c][h] - x0) * (v[c][h] - x0);
+            T x0[2] = {0, 0};
+            if (x0p) ld2(x0p + c * a.ps_aux[0] + (long)i * a.ld_aux[0] + j, two, x0[0], x0[1]);
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+              if (h && !two) continue;
               s_x += v[c][h] * v[c][h];
-              s_bad += isfinite(v[c][h]) ? 0 : 1;
+              if (x0p) {
+                const T dx = v[c][h] - x0[h];
+                s_dx += dx * dx;
+              }
+              s_bad += nonfinite_bits(v[c][h]);
             }
+          }
         }
-        if (O.mp)
-          for (int c = 0; c < 4; c++) {
-            float* dst = (float*)O.mp + c * O.mps + (long)i * O.mld + j;
-            if (two) *reinterpret_cast<float2*>(dst) = make_float2(v[c][0], v[c][1]);
-            else dst[0] = v[c][0];
-          }
-        if (O.s16.a)
-          for (int c = 0; c < 4; c++) {
-            const long idx = c * O.s16.psa + (long)i * O.s16.lda + j;
-            if (two) {
-              split_store2(O.s16.a, idx, 4 * O.s16.psa, O.s16.levels, v[c][0], v[c][1]);
-            } else {
-              split_store(O.s16.a, idx, 4 * O.s16.psa, O.s16.levels, v[c][0]);
-            }
-          }
+        if (O.mp) {
+          T* dst = (T*)O.mp + (long)i * O.mld + j;
+#pragma unroll
+          for (int c = 0; c < 4; c++) st2(dst + c * O.mps, two, v[c][0], v[c][1]);
+        }
+        if (O.s16.a) {
+          // operand rows are padded to 64 entries: the pair's second half is
+          // written beyond an odd width too (zero)
+          const long idx = (long)i * O.s16.lda + j;
+#pragma unroll
+          for (int c = 0; c < 4; c++)
+            split_store2(O.s16.a, c * O.s16.psa + idx, 4 * O.s16.psa, O.s16.levels, to_float(v[c][0]),
+                         to_float(v[c][1]));
+        }
       }
-      if (O.s16.b)
+      if (O.s16.b) {
+#pragma unroll
         for (int c = 0; c < 4; c++) {
-          stage[c][2 * tx][ty + q * TROWS] = v[c][0];
-          stage[c][2 * tx + 1][ty + q * TROWS] = v[c][1];
+          stage[c][2 * tx][ty + q * TROWS] = to_float(v[c][0]);
+          stage[c][2 * tx + 1][ty + q * TROWS] = to_float(v[c][1]);
         }
+      }
     }
     if (O.s16.b) {
       __syncthreads();
-      // B-form row jj (an output column) holds the block's 32 rows ii: thread
-      // t writes the pair ii = 2 (t % 16), +1 of columns t / 16 + 16 k.
-      const int p = threadIdx.x & 15;
-      for (int k = 0; k < 4; k++) {
-        const int jl = (threadIdx.x >> 4) + 16 * k, jj = c0 + jl, ii = r0 + 2 * p;
+      // B-form row jj (an output column) holds the block's rows in pairs
+      const int np = rows_b / 2;
+      for (int t = threadIdx.x; t < 2 * TILE * np; t += 256) {
+        const int jl = t / np, p = t % np, jj = c0 + jl, ii = r0 + 2 * p;
         if (jj < a.cols && ii < a.rows) {
-          const bool pair = ii + 1 < a.rows;
-          for (int c = 0; c < 4; c++) {
-            const long idx = c * O.s16.psb + (long)jj * O.s16.ldb + ii;
-            const float x = stage[c][jl][2 * p], y = stage[c][jl][2 * p + 1];
-            if (pair) {
-              split_store2(O.s16.b, idx, 4 * O.s16.psb, O.s16.levels, x, y);
-            } else {
-              split_store(O.s16.b, idx, 4 * O.s16.psb, O.s16.levels, x);
-            }
-          }
+          const long idx = (long)jj * O.s16.ldb + ii;
+#pragma unroll
+          for (int c = 0; c < 4; c++)
+            split_store2(O.s16.b, c * O.s16.psb + idx, 4 * O.s16.psb, O.s16.levels, stage[c][jl][2 * p],
+                         stage[c][jl][2 * p + 1]);
         }
       }
       __syncthreads();
     }
   }
-  if (a.partials) {
+  if (a.red.partials) {
+    if (!a.aux[0]) s_dx = s_x;  // ||v - 0||^2
     const long b = (long)blockIdx.y * gridDim.x + blockIdx.x;
     const double t0 = block_sum((double)s_dx, red);
     const double t1 = block_sum((double)s_x, red);
-    const double t2 = block_sum((double)s_bad, red);
+    const double t2 = block_count(s_bad, red);
     if (threadIdx.x == 0) {
-      a.partials[3 * b + 0] = t0;
-      a.partials[3 * b + 1] = t1;
-      a.partials[3 * b + 2] = t2;
+      a.red.partials[3 * b + 0] = t0;
+      a.red.partials[3 * b + 1] = t1;
+      a.red.partials[3 * b + 2] = t2;
     }
+    reduce_last_block<3>(a.red, (long)gridDim.x * gridDim.y, red);
   }
 }
 
-// The pair kernel applies to FP32 passes whose FP32 / FP64 / int64 planes all
-// have even leading dimensions, plane strides and 16-byte aligned bases.
-static bool combine_pairs_ok(const CombineArgs& a) {
-  if (a.f64) return false;
-  auto even = [](long x) { return (x & 1) == 0; };
-  auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  if (a.acc && (!even(a.ld_acc) || !even(a.ps_acc) || !al(a.acc))) return false;
-  for (int t = 0; t < 4; t++)
-    if (a.aux[t] && (!even(a.ld_aux[t]) || !even(a.ps_aux[t]) || !al(a.aux[t]))) return false;
-  for (int o = 0; o < a.nout; o++) {
-    const OutSpec& O = a.out[o];
-    if (O.mp && (!even(O.mld) || !even(O.mps) || !al(O.mp))) return false;
-    if (O.s16.a && (!al(O.s16.a) || (O.s16.lda & 1) || (O.s16.psa & 1))) return false;
-    if (O.s16.b && (!al(O.s16.b) || (O.s16.ldb & 1) || (O.s16.psb & 1))) return false;
-  }
-  return true;
+// Row groups of 8 per block: four, or one while that leaves SMs without work.
+static int combine_groups(const CombineArgs& a) {
+  const long blocks = (long)((a.cols + 2 * TILE - 1) / (2 * TILE)) * ((a.rows + TILE - 1) / TILE);
+  return blocks < 2 * 152 ? 1 : TILE / TROWS;
 }
 
 // ---------------------------------------------------------------- exact slicing
@@ -506,7 +443,7 @@ __device__ __forceinline__ void slices_store(bf16* dst, long ps, int S, int p0, 
 // then slice it (the second read hits L1 / L2: a row is at most a few
 // hundred KB), so no separate exponent pass is needed.
 template <typename T, int WPR>
-__global__ void __launch_bounds__(256) k_slice_rows(Planes<const T> A, int rows, int cols, int* __restrict__ e_out,
+__global__ void __launch_bounds__(256, 2) k_slice_rows(Planes<const T> A, int rows, int cols, int* __restrict__ e_out,
                                                     int S, int p0, int np, bf16* dst, long ld, long ps) {
   __shared__ int sh[8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -552,7 +489,7 @@ __global__ void __launch_bounds__(256) k_slice_rows(Planes<const T> A, int rows,
 // bytes of each of 4 slice rows).  Rows past `rows` up to the padded pitch are 0.
 constexpr int SC_ROWS = 64, SC_COLS = 32;
 template <typename T>
-__global__ void __launch_bounds__(256) k_slice_cols(Planes<const T> A, int rows, int cols, const int* __restrict__ e,
+__global__ void __launch_bounds__(256, 2) k_slice_cols(Planes<const T> A, int rows, int cols, const int* __restrict__ e,
                                                     int S, int p0, int np, bf16* dst, long ld, long ps) {
   extern __shared__ __align__(16) unsigned char sc_smem[];
   T(*tile)[SC_COLS][SC_ROWS + 1] = reinterpret_cast<T(*)[SC_COLS][SC_ROWS + 1]>(sc_smem);
@@ -580,16 +517,6 @@ __global__ void __launch_bounds__(256) k_slice_cols(Planes<const T> A, int rows,
       slice_bias<T>(v, S, ej, G[c]);
     }
     slices_store<false>(dst + (long)j * ld + i0 + ig, ps, S, p0, np, G);
-  }
-}
-
-__global__ void k_reduce_partials(const double* p, int nblocks, int nvals, double* out) {
-  __shared__ double sh[8];
-  for (int v = 0; v < nvals; v++) {
-    double s = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) s += p[(long)b * nvals + v];
-    const double t = block_sum(s, sh);
-    if (threadIdx.x == 0) out[v] = t;
   }
 }
 
@@ -658,83 +585,108 @@ __global__ void k_max(const double* v, int n, double* out) {
   if (threadIdx.x == 0) out[0] = sh[0];
 }
 
-// partials per block: sum |A - B|^2 (or |A|^2 if B is null), non-finite count of A.
-// ||scale A + diag I - B||_F^2 (B optional; diag on plane s) and the
-// non-finite count of A.  Work is split into tasks of one row and FRO_COLS
-// consecutive columns; a block takes tasks blockIdx.x + k gridDim.x, FRO_U of
-// them at a time with all their loads of A issued before the first use.  Per
-// element four FP64 FMAs (and the scaling and the subtraction of B where
-// asked).
+// ||A - B||_F^2 (B optional) and the non-finite count of A.  Work is split
+// into tasks of one row and FRO_COLS consecutive columns; a block takes tasks
+// blockIdx.x + k gridDim.x, FRO_U of them at a time with all their loads of A
+// issued before the first use.  FP64 pipe: one FMA per value and nothing else
+// (a run-time scale compared with 1.0 and a diagonal term compared with 0.0
+// made it four: 136 us for a 2048^2 matrix, 20 at the copy bandwidth).
 constexpr int FRO_COLS = 256, FRO_U = 2;
-__global__ void __launch_bounds__(FRO_COLS) k_fro2(Planes<const double> A, Planes<const double> B, int hasB, int m,
-                                                   int n, double scale, double diag, double* partials) {
-  __shared__ double sh[8];
-  const long chunks = (n + FRO_COLS - 1) / FRO_COLS, tasks = (long)m * chunks;
+template <bool HASB>
+__global__ void __launch_bounds__(FRO_COLS) k_fro2(Planes<const double> A, Planes<const double> B, int m, int n,
+                                                   Reduce r) {
+  __shared__ double sh[256];
+  const unsigned chunks = (n + FRO_COLS - 1) / FRO_COLS;
+  const unsigned tasks = (unsigned)m * chunks;  // below 2^31 for any matrix that fits the device
   double s = 0.0;
   int bad = 0;
-  for (long t0 = blockIdx.x; t0 < tasks; t0 += (long)FRO_U * gridDim.x) {
+  for (unsigned t0 = blockIdx.x; t0 < tasks; t0 += FRO_U * gridDim.x) {
     double x[FRO_U][4];
-    long ii[FRO_U];
+    long off[FRO_U];
     int jj[FRO_U];
     bool ok[FRO_U];
 #pragma unroll
     for (int u = 0; u < FRO_U; u++) {
-      const long t = t0 + (long)u * gridDim.x;
-      ii[u] = t / chunks;
-      jj[u] = (int)(t - ii[u] * chunks) * FRO_COLS + threadIdx.x;
+      const unsigned t = t0 + u * gridDim.x, row = t / chunks;
+      off[u] = row;
+      jj[u] = (int)(t - row * chunks) * FRO_COLS + threadIdx.x;
       ok[u] = t < tasks && jj[u] < n;
 #pragma unroll
-      for (int c = 0; c < 4; c++) x[u][c] = ok[u] ? A.p[c * A.ps + ii[u] * A.ld + jj[u]] : 0.0;
+      for (int c = 0; c < 4; c++) x[u][c] = ok[u] ? A.p[c * A.ps + off[u] * A.ld + jj[u]] : 0.0;
     }
 #pragma unroll
     for (int u = 0; u < FRO_U; u++) {
-      if (!ok[u]) continue;
 #pragma unroll
       for (int c = 0; c < 4; c++) {
         double v = x[u][c];
         bad += nonfinite_bits(v);
-        if (scale != 1.0) v *= scale;
-        if (c == 0 && ii[u] == jj[u] && diag != 0.0) v += diag;
-        if (hasB) v -= B.p[c * B.ps + ii[u] * B.ld + jj[u]];
+        if (HASB) v -= ok[u] ? B.p[c * B.ps + off[u] * B.ld + jj[u]] : 0.0;
         s = fma(v, v, s);
       }
     }
   }
   const double t0 = block_sum(s, sh);
-  const double t1 = block_sum((double)bad, sh);
+  const double t1 = block_count(bad, sh);
   if (threadIdx.x == 0) {
-    partials[2 * blockIdx.x] = t0;
-    partials[2 * blockIdx.x + 1] = t1;
+    r.partials[2 * blockIdx.x] = t0;
+    r.partials[2 * blockIdx.x + 1] = t1;
   }
+  reduce_last_block<2>(r, gridDim.x, sh);
 }
 
-// sum over (i, j) of |conj(M_ji) - M_ij|^2 for square M: ||M^H - M||_F^2.
-__global__ void __launch_bounds__(256) k_antiherm(Planes<const double> M, int n, double* partials) {
+// The Penrose pass's sums over a residual plane set (see launch_penrose_norms)
+// in one read: a block takes the tile pair (I, J), (J, I), I <= J, so that the
+// anti-Hermitian part |conj(R_ji) - R_ij|^2 is formed once per pair and counted
+// twice (diagonal tiles once).  Replaces three passes per residual (its norm,
+// the norm of +-R + I, which differs on the diagonal's s plane only, and the
+// anti-Hermitian part) at 2 FP64 operations per value instead of 7.
+__global__ void __launch_bounds__(256) k_penrose_norms(Planes<const double> R, int n, int neg, Reduce r) {
   __shared__ double t[4][TILE][TILE + 1];
-  __shared__ double sh[8];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int r0 = blockIdx.y * TILE, c0 = blockIdx.x * TILE;
-  // load the mirrored tile M[c0.., r0..] transposed into shared memory
+  __shared__ double sh[256];
+  // blockIdx.x = J (J + 1) / 2 + I
+  int J = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+  while ((long)J * (J + 1) / 2 > blockIdx.x) J--;
+  while ((long)(J + 1) * (J + 2) / 2 <= blockIdx.x) J++;
+  const int I = (int)(blockIdx.x - (long)J * (J + 1) / 2);
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, r0 = I * TILE, c0 = J * TILE;
+  double s = 0.0, sd = 0.0, s1 = 0.0, ah = 0.0;
+  // the mirrored tile R[c0.., r0..], transposed into shared memory
   for (int q = 0; q < TILE / TROWS; q++) {
     const int i = c0 + ty + q * TROWS, j = r0 + tx;
-    for (int c = 0; c < 4; c++)
-      t[c][tx][ty + q * TROWS] = (i < n && j < n) ? M.p[c * M.ps + (long)i * M.ld + j] : 0.0;
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const double v = (i < n && j < n) ? R.p[c * R.ps + (long)i * R.ld + j] : 0.0;
+      t[c][tx][ty + q * TROWS] = v;
+      if (I != J) s = fma(v, v, s);
+    }
   }
   __syncthreads();
-  double s = 0.0;
   for (int q = 0; q < TILE / TROWS; q++) {
     const int i = r0 + ty + q * TROWS, j = c0 + tx;
-    if (i < n && j < n) {
-      for (int c = 0; c < 4; c++) {
-        const double mij = M.p[c * M.ps + (long)i * M.ld + j];
-        const double mji = t[c][ty + q * TROWS][tx];  // M[j][i]
-        const double d = (c == 0 ? mji : -mji) - mij;
-        s += d * d;
+    if (i >= n || j >= n) continue;
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const double v = R.p[c * R.ps + (long)i * R.ld + j], w = t[c][ty + q * TROWS][tx];  // R_ij, R_ji
+      const double d = c == 0 ? w - v : w + v;
+      ah = fma(d, d, ah);
+      if (c == 0 && i == j) {
+        sd = fma(v, v, sd);
+        const double x = (neg ? flip_sign(v) : v) + 1.0;
+        s1 = fma(x, x, s1);
+      } else {
+        s = fma(v, v, s);
       }
     }
   }
-  const double tot = block_sum(s, sh);
-  if (threadIdx.x == 0) partials[(long)blockIdx.y * gridDim.x + blockIdx.x] = tot;
+  const double b0 = block_sum(s, sh), b1 = block_sum(sd, sh), b2 = block_sum(s1, sh), b3 = block_sum(ah, sh);
+  if (threadIdx.x == 0) {
+    double* p = r.partials + 4 * (long)blockIdx.x;
+    p[0] = b0;
+    p[1] = b1;
+    p[2] = b2;
+    p[3] = I == J ? b3 : 2.0 * b3;
+  }
+  reduce_last_block<4>(r, gridDim.x, sh);
 }
 
 // X (n x m) = alpha * A^H, A m x n: X[j][i] = alpha * conj(A[i][j]).
@@ -799,7 +751,7 @@ __global__ void k_f32_to_f64(Planes<const float> S, int rows, int cols, Planes<d
   const long total = (long)rows * cols;
   for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
     const long i = t / cols, j = t % cols;
-    for (int c = 0; c < 4; c++) D.p[c * D.ps + i * D.ld + j] = (double)S.p[c * S.ps + i * S.ld + j];
+    for (int c = 0; c < 4; c++) D.p[c * D.ps + i * D.ld + j] = widen(S.p[c * S.ps + i * S.ld + j]);
   }
 }
 
@@ -807,7 +759,7 @@ __global__ void k_f64_to_f32(Planes<const double> S, int rows, int cols, Planes<
   const long total = (long)rows * cols;
   for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
     const long i = t / cols, j = t % cols;
-    for (int c = 0; c < 4; c++) D.p[c * D.ps + i * D.ld + j] = (float)S.p[c * S.ps + i * S.ld + j];
+    for (int c = 0; c < 4; c++) D.p[c * D.ps + i * D.ld + j] = narrow(S.p[c * S.ps + i * S.ld + j]);
   }
 }
 
@@ -821,32 +773,20 @@ int grid_for(long total) {
 }  // namespace
 
 int combine_blocks(const CombineArgs& a) {
-  const int cw = combine_pairs_ok(a) ? 2 * TILE : TILE;
-  return ((a.cols + cw - 1) / cw) * ((a.rows + TILE - 1) / TILE);
+  const int rows = TROWS * combine_groups(a);
+  return ((a.cols + 2 * TILE - 1) / (2 * TILE)) * ((a.rows + rows - 1) / rows);
 }
 
-cudaError_t launch_combine(const CombineArgs& a, cudaStream_t st, int* blocks_out) {
-  const bool pairs = combine_pairs_ok(a);
-  const int cw = pairs ? 2 * TILE : TILE;
-  dim3 grid((a.cols + cw - 1) / cw, (a.rows + TILE - 1) / TILE);
-  if (blocks_out) *blocks_out = grid.x * grid.y;
+cudaError_t launch_combine(const CombineArgs& args, cudaStream_t st) {
+  CombineArgs a = args;
+  for (int o = 0; o < a.nout; o++) a.out[o].set_coefs();
   if (a.rows <= 0 || a.cols <= 0) return cudaSuccess;
-  if (pairs) {
-    k_combine_f2<<<grid, TILE * TROWS, 0, st>>>(a);
-    ++g_kernel_launches;
-    return cudaGetLastError();
-  }
+  const int groups = combine_groups(a), rows = TROWS * groups;
+  dim3 grid((a.cols + 2 * TILE - 1) / (2 * TILE), (a.rows + rows - 1) / rows);
   if (a.f64)
-    k_combine<double><<<grid, TILE * TROWS, 0, st>>>(a);
+    k_combine<double><<<grid, 256, 0, st>>>(a, groups);
   else
-    k_combine<float><<<grid, TILE * TROWS, 0, st>>>(a);
-  ++g_kernel_launches;
-  return cudaGetLastError();
-}
-
-cudaError_t launch_reduce_partials(const double* partials, int nblocks, int nvals, double* out,
-                                   cudaStream_t st) {
-  k_reduce_partials<<<1, 256, 0, st>>>(partials, nblocks, nvals, out);
+    k_combine<float><<<grid, 256, 0, st>>>(a, groups);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
@@ -870,23 +810,24 @@ cudaError_t launch_max(const double* v, int n, double* out, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_fro2_partials(const Planes<const double>& A, const Planes<const double>* B, int m, int n,
-                                 double* partials, cudaStream_t st, int* blocks_out, double scale, double diag) {
+cudaError_t launch_fro2(const Planes<const double>& A, const Planes<const double>* B, int m, int n, const Reduce& r,
+                        cudaStream_t st) {
   const long tasks = (long)m * ((n + FRO_COLS - 1) / FRO_COLS);
-  int blocks = (int)(tasks < 1024 ? tasks : 1024);
-  if (blocks < 1) blocks = 1;
-  *blocks_out = blocks;
-  Planes<const double> Bz = B ? *B : Planes<const double>();
-  k_fro2<<<blocks, FRO_COLS, 0, st>>>(A, Bz, B ? 1 : 0, m, n, scale, diag, partials);
+  const int blocks = (int)std::max(1L, std::min<long>(tasks, kFroBlocks));
+  if (B)
+    k_fro2<true><<<blocks, FRO_COLS, 0, st>>>(A, *B, m, n, r);
+  else
+    k_fro2<false><<<blocks, FRO_COLS, 0, st>>>(A, A, m, n, r);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
 
-cudaError_t launch_antiherm_partials(const Planes<const double>& M, int n, double* partials, cudaStream_t st,
-                                     int* blocks_out) {
-  dim3 grid((n + TILE - 1) / TILE, (n + TILE - 1) / TILE);
-  *blocks_out = grid.x * grid.y;
-  k_antiherm<<<grid, TILE * TROWS, 0, st>>>(M, n, partials);
+int penrose_norm_blocks(int n) {
+  const int t = (n + TILE - 1) / TILE;
+  return t * (t + 1) / 2;
+}
+cudaError_t launch_penrose_norms(const Planes<const double>& R, int n, double sr, const Reduce& r, cudaStream_t st) {
+  k_penrose_norms<<<penrose_norm_blocks(n), TILE * TROWS, 0, st>>>(R, n, sr < 0 ? 1 : 0, r);
   ++g_kernel_launches;
   return cudaGetLastError();
 }

@@ -413,7 +413,9 @@ EmuPlan emu_plan(int M, int N, int K, int S) {
         }
         const double items = 8.0 * tiles * ng * nk;
         double t = ng == 1 ? std::ceil(items / nsm) * cmax : std::max(cmax, sum / nsm + 0.5 * cmin);
-        // 64 bytes written and read per entry and part at about 5 TB/s
+        // each further part: 64 bytes written and read per entry at about 5 TB/s,
+        // and one more dependent load in the combine pass
+        t += 3.0 * (ng * nk - 1);
         t += 128.0 * M * (double)N * ng * nk / 5e12 / (256 / 1.9e9);
         if (t < best * 0.97) {
           best = t;

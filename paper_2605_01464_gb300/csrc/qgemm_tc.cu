@@ -86,33 +86,6 @@ struct KParams {
 
 __device__ __forceinline__ bool al16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-// FP32 <-> FP64 conversions from the bits: GB300's FP64 pipe, which the
-// conversion instructions use, does two operations per clock and SM, the
-// integer pipe 64.  Zeros, subnormals, infinities and NaN take the
-// instruction.
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t b = __float_as_uint(x);
-  if (((b >> 23) & 0xFFu) - 1u >= 254u) return (double)x;
-  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
-}
-__device__ __forceinline__ float narrow(double x) {  // round to nearest even, as the cast
-  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-  const uint32_t ex = (hi >> 20) & 0x7FFu;
-  if (ex - 897u >= 253u) return (float)x;  // below the FP32 normal range, or near overflow
-  const uint32_t m = ((ex - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
-  const uint32_t rem = lo & 0x1FFFFFFFu;
-  const uint32_t up = (rem > 0x10000000u || (rem == 0x10000000u && (m & 1u))) ? 1u : 0u;
-  return __uint_as_float((hi & 0x80000000u) | (m + up));
-}
-template <typename T>
-__device__ __forceinline__ T to_master(float x);
-template <>
-__device__ __forceinline__ float to_master<float>(float x) { return x; }
-template <>
-__device__ __forceinline__ double to_master<double>(float x) { return widen(x); }
-__device__ __forceinline__ float to_float(float x) { return x; }
-__device__ __forceinline__ float to_float(double x) { return narrow(x); }
-
 // Two adjacent entries (x, y) of a row; `two`: y is inside the matrix.
 __device__ __forceinline__ void load2(const float* p, bool two, float* u) {
   if (two && (reinterpret_cast<uintptr_t>(p) & 7) == 0) {
@@ -189,28 +162,28 @@ __device__ __forceinline__ void epi_piece(const EpiArgs& E, int c, int r0, int M
   for (int o = 0; o < E.nout; o++) {
     const EpiOut& O = E.out[o];
     T w[8];
-    const T cacc = (T)O.cacc;
+    const int ck = O.cacc.kind;
 #pragma unroll
     for (int t = 0; t < 8; t++)  // +-1 as a sign flip (the combine kernel's arithmetic)
-      w[t] = cacc == (T)0 ? (T)0 : to_master<T>(cacc == (T)-1 ? -v[t] : v[t]);
-    if (cacc != (T)0 && cacc != (T)1 && cacc != (T)-1) {
+      w[t] = ck == CK_ZERO ? (T)0 : to_master<T>(ck == CK_MINUS ? -v[t] : v[t]);
+    if (ck == CK_GENERAL) {
 #pragma unroll
-      for (int t = 0; t < 8; t++) w[t] *= cacc;
+      for (int t = 0; t < 8; t++) w[t] *= coef<T>(O.cacc);
     }
 #pragma unroll
     for (int a = 0; a < kEpiAux; a++) {
-      if (!E.aux[a] || O.caux[a] == 0.0) continue;
-      const T ca = (T)O.caux[a];
+      if (!E.aux[a] || O.caux[a].kind == CK_ZERO) continue;
+      const T ca = coef<T>(O.caux[a]);
       if (!PRE) load_aux(a, u[0]);
 #pragma unroll
       for (int t = 0; t < 8; t++) w[t] += ca * u[PRE ? a : 0][t];
     }
-    if (c == 0 && O.diag != 0.0) {
+    if (c == 0 && O.diag.kind != CK_ZERO && r0 < j0 + 16 && j0 < r0 + 16) {
 #pragma unroll
       for (int t = 0; t < 8; t++)
-        if (i0 + 8 * ((t >> 1) & 1) == jc + 8 * (t >> 2) + (t & 1)) w[t] += (T)O.diag;
+        if (i0 + 8 * ((t >> 1) & 1) == jc + 8 * (t >> 2) + (t & 1)) w[t] += coef<T>(O.diag);
     }
-    if (PRE && o == 0 && E.partials) {
+    if (PRE && o == 0 && E.red.partials) {
 #pragma unroll
       for (int t = 0; t < 8; t++)
         if (i0 + 8 * ((t >> 1) & 1) < M && jc + 8 * (t >> 2) + (t & 1) < N) {
@@ -292,6 +265,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   __shared__ uint64_t bar_full[STAGES], bar_empty[STAGES], bar_acc_full[NBUF], bar_acc_empty[NBUF];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
+  __shared__ double red_sh[32];
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -459,7 +433,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[b]));
     }
-    if (P.E.partials) {
+    if (P.E.red.partials) {
       double d0 = sdx, d1 = sx, d2 = bad;
       for (int o = 16; o > 0; o >>= 1) {
         d0 += __shfl_xor_sync(0xffffffffu, d0, o);
@@ -467,7 +441,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         d2 += __shfl_xor_sync(0xffffffffu, d2, o);
       }
       if (lane == 0) {
-        double* pp = P.E.partials + 3 * ((long)blockIdx.x * EPI_WARPS + e);
+        double* pp = P.E.red.partials + 3 * ((long)blockIdx.x * EPI_WARPS + e);
         pp[0] = d0;
         pp[1] = d1;
         pp[2] = d2;
@@ -477,6 +451,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 
   fence_before();
   __syncthreads();
+  if (P.E.red.partials) reduce_last_block<3>(P.E.red, (long)gridDim.x * EPI_WARPS, red_sh);
   if (warp == 0 && lane == 0 && abort_flag) {
     for (int u = (issued > STAGES ? issued - STAGES : 0); u < issued; u++)
       (void)mbar_wait(smem_u32(&bar_full[u % STAGES]), (u / STAGES) & 1, &abort_flag, nullptr, 0);
@@ -588,7 +563,7 @@ cudaError_t launch_qgemm_tc(const TcGemmArgs& a, cudaStream_t st) {
   }
   P.C = a.C;
   P.E = a.epi;
-  if (P.E.nout < 0 || P.E.nout > kMaxOut || (P.E.f64 && P.E.partials)) return cudaErrorInvalidValue;
+  if (P.E.nout < 0 || P.E.nout > kMaxOut || (P.E.f64 && P.E.red.partials)) return cudaErrorInvalidValue;
   P.err = a.err;
   switch (tc_shape(a.broad, P.E.nout > 0, a.M, a.N, units_of(a))) {
     case SHAPE_FULL: return launch_cfg<Cfg<128, 4>>(a, P, st);

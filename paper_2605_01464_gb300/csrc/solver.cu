@@ -83,6 +83,7 @@ struct qpinv_ctx {
   std::vector<EvRec> pending;
   std::vector<cudaEvent_t> pool;
   int* d_err = nullptr;
+  unsigned int* d_count = nullptr;  // block counter of the kernels that finish their own sums (0 between launches)
   double* h_pin = nullptr;  // pinned host scalars
   cudaStream_t st = nullptr;
   bool trace = false;
@@ -303,8 +304,6 @@ struct Solver {
   long long gemms = 0;
   QMat A, X[2];
   int cur = 0;
-  double* partials = nullptr;
-  int partial_cap = 0;
 
   // ---------------- products ----------------
   struct Acc {
@@ -373,6 +372,15 @@ struct Solver {
     return g;
   }
 
+  // Sums of `blocks` blocks' partials into the "red" buffer from `slot` on.
+  Reduce reduce_to(int blocks, int nvals, int slot) {
+    Reduce r;
+    r.partials = (double*)buf(c, "partials", sizeof(double) * nvals * (size_t)blocks + 64);
+    r.out = (double*)buf(c, "red", sizeof(double) * 8) + slot;
+    r.count = c->d_count;
+    return r;
+  }
+
   static void set_acc(CombineArgs& a, const Acc& acc) {
     a.acc = acc.p;
     a.acc_kind = acc.kind;
@@ -426,9 +434,9 @@ struct Solver {
         d.ldb = O.s16.ldb;
         d.psb = O.s16.psb;
         d.levels = O.s16.levels;
-        d.cacc = O.cacc;
-        for (int t = 0; t < kEpiAux; t++) d.caux[t] = O.caux[t];
-        d.diag = O.diag;
+        d.cacc.set(O.cacc);
+        for (int t = 0; t < kEpiAux; t++) d.caux[t].set(O.caux[t]);
+        d.diag.set(O.diag);
       }
       e.f64 = a.f64;
       for (int t = 0; t < kEpiAux; t++) {
@@ -437,20 +445,9 @@ struct Solver {
         e.ps_aux[t] = a.ps_aux[t];
       }
       const int blocks = tc_partial_blocks(g);
-      if (with_partials) {
-        if (blocks > partial_cap) {
-          partials = (double*)buf(c, "partials", sizeof(double) * 3 * (size_t)blocks + 64);
-          partial_cap = blocks;
-        }
-        e.partials = partials;
-      }
+      if (with_partials) e.red = reduce_to(blocks, 3, red_slot);
       timed(c, EV_TC, flops, flops * g.npairs, 0, [&] { return launch_qgemm_tc(g, c->st); });
       c->stats.fused_epilogues++;
-      if (with_partials) {
-        double* red = (double*)buf(c, "red", sizeof(double) * 8);
-        timed(c, EV_EW, 0, 0, 24.0 * blocks,
-              [&] { return launch_reduce_partials(partials, blocks, 3, red + red_slot, c->st); });
-      }
       return;
     }
     Acc acc = prod(P, Q, mode);
@@ -593,14 +590,7 @@ struct Solver {
   // with_partials: block partials of ||out - aux0||^2, ||out||^2 and the
   // non-finite count, reduced into red_slot[0..2] of the "red" buffer.
   void run(CombineArgs& a, bool with_partials = false, int red_slot = 0) {
-    const int blocks = combine_blocks(a);
-    if (with_partials) {
-      if (blocks > partial_cap) {
-        partials = (double*)buf(c, "partials", sizeof(double) * 3 * (size_t)blocks + 64);
-        partial_cap = blocks;
-      }
-      a.partials = partials;
-    }
+    if (with_partials) a.red = reduce_to(combine_blocks(a), 3, red_slot);
     double bytes = 0;
     const double el = (double)a.rows * a.cols * 4, ms = dbl ? 8 : 4;
     if (a.acc) bytes += el * (a.acc_kind == ACC_F32 ? 4 : a.acc_kind == ACC_F64 ? 8 : 16 * a.acc_sets);
@@ -611,12 +601,7 @@ struct Solver {
       if (a.out[o].s16.a) bytes += el * 2 * a.out[o].s16.levels;
       if (a.out[o].s16.b) bytes += el * 2 * a.out[o].s16.levels;
     }
-    timed(c, EV_EW, 0, 0, bytes, [&] { return launch_combine(a, c->st, nullptr); });
-    if (with_partials) {
-      double* red = (double*)buf(c, "red", sizeof(double) * 8);
-      timed(c, EV_EW, 0, 0, 24.0 * blocks,
-            [&] { return launch_reduce_partials(partials, blocks, 3, red + red_slot, c->st); });
-    }
+    timed(c, EV_EW, 0, 0, bytes, [&] { return launch_combine(a, c->st); });
   }
 
   // ---------------- shape helpers ----------------
@@ -944,31 +929,29 @@ void store_planes(qpinv_ctx* c, const QMat& src, double* const dst[4], long ld, 
   }
 }
 
-// ||scale P + diag I - Q||_F^2 (Q optional; diag on plane s).
-double fro2(qpinv_ctx* c, const Planes<const double>& P, const Planes<const double>* Q, int rows, int cols,
-            double* bad = nullptr, double scale = 1.0, double diag = 0.0) {
-  int blocks = 0;
-  double* part = (double*)buf(c, "fro_part", sizeof(double) * 2 * 1024 + 64);
-  double* red = (double*)buf(c, "fro_red", sizeof(double) * 4);
+// ||P - Q||_F^2 (Q optional) and P's non-finite count into two device doubles.
+void fro2_to(qpinv_ctx* c, const Planes<const double>& P, const Planes<const double>* Q, int rows, int cols,
+             double* dst) {
+  const Reduce r{(double*)buf(c, "fro_part", sizeof(double) * 2 * kFroBlocks + 64), dst, c->d_count};
   timed(c, EV_EW, 0, 0, (double)rows * cols * 32 * (Q ? 2 : 1),
-        [&] { return launch_fro2_partials(P, Q, rows, cols, part, c->st, &blocks, scale, diag); });
-  timed(c, EV_EW, 0, 0, 16.0 * blocks, [&] { return launch_reduce_partials(part, blocks, 2, red, c->st); });
+        [&] { return launch_fro2(P, Q, rows, cols, r, c->st); });
+}
+double fro2(qpinv_ctx* c, const Planes<const double>& P, const Planes<const double>* Q, int rows, int cols,
+            double* bad = nullptr) {
+  double* red = (double*)buf(c, "fro_red", sizeof(double) * 16);
+  fro2_to(c, P, Q, rows, cols, red);
   double h[2];
   read_back(c, red, 2, h);
   if (bad) *bad = h[1];
   return h[0];
 }
 
-double antiherm2(qpinv_ctx* c, const QMat& M) {
-  int blocks = ((M.rows + 31) / 32) * ((M.rows + 31) / 32);
-  double* part = (double*)buf(c, "ah_part", sizeof(double) * (size_t)blocks + 64);
-  double* red = (double*)buf(c, "fro_red", sizeof(double) * 4);
-  timed(c, EV_EW, 0, 0, (double)M.rows * M.rows * 64,
-        [&] { return launch_antiherm_partials(dview(M), M.rows, part, c->st, &blocks); });
-  timed(c, EV_EW, 0, 0, 8.0 * blocks, [&] { return launch_reduce_partials(part, blocks, 1, red, c->st); });
-  double h;
-  read_back(c, red, 1, &h);
-  return h;
+// The four sums of launch_penrose_norms into dst.
+void penrose_norms_to(qpinv_ctx* c, const QMat& R, double sr, double* dst) {
+  const Reduce r{(double*)buf(c, "ah_part", sizeof(double) * 4 * (size_t)penrose_norm_blocks(R.rows) + 64), dst,
+                 c->d_count};
+  timed(c, EV_EW, 0, 0, (double)R.rows * R.rows * 32,
+        [&] { return launch_penrose_norms(dview(R), R.rows, sr, r, c->st); });
 }
 
 // Penrose residuals (Sec. 4) for A (m x n) and X (n x m) FP64 masters, with
@@ -1010,34 +993,37 @@ void penrose(qpinv_ctx* c, const QMat& A, const QMat& X, int mode, double* E, do
     product(X, A, Rl, 8, -1.0);
   }
   Planes<const double> a = dview(A), x = dview(X);
-  const double fa = std::sqrt(fro2(c, a, nullptr, m, n)), fx = std::sqrt(fro2(c, x, nullptr, n, m));
-  // ||R Q||_F with R = AX - I or XA - I.  When R is small (square
+  // the norms of A, X and both residuals: one host read
+  double* red = (double*)buf(c, "fro_red", sizeof(double) * 16);
+  fro2_to(c, a, nullptr, m, n, red);
+  fro2_to(c, x, nullptr, n, m, red + 2);
+  penrose_norms_to(c, Rr, sr, red + 4);
+  penrose_norms_to(c, Rl, sl, red + 8);
+  double h[12];
+  read_back(c, red, 12, h);
+  const double fa = std::sqrt(h[0]), fx = std::sqrt(h[2]);
+  // ||R Q||_F with R = AX - I or XA - I (norm fr).  When R is small (square
   // full-rank A) the product needs only a few digits relative to ||R|| ||Q||:
   // 6 slices are accepted when the result exceeds 1e3 times a bound on their
   // truncation error, 2^(10 - 7S) K ||R||_F ||Q||_F; otherwise 8 slices.
-  auto outer = [&](const QMat& R, const QMat& Q, QMat& Out, double fq) {
+  auto outer = [&](const QMat& R, const QMat& Q, QMat& Out, double fr, double fq) {
     const int rows = R.rows, cols = Q.cols, K = R.cols;
-    if (mode == PM_EMU) {
-      const double fr = std::sqrt(fro2(c, dview(R), nullptr, R.rows, R.cols));
-      if (fr <= 1e-3) {
-        product(R, Q, Out, 6, 0.0);
-        const double e = std::sqrt(fro2(c, dview(Out), nullptr, rows, cols));
-        if (e >= 1e3 * std::ldexp(1.0, 10 - 7 * 6) * K * fr * fq) return e;
-      }
+    if (mode == PM_EMU && fr <= 1e-3) {
+      product(R, Q, Out, 6, 0.0);
+      const double e = std::sqrt(fro2(c, dview(Out), nullptr, rows, cols));
+      if (e >= 1e3 * std::ldexp(1.0, 10 - 7 * 6) * K * fr * fq) return e;
     }
     product(R, Q, Out, 8, 0.0);
     return std::sqrt(fro2(c, dview(Out), nullptr, rows, cols));
   };
-  E[0] = outer(Rr, A, E1m, fa);
-  E[1] = outer(Rl, X, E2m, fx);
+  E[0] = outer(Rr, A, E1m, std::sqrt(h[4] + h[5]), fa);
+  E[1] = outer(Rl, X, E2m, std::sqrt(h[8] + h[9]), fx);
   if (gemms) *gemms += S.gemms;
-  E[2] = std::sqrt(antiherm2(c, Rr));
-  E[3] = std::sqrt(antiherm2(c, Rl));
-  // ||AX||_F^2 = ||Rr||^2 + 2 Re tr(Rr) + m: computed directly from
-  // AX = sr Rr + I instead (each element formed in registers, as a combine
-  // pass would store it), and XA = sl Rl + I likewise
-  const double nr[4] = {fa, fx, std::sqrt(fro2(c, dview(Rr), nullptr, m, m, nullptr, sr, 1.0)),
-                        std::sqrt(fro2(c, dview(Rl), nullptr, n, n, nullptr, sl, 1.0))};
+  E[2] = std::sqrt(h[7]);
+  E[3] = std::sqrt(h[11]);
+  // AX = sr Rr + I differs from sr Rr on the diagonal's s plane only (its own
+  // sum, so no cancellation), and XA = sl Rl + I likewise
+  const double nr[4] = {fa, fx, std::sqrt(h[4] + h[6]), std::sqrt(h[8] + h[10])};
   for (int t = 0; t < 4; t++) Er[t] = nr[t] > 0 ? E[t] / nr[t] : E[t];
 }
 
@@ -1144,12 +1130,13 @@ int qpinv_init(qpinv_ctx** out, int device, const qpinv_options* opt) {
   const char* tr = getenv("QPINV_TRACE");
   c->trace = tr && tr[0] == '1';
   DeviceGuard g(device);
-  if (cudaMalloc(&c->d_err, sizeof(int)) != cudaSuccess || cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess ||
+  if (cudaMalloc(&c->d_err, 256) != cudaSuccess || cudaMemset(c->d_err, 0, 256) != cudaSuccess ||
       cudaMallocHost(&c->h_pin, sizeof(double) * 64) != cudaSuccess) {
     cudaGetLastError();
     qpinv_free(c);
     return QPINV_E_NOMEM;
   }
+  c->d_count = (unsigned int*)c->d_err + 32;
   init_constants();
   *out = c;
   return QPINV_OK;
