@@ -207,6 +207,9 @@ cudaError_t launch_init_x0(const Planes<const double>& A, int m, int n, double a
                            cudaStream_t st);
 // Column exponents e (|v| < 2^e over the four planes); `scratch`: COL_SCRATCH(cols) ints
 cudaError_t launch_maxexp(const Planes<const float>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st);
+// D = S (FP64 planes, any strides)
+cudaError_t launch_copy_planes(const Planes<const double>& S, int rows, int cols, const Planes<double>& D,
+                               cudaStream_t st);
 cudaError_t launch_f64_to_f32(const Planes<const double>& src, int rows, int cols, const Planes<float>& dst,
                               cudaStream_t st);
 cudaError_t launch_maxexp(const Planes<const double>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st);

@@ -763,6 +763,19 @@ __global__ void k_f64_to_f32(Planes<const double> S, int rows, int cols, Planes<
   }
 }
 
+// D = S, four planes: a block takes 512 columns of a row (two per thread).
+__global__ void __launch_bounds__(256) k_copy_planes(Planes<const double> S, int rows, int cols, Planes<double> D) {
+  const int j = (blockIdx.x * 256 + threadIdx.x) * 2;
+  if (j >= cols) return;
+  for (int i = blockIdx.y; i < rows; i += gridDim.y) {
+    double u[4][2];
+#pragma unroll
+    for (int c = 0; c < 4; c++) ld2(S.p + c * S.ps + (long)i * S.ld + j, j + 1 < cols, u[c][0], u[c][1]);
+#pragma unroll
+    for (int c = 0; c < 4; c++) st2(D.p + c * D.ps + (long)i * D.ld + j, j + 1 < cols, u[c][0], u[c][1]);
+  }
+}
+
 int grid_for(long total) {
   long blocks = (total + 255) / 256;
   if (blocks > 4096) blocks = 4096;
@@ -854,6 +867,14 @@ cudaError_t launch_maxexp(const Planes<const double>& A, int rows, int cols, int
 }
 cudaError_t launch_maxexp(const Planes<const float>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st) {
   return maxexp_t<float>(A, rows, cols, e, scratch, st);
+}
+
+cudaError_t launch_copy_planes(const Planes<const double>& S, int rows, int cols, const Planes<double>& D,
+                               cudaStream_t st) {
+  if (rows <= 0 || cols <= 0) return cudaSuccess;
+  k_copy_planes<<<dim3((cols + 511) / 512, std::min(rows, 8192)), 256, 0, st>>>(S, rows, cols, D);
+  ++g_kernel_launches;
+  return cudaGetLastError();
 }
 
 cudaError_t launch_f32_to_f64(const Planes<const float>& src, int rows, int cols, const Planes<double>& dst,

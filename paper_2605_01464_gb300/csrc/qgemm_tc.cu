@@ -483,19 +483,19 @@ long shape_items(int sh, int M, int N) {
 // 64-column one, -1 by the time of the busiest SM): a stage costs its MMAs or
 // its operand bytes, whichever is longer (cycles per stage below), an item
 // its stages, and the last item of an SM its epilogue (every item of the
-// four-component shape, which has one accumulator; fused products do not take
-// it).  Measured where the line lies: 500 x 1000 x 500, 2 terms, 0.059 ms with
+// four-component shape, which has one accumulator).  Measured where the line lies: 500 x 1000 x 500, 2 terms, 0.059 ms with
 // 64 columns against 0.125 with 128; 1000^3, 3 terms, 0.143 (component pair)
 // against 0.240 (four components) and 0.41 (64 columns); 2048^3 0.173 (four
 // components) against 0.204 and 0.453.
-TcShape tc_shape(int broad, bool fused, int M, int N, int units) {
+TcShape tc_shape(int broad, bool fused, bool f64, int M, int N, int units) {
   if (broad == 0) return SHAPE_64;
   if (broad == 1) return fused ? SHAPE_PAIR : SHAPE_FULL;
-  const double stage[4] = {1950, 1100, 600, 450}, tail[4] = {12000, 12000, 5000, 4000};
+  const double stage[4] = {1950, 1100, 600, 450};
+  const double tail[4] = {!fused ? 12000. : f64 ? 40000. : 30000., f64 ? 24000. : 12000., 5000, 4000};
   const int nsm = std::max(1, sm_count());
   int best = SHAPE_PAIR;
   double tb = 1e300;
-  for (int sh = fused ? SHAPE_PAIR : SHAPE_FULL; sh <= SHAPE_32; sh++) {
+  for (int sh = SHAPE_FULL; sh <= SHAPE_32; sh++) {
     const double waves = (double)((shape_items(sh, M, N) + nsm - 1) / nsm);
     const double t = waves * units * stage[sh] + tail[sh] * (sh == SHAPE_FULL ? waves : 1.0) +
                      (waves - 1) * 1000.0;
@@ -530,16 +530,17 @@ int units_of(const TcGemmArgs& a) { return ((a.k1 + BK - 1) / BK - a.k0 / BK) * 
 }  // namespace
 
 int tc_partial_blocks(const TcGemmArgs& a) {
-  const TcShape sh = tc_shape(a.broad, true, a.M, a.N, units_of(a));
+  const TcShape sh = tc_shape(a.broad, true, a.epi.f64 != 0, a.M, a.N, units_of(a));
   return (int)std::min<long>(shape_items(sh, a.M, a.N), std::max(1, sm_count())) * EPI_WARPS;
 }
 
-bool tc_supported() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return false;
-  cudaDeviceProp p;
-  if (cudaGetDeviceProperties(&p, dev) != cudaSuccess) return false;
-  return p.major == 10 && p.minor == 3 && get_encode() != nullptr;
+bool tc_supported() {  // sm_103; attributes only (cudaGetDeviceProperties takes tens of microseconds)
+  int dev = 0, major = 0, minor = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess)
+    return false;
+  return major == 10 && minor == 3 && get_encode() != nullptr;
 }
 
 cudaError_t launch_qgemm_tc(const TcGemmArgs& a, cudaStream_t st) {
@@ -565,7 +566,7 @@ cudaError_t launch_qgemm_tc(const TcGemmArgs& a, cudaStream_t st) {
   P.E = a.epi;
   if (P.E.nout < 0 || P.E.nout > kMaxOut || (P.E.f64 && P.E.red.partials)) return cudaErrorInvalidValue;
   P.err = a.err;
-  switch (tc_shape(a.broad, P.E.nout > 0, a.M, a.N, units_of(a))) {
+  switch (tc_shape(a.broad, P.E.nout > 0, P.E.f64 != 0, a.M, a.N, units_of(a))) {
     case SHAPE_FULL: return launch_cfg<Cfg<128, 4>>(a, P, st);
     case SHAPE_PAIR: return launch_cfg<Cfg<128, 2>>(a, P, st);
     case SHAPE_64: return launch_cfg<Cfg<64, 1>>(a, P, st);

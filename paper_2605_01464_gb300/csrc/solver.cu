@@ -74,6 +74,12 @@ long rup64(long x) { return (x + 63) / 64 * 64; }
 
 }  // namespace
 
+// The context's 256-byte device status block: the kernels' error word, the
+// block counter of the kernels that finish their own sums (0 between
+// launches), and the sums the host reads every iteration.
+constexpr size_t kStatusCount = 64, kStatusSums = 128;
+constexpr int kRedSums = 16;
+
 struct qpinv_ctx {
   int device = 0;
   qpinv_options opt;
@@ -83,7 +89,8 @@ struct qpinv_ctx {
   std::vector<EvRec> pending;
   std::vector<cudaEvent_t> pool;
   int* d_err = nullptr;
-  unsigned int* d_count = nullptr;  // block counter of the kernels that finish their own sums (0 between launches)
+  unsigned int* d_count = nullptr;  // in the status block
+  double* d_red = nullptr;          // in the status block: kRedSums sums
   double* h_pin = nullptr;  // pinned host scalars
   cudaStream_t st = nullptr;
   bool trace = false;
@@ -261,13 +268,19 @@ void read_back(qpinv_ctx* c, const double* d, int n, double* h) {
   memcpy(h, c->h_pin, sizeof(double) * n);
 }
 
-void check_kernel_error(qpinv_ctx* c) {
-  int h = 0;
-  ck(c, cudaMemcpyAsync(&h, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st), "read error word");
+// Host read of the status block: the kernels' error word (throws if a bounded
+// wait expired) and, when h is given, the first n of its kRedSums sums -- one
+// copy and one synchronisation for both.
+void read_status(qpinv_ctx* c, int n = 0, double* h = nullptr) {
+  const size_t bytes = kStatusSums + sizeof(double) * n;
+  ck(c, cudaMemcpyAsync(c->h_pin, c->d_err, bytes, cudaMemcpyDeviceToHost, c->st), "read status");
   ck(c, cudaStreamSynchronize(c->st), "stream sync");
-  if (h != 0) {
+  int code = 0;
+  memcpy(&code, c->h_pin, sizeof(int));
+  if (n) memcpy(h, (const char*)c->h_pin + kStatusSums, sizeof(double) * n);
+  if (code != 0) {
     cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
-    throw QpError{QPINV_E_TIMEOUT, "tensor-core GEMM bounded wait expired (code " + std::to_string(h) + ")"};
+    throw QpError{QPINV_E_TIMEOUT, "tensor-core GEMM bounded wait expired (code " + std::to_string(code) + ")"};
   }
 }
 
@@ -372,11 +385,11 @@ struct Solver {
     return g;
   }
 
-  // Sums of `blocks` blocks' partials into the "red" buffer from `slot` on.
+  // Sums of `blocks` blocks' partials into the status block from sum `slot` on.
   Reduce reduce_to(int blocks, int nvals, int slot) {
     Reduce r;
     r.partials = (double*)buf(c, "partials", sizeof(double) * nvals * (size_t)blocks + 64);
-    r.out = (double*)buf(c, "red", sizeof(double) * 8) + slot;
+    r.out = c->d_red + slot;
     r.count = c->d_count;
     return r;
   }
@@ -588,7 +601,7 @@ struct Solver {
     return o;
   }
   // with_partials: block partials of ||out - aux0||^2, ||out||^2 and the
-  // non-finite count, reduced into red_slot[0..2] of the "red" buffer.
+  // non-finite count, reduced into the status block's sums from red_slot on.
   void run(CombineArgs& a, bool with_partials = false, int red_slot = 0) {
     if (with_partials) a.red = reduce_to(combine_blocks(a), 3, red_slot);
     double bytes = 0;
@@ -909,6 +922,36 @@ bool is_device_ptr(const void* p) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Four equally spaced planes in this device's memory, as one plane set: the
+// kernels then read (or write) the caller's matrix in place.  False for host
+// memory, another device's memory, and planes at irregular distances.
+bool direct_planes(qpinv_ctx* c, const double* const src[4], long ld, Planes<double>* P) {
+  for (int p = 0; p < 4; p++) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, src[p]) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (at.type == cudaMemoryTypeManaged) continue;
+    if (at.type != cudaMemoryTypeDevice || at.device != c->device) return false;
+  }
+  const intptr_t d = (intptr_t)src[1] - (intptr_t)src[0];
+  if (d % (intptr_t)sizeof(double) || (intptr_t)src[0] % (intptr_t)sizeof(double) ||
+      (intptr_t)src[2] - (intptr_t)src[1] != d || (intptr_t)src[3] - (intptr_t)src[2] != d)
+    return false;
+  P->p = const_cast<double*>(src[0]);
+  P->ld = ld;
+  P->ps = d / (intptr_t)sizeof(double);
+  return true;
+}
+// The byte range that a plane set touches.
+void planes_range(const Planes<double>& P, int rows, int cols, uintptr_t* lo, uintptr_t* hi) {
+  const double* a = P.p + (P.ps < 0 ? 3 * P.ps : 0);
+  const double* b = P.p + (P.ps > 0 ? 3 * P.ps : 0) + (long)(rows - 1) * P.ld + cols;
+  *lo = (uintptr_t)a;
+  *hi = (uintptr_t)b;
+}
+
 // Copies a caller matrix (device or host planes) into a workspace FP64 master.
 void load_planes(qpinv_ctx* c, const double* const src[4], long ld, int rows, int cols, const QMat& dst) {
   for (int p = 0; p < 4; p++) {
@@ -920,6 +963,13 @@ void load_planes(qpinv_ctx* c, const double* const src[4], long ld, int rows, in
   }
 }
 void store_planes(qpinv_ctx* c, const QMat& src, double* const dst[4], long ld, int rows, int cols) {
+  Planes<double> P;
+  if (direct_planes(c, dst, ld, &P)) {
+    if (P.p == src.d.p) return;  // written in place
+    // one launch for the four planes (cudaMemcpy2D moves them at about 1 TB/s)
+    timed(c, EV_EW, 0, 0, 64.0 * rows * cols, [&] { return launch_copy_planes(dview(src), rows, cols, P, c->st); });
+    return;
+  }
   for (int p = 0; p < 4; p++) {
     const bool dev = is_device_ptr(dst[p]);
     ck(c,
@@ -927,6 +977,16 @@ void store_planes(qpinv_ctx* c, const QMat& src, double* const dst[4], long ld, 
                          sizeof(double) * cols, rows, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->st),
        "copy out");
   }
+}
+// FP64 master of a caller matrix that a call only reads: its own planes where
+// the kernels can read them, else a workspace copy called `name`.
+Planes<double> input_planes(qpinv_ctx* c, const double* const src[4], long ld, int rows, int cols,
+                            const std::string& name) {
+  Planes<double> P;
+  if (direct_planes(c, src, ld, &P)) return P;
+  const QMat M = mat(c, name, rows, cols, MST_D, false, false);
+  load_planes(c, src, ld, rows, cols, M);
+  return M.d;
 }
 
 // ||P - Q||_F^2 (Q optional) and P's non-finite count into two device doubles.
@@ -1136,7 +1196,8 @@ int qpinv_init(qpinv_ctx** out, int device, const qpinv_options* opt) {
     qpinv_free(c);
     return QPINV_E_NOMEM;
   }
-  c->d_count = (unsigned int*)c->d_err + 32;
+  c->d_count = (unsigned int*)((char*)c->d_err + kStatusCount);
+  c->d_red = (double*)((char*)c->d_err + kStatusSums);
   init_constants();
   *out = c;
   return QPINV_OK;
@@ -1231,8 +1292,8 @@ int qpinv_solve(qpinv_ctx* c, void* stream, int m, int n, const double* const A[
     S.left = o.side == QPINV_SIDE_LEFT || (o.side == QPINV_SIDE_AUTO && m > n);
     S.s = S.left ? n : m;
     res.side = S.left ? QPINV_SIDE_LEFT : QPINV_SIDE_RIGHT;
-    S.A = mat(c, "A", m, n, MST_D | MST_F, !S.left, S.left);
-    load_planes(c, A, lda, m, n, S.A);
+    S.A = mat(c, "A", m, n, MST_F, !S.left, S.left);
+    S.A.d = input_planes(c, A, lda, m, n, "A");
     Planes<const double> a = dview(S.A);
     double bad = 0.0;
     const double a_f2 = fro2(c, a, nullptr, m, n, &bad);
@@ -1380,7 +1441,7 @@ int qpinv_solve(qpinv_ctx* c, void* stream, int m, int n, const double* const A[
         S.pre_R = S.residual(S.X[S.cur], "R", "fab", true);
         S.pre_res = true;
         double hr[8];
-        read_back(c, (const double*)buf(c, "red", sizeof(double) * 8), 6, hr);
+        read_status(c, 6, hr);
         const double rn = std::sqrt(hr[4]);
         const double floor_rel = 0x1p-53 * a2est * xnorm;
         if (c->trace) fprintf(stderr, "qpinv it %d polish residual |R|_F %.3e floor %.3e\n", j, rn, floor_rel);
@@ -1402,9 +1463,8 @@ int qpinv_solve(qpinv_ctx* c, void* stream, int m, int n, const double* const A[
         case QPINV_QHPIM: S.step_qhpim(o.hyper_order); break;
         default: S.step_qhpi19(hpi19_k); break;
       }
-      if (!fp64) check_kernel_error(c);
       double h[8];
-      read_back(c, (const double*)buf(c, "red", sizeof(double) * 8), 6, h);
+      read_status(c, 6, h);
       const double rnorm = std::sqrt(h[4]);  // ||R_j||_F of this step's residual
       const double d = std::sqrt(h[0]), nx = std::sqrt(h[1]);
       if (c->trace)
@@ -1516,7 +1576,7 @@ int qpinv_solve(qpinv_ctx* c, void* stream, int m, int n, const double* const A[
           // in R of this kind with coefficients at most 1 in modulus).
           S.residual(S.X[S.cur], "R", "fab", true);
           double hr[8];
-          read_back(c, (const double*)buf(c, "red", sizeof(double) * 8), 6, hr);
+          read_status(c, 6, hr);
           const double rn = std::sqrt(hr[4]);
           const bool next_ok = o.stop_rule == QPINV_STOP_PAPER_ABS ? rn < 1.0 && nx * rn / (1.0 - rn) < tol
                                                                    : rn <= tol;
@@ -1547,7 +1607,7 @@ int qpinv_solve(qpinv_ctx* c, void* stream, int m, int n, const double* const A[
       const bool reuse = S.res_cur == S.cur;
       penrose(c, S.A, Xf, fp64 ? PM_F64 : PM_EMU, res.E, res.E_rel, nullptr, reuse ? &S.res_R : nullptr, S.left);
       if (reuse) c->stats.penrose_reused++;
-      if (!fp64) check_kernel_error(c);
+      if (!fp64) read_status(c);
     }
     res.gemms = gemms_before + S.gemms;
     if (c->trace)
@@ -1590,14 +1650,32 @@ int qpinv_qgemm(qpinv_ctx* c, void* stream, int m, int k, int n, const double* c
     if (precision != QPINV_PREC_FP64 && !tc_supported())
       return fail(c, QPINV_E_UNSUPPORTED, "tcgen05 path needs an sm_103 device");
     const int kk = k > 0 ? k : 1;
-    QMat a = mat(c, "gA", m, kk, MST_D, precision == QPINV_PREC_TC, false);
-    QMat b = mat(c, "gB", kk, n, MST_D, false, precision == QPINV_PREC_TC);
-    QMat cc = mat(c, "gC", m, n, MST_D, false, false);
+    QMat a = mat(c, "gA", m, kk, 0, precision == QPINV_PREC_TC, false);
+    QMat b = mat(c, "gB", kk, n, 0, false, precision == QPINV_PREC_TC);
+    QMat cc = mat(c, "gC", m, n, 0, false, false);
+    // C is written in place unless it is host memory or shares memory with A or B
+    bool in_place = direct_planes(c, (const double* const*)C, ldc, &cc.d);
+    if (k > 0) {
+      a.d = input_planes(c, A, lda, m, k, "gA");
+      b.d = input_planes(c, B, ldb, k, n, "gB");
+      if (in_place) {
+        uintptr_t c0, c1, lo, hi;
+        planes_range(cc.d, m, n, &c0, &c1);
+        planes_range(a.d, m, k, &lo, &hi);
+        in_place = c1 <= lo || hi <= c0;
+        planes_range(b.d, k, n, &lo, &hi);
+        in_place = in_place && (c1 <= lo || hi <= c0);
+      }
+    }
+    if (!in_place) cc.d = mat(c, "gC", m, n, MST_D, false, false).d;
     if (k == 0) {
-      ck(c, cudaMemsetAsync(cc.d.p, 0, sizeof(double) * 4 * cc.d.ps, c->st), "memset");
+      for (int p = 0; p < 4; p++)
+        ck(c, cudaMemset2DAsync(cc.d.p + p * cc.d.ps, sizeof(double) * cc.d.ld, 0, sizeof(double) * n, m, c->st),
+           "memset");
+    } else if (precision == QPINV_PREC_FP64) {
+      const double fl = 32.0 * m * (double)k * n;
+      timed(c, EV_F64, fl, fl, 0, [&] { return launch_qgemm_f64(m, k, n, dview(a), dview(b), cc.d, c->st); });
     } else {
-      load_planes(c, A, lda, m, k, a);
-      load_planes(c, B, ldb, k, n, b);
       Solver S;
       S.c = c;
       S.dbl = true;
@@ -1608,15 +1686,13 @@ int qpinv_qgemm(qpinv_ctx* c, void* stream, int m, int k, int n, const double* c
         S.forms(a, true, false);
         S.forms(b, false, true);
       }
-      Solver::Acc acc = S.prod(a, b, precision == QPINV_PREC_FP64 ? PM_F64 : (precision == QPINV_PREC_TC ? PM_TC : PM_EMU));
       S.L = 0;
-      CombineArgs args = S.base_args(m, n, &acc);
+      CombineArgs args = S.base_args(m, n, nullptr);
       S.out(args, cc, "f", 1.0);
-      S.run(args);
-      if (precision != QPINV_PREC_FP64) check_kernel_error(c);
+      S.prod_run(a, b, precision == QPINV_PREC_TC ? PM_TC : PM_EMU, args);
     }
-    store_planes(c, cc, C, ldc, m, n);
-    ck(c, cudaStreamSynchronize(c->st), "stream sync");
+    if (!in_place) store_planes(c, cc, C, ldc, m, n);
+    read_status(c);  // synchronises
   } catch (const QpError& e) {
     cudaGetLastError();
     return fail(c, e.code, e.msg);
@@ -1634,11 +1710,11 @@ int qpinv_penrose(qpinv_ctx* c, void* stream, int m, int n, const double* const 
   try {
     const int mode = c->opt.precision == QPINV_PREC_FP64 ? PM_F64 : PM_EMU;
     if (mode == PM_EMU && !tc_supported()) return fail(c, QPINV_E_UNSUPPORTED, "tcgen05 path needs an sm_103 device");
-    QMat a = mat(c, "A", m, n, MST_D, false, false), x = mat(c, "X0", n, m, MST_D, false, false);
-    load_planes(c, A, lda, m, n, a);
-    load_planes(c, X, ldx, n, m, x);
+    QMat a = mat(c, "A", m, n, 0, false, false), x = mat(c, "X0", n, m, 0, false, false);
+    a.d = input_planes(c, A, lda, m, n, "A");
+    x.d = input_planes(c, X, ldx, n, m, "X0");
     penrose(c, a, x, mode, E, E_rel, nullptr);
-    if (mode == PM_EMU) check_kernel_error(c);
+    if (mode == PM_EMU) read_status(c);
   } catch (const QpError& e) {
     cudaGetLastError();
     return fail(c, e.code, e.msg);
@@ -1711,7 +1787,6 @@ int qpinv_cur_complete(qpinv_ctx* c, void* stream, int m, int n, const double* c
       CombineArgs a = S.base_args(R.rows, R.cols, &acc);
       S.out(a, R, "f", 1.0);
       S.run(a);
-      if (!fp64) check_kernel_error(c);
     };
     auto planes = [](const QMat& Q, double* p[4]) {
       for (int q = 0; q < 4; q++) p[q] = Q.d.p + q * Q.d.ps;
@@ -1753,7 +1828,7 @@ int qpinv_cur_complete(qpinv_ctx* c, void* stream, int m, int n, const double* c
       timed(c, EV_EW, 0, 0, bytes_mn * 2.5, [&] { return launch_cur_fill(f, st); });  // C^(t+1)
     }
     store_planes(c, Cm, C, ldc, m, n);
-    ck(c, cudaStreamSynchronize(st), "stream sync");
+    read_status(c);  // the products' error word (the solves read it every iteration); synchronises
   } catch (const std::bad_alloc&) {
     cudaGetLastError();
     return fail(c, QPINV_E_NOMEM, "host allocation failed");
@@ -1811,7 +1886,7 @@ int qpinv_toeplitz_filter(qpinv_ctx* c, void* stream, int N, const double* const
       CombineArgs ca = S2.base_args(R.rows, R.cols, &acc);
       S2.out(ca, R, "f", 1.0);
       S2.run(ca);
-      if (!fp64) check_kernel_error(c);
+      if (!fp64) read_status(c);
     };
     gemm(Xp, S, H);   // h = X^dagger s
     gemm(X, H, Sh);   // s_hat = X h
@@ -2118,7 +2193,7 @@ int qpinv_solve_batched(qpinv_ctx* c, void* stream, int batch, const int* m, con
           // three iterations per matrix: the tiles' relative speed, not a converged solve
           solve_with(t, cnt, sm.data(), sn.data(), sa.data(), sla.data(), sx.data(), slx.data(), nullptr,
                      std::min(max_iter, 3));
-          check_kernel_error(c);
+          read_status(c);
           const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - a0).count();
           if (c->trace)
             fprintf(stderr, "qpinv batched tile %s: %.2f ms on %d sampled matrices\n", batched_tile_name(t), ms, cnt);
@@ -2138,7 +2213,7 @@ int qpinv_solve_batched(qpinv_ctx* c, void* stream, int batch, const int* m, con
       solve_with(tile, batch, m, n, A, lda, X, ldx, &c->bgraph, max_iter);
       return cudaSuccess;
     });
-    check_kernel_error(c);  // bounded waits of the tensor-core engine
+    read_status(c);  // bounded waits of the tensor-core engine
     if (c->bgraph.replays > replays && c->bgraph.replays > 1) c->stats.batched_graph_replays++;
     const double ms =
         std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_start).count();
@@ -2176,8 +2251,8 @@ int qpinv_alpha_features(qpinv_ctx* c, void* stream, int m, int n, const double*
   DeviceGuard g(c->device);
   c->st = (cudaStream_t)stream;
   try {
-    QMat a = mat(c, "A", m, n, MST_D | MST_F, false, false);
-    load_planes(c, A, lda, m, n, a);
+    QMat a = mat(c, "A", m, n, MST_F, false, false);
+    a.d = input_planes(c, A, lda, m, n, "A");
     Planes<const double> av = dview(a);
     double bad = 0.0;
     const double f2 = fro2(c, av, nullptr, m, n, &bad);
