@@ -397,8 +397,16 @@ cudaError_t launch_block_sub(double* W, const double* V, const double* h, int c,
 cudaError_t launch_norm_scale(const double* W, long L, double* nrm, double* out, cudaStream_t st);
 cudaError_t launch_basis_add(double* X, const double* V, const double* y, int k, long L, cudaStream_t st);
 cudaError_t launch_sub(double* out, const double* a, const double* b, long L, cudaStream_t st);
-cudaError_t launch_givens(double* col, double* cs, double* sn, double* g, int j, int fom, double* res,
-                          cudaStream_t st);
+// Givens rotations of Hessenberg columns j0 .. j0 + nb - 1 (columns hstride apart, nb <= 32).
+cudaError_t launch_givens(double* H, long hstride, double* cs, double* sn, double* g, int j0, int nb, int fom,
+                          double* res, cudaStream_t st);
+// nb Arnoldi steps on blocks of L = 4 n m doubles in one cooperative launch
+// (arnoldi_ok(L, m)): writes V_{j0+1} .. and Hessenberg columns j0 .. (unrotated);
+// h: 2 hlen doubles, part: (L + 31) / 32 doubles of scratch, bar: a counter.
+bool arnoldi_ok(long L, int m);
+cudaError_t launch_arnoldi(const Planes<const double>& A, int n, int m, double* V, double* W, double* h, long hlen,
+                           double* H, long hstride, double* part, int j0, int nb, unsigned int* bar, int* err,
+                           cudaStream_t st);
 // C = A B (FP64) for B with 1..16 columns: one block per row of C.
 bool skinny_ok(int m);
 cudaError_t launch_qgemm_skinny(int M, int K, int m, const Planes<const double>& A, const Planes<const double>& B,

@@ -1967,15 +1967,19 @@ int qpinv_global_krylov(qpinv_ctx* c, void* stream, int n, int m, const double* 
     double* V = (double*)buf(c, "kry.V", sizeof(double) * (size_t)(cycle + 1) * L + 64);
     QMat Xm = mat(c, "kry.X", n, m, MST_D, false, false), R = mat(c, "kry.R", n, m, MST_D, false, false);
     QMat Wm = mat(c, "kry.W", n, m, MST_D, false, false);
-    // device: h scratch | norm | Hessenberg columns (rotated in place) | c | s | g | residual estimates
+    // device: dots (two passes) | norm | Hessenberg columns (rotated in place) | c | s | g | residual estimates |
+    // group sums of the fused Arnoldi steps
     const size_t hstride = (size_t)cycle + 1;
-    double* dh = (double*)buf(c, "kry.h", sizeof(double) * ((size_t)cycle + 2 + hstride * cycle + 4 * hstride) + 64);
-    double* dnrm = dh + cycle + 1;
-    double* dH = dh + cycle + 2;
+    bool fused = arnoldi_ok(L, m);
+    double* dh = (double*)buf(c, "kry.h", sizeof(double) * (2 * hstride + 1 + hstride * cycle + 4 * hstride +
+                                                            (fused ? (L + 31) / 32 : 0)) + 64);
+    double* dnrm = dh + 2 * hstride;
+    double* dH = dnrm + 1;
     double* dcs = dH + hstride * cycle;
     double* dsn = dcs + hstride;
     double* dg = dsn + hstride;
     double* dres = dg + hstride;
+    double* dpart = dres + hstride;
     ck(c, cudaMemsetAsync(Xm.d.p, 0, sizeof(double) * L, st), "memset");
     ck(c, cudaMemcpyAsync(R.d.p, Bs.d.p, sizeof(double) * L, cudaMemcpyDeviceToDevice, st), "copy");  // X_0 = 0
     timed(c, EV_EW, 0, 0, 8.0 * L, [&] { return launch_norm_scale(R.d.p, L, dnrm, nullptr, st); });
@@ -2005,26 +2009,41 @@ int qpinv_global_krylov(qpinv_ctx* c, void* stream, int n, int m, const double* 
       bool done = false;
       while (!done) {
         const int j0 = j, nb = std::min({kCheck, cycle - j, max_iter - steps});  // >= 1: not done
-        for (int b = 0; b < nb; b++, j++) {
-          double* Vj = V + (size_t)j * L;
-          Planes<const double> vj{Vj, (long)m, (long)n * m};
-          Planes<double> w{Wm.d.p, (long)m, (long)n * m};
-          timed(c, EV_F64, 32.0 * n * n * m, 32.0 * n * n * m, 0, [&] {
-            return skinny_ok(m) ? launch_qgemm_skinny(n, n, m, dview(As), vj, w, st)
-                                : launch_qgemm_f64(n, n, m, dview(As), vj, w, st);
+        if (fused) {
+          cudaError_t le = cudaSuccess;
+          timed(c, EV_EW, 0, 0, 8.0 * L * nb * (4.0 * j0 + 2 * nb + 8) + 32.0 * n * n * nb, [&] {
+            le = launch_arnoldi(dview(As), n, m, V, Wm.d.p, dh, (long)hstride, dH, (long)hstride, dpart, j0, nb,
+                                c->d_count + 1, c->d_err, st);
+            if (le != cudaErrorCooperativeLaunchTooLarge && le != cudaErrorNotSupported) return le;
+            cudaGetLastError();  // the device does not hold the grid at once: a launch per phase instead
+            fused = false;
+            return cudaSuccess;
           });
-          double* hcol = dH + hstride * j;  // Hessenberg column j (j + 2 entries)
-          ck(c, cudaMemsetAsync(hcol, 0, sizeof(double) * (j + 2), st), "memset");
-          for (int pass = 0; pass < 2; pass++) {  // classical Gram-Schmidt, applied twice
-            timed(c, EV_EW, 0, 0, 8.0 * L * (j + 2), [&] { return launch_block_dot(V, j + 1, Wm.d.p, L, dh, st); });
-            timed(c, EV_EW, 0, 0, 8.0 * L * (j + 3),
-                  [&] { return launch_block_sub(Wm.d.p, V, dh, j + 1, L, hcol, st); });
-          }
-          double* Vn = V + (size_t)(j + 1) * L;  // V_{j+1} = W / h_{j+1,j}
-          timed(c, EV_EW, 0, 0, 16.0 * L, [&] { return launch_norm_scale(Wm.d.p, L, hcol + j + 1, Vn, st); });
-          timed(c, EV_EW, 0, 0, 8.0 * (3 * j + 8),
-                [&] { return launch_givens(hcol, dcs, dsn, dg, j, kind, dres, st); });
         }
+        if (fused) {
+          j += nb;
+        } else {
+          for (int b = 0; b < nb; b++, j++) {
+            double* Vj = V + (size_t)j * L;
+            Planes<const double> vj{Vj, (long)m, (long)n * m};
+            Planes<double> w{Wm.d.p, (long)m, (long)n * m};
+            timed(c, EV_F64, 32.0 * n * n * m, 32.0 * n * n * m, 0, [&] {
+              return skinny_ok(m) ? launch_qgemm_skinny(n, n, m, dview(As), vj, w, st)
+                                  : launch_qgemm_f64(n, n, m, dview(As), vj, w, st);
+            });
+            double* hcol = dH + hstride * j;  // Hessenberg column j (j + 2 entries)
+            ck(c, cudaMemsetAsync(hcol, 0, sizeof(double) * (j + 2), st), "memset");
+            for (int pass = 0; pass < 2; pass++) {  // classical Gram-Schmidt, applied twice
+              timed(c, EV_EW, 0, 0, 8.0 * L * (j + 2), [&] { return launch_block_dot(V, j + 1, Wm.d.p, L, dh, st); });
+              timed(c, EV_EW, 0, 0, 8.0 * L * (j + 3),
+                    [&] { return launch_block_sub(Wm.d.p, V, dh, j + 1, L, hcol, st); });
+            }
+            double* Vn = V + (size_t)(j + 1) * L;  // V_{j+1} = W / h_{j+1,j}
+            timed(c, EV_EW, 0, 0, 16.0 * L, [&] { return launch_norm_scale(Wm.d.p, L, hcol + j + 1, Vn, st); });
+          }
+        }
+        timed(c, EV_EW, 0, 0, 8.0 * nb * (3 * j0 + 8),
+              [&] { return launch_givens(dH, (long)hstride, dcs, dsn, dg, j0, nb, kind, dres, st); });
         // the new columns' rows 0 .. j (rotated R and raw h_{j+1,j}), c, g, estimates
         ck(c, cudaMemcpy2DAsync(H.data() + hstride * j0, sizeof(double) * hstride, dH + hstride * j0,
                                 sizeof(double) * hstride, sizeof(double) * (j + 1), nb, cudaMemcpyDeviceToHost, st),
@@ -2078,7 +2097,7 @@ int qpinv_global_krylov(qpinv_ctx* c, void* stream, int n, int m, const double* 
     read_back(c, dnrm, 1, &bn);
     res.true_rel_res = bn > 0.0 ? tn / bn : tn;
     store_planes(c, Xm, X, ldx, n, m);
-    ck(c, cudaStreamSynchronize(st), "stream sync");
+    read_status(c);  // bounded grid barriers; synchronises
   } catch (const std::bad_alloc&) {
     cudaGetLastError();
     return fail(c, QPINV_E_NOMEM, "host allocation failed");
