@@ -1985,8 +1985,9 @@ int qpinv_global_krylov(qpinv_ctx* c, void* stream, int n, int m, const double* 
     timed(c, EV_EW, 0, 0, 8.0 * L, [&] { return launch_norm_scale(R.d.p, L, dnrm, nullptr, st); });
     double r0 = 0.0;
     read_back(c, dnrm, 1, &r0);
-    // host copies: rotated columns (upper triangle), c, g, residual estimates
-    std::vector<double> H(hstride * cycle), cs(cycle), gv(hstride), rs(cycle), y(cycle);
+    // host copies: rotated columns (upper triangle; grown as they are read: a
+    // whole cycle's matrix is 72 MB at the default 3000 steps), c, g, estimates
+    std::vector<double> H, cs(cycle), gv(hstride), rs(cycle), y(cycle);
     constexpr int kCheck = 16;  // steps launched between host checks of the residual estimates
     int steps = 0;
     bool converged = r0 == 0.0;
@@ -2045,6 +2046,7 @@ int qpinv_global_krylov(qpinv_ctx* c, void* stream, int n, int m, const double* 
         timed(c, EV_EW, 0, 0, 8.0 * nb * (3 * j0 + 8),
               [&] { return launch_givens(dH, (long)hstride, dcs, dsn, dg, j0, nb, kind, dres, st); });
         // the new columns' rows 0 .. j (rotated R and raw h_{j+1,j}), c, g, estimates
+        if (H.size() < hstride * j) H.resize(hstride * j);
         ck(c, cudaMemcpy2DAsync(H.data() + hstride * j0, sizeof(double) * hstride, dH + hstride * j0,
                                 sizeof(double) * hstride, sizeof(double) * (j + 1), nb, cudaMemcpyDeviceToHost, st),
            "read columns");
