@@ -115,20 +115,23 @@ __device__ __forceinline__ void reduce_last_block(const Reduce& r, long nblocks,
   __syncthreads();
   if (!last) return;
   __threadfence();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-#pragma unroll
-  for (int v = 0; v < NVALS; v++) {
-    double s = 0.0;
-    for (long b = threadIdx.x; b < nblocks; b += blockDim.x) s += __ldcg(r.partials + b * NVALS + v);
+  // the warps share the values: warp w adds value w % NVALS over every
+  // (warps / NVALS)-th group of 32 blocks (one value after another with the
+  // whole block took 12-15 k cycles, mostly barriers and FP64 shuffles)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, per = (int)(blockDim.x >> 5) / NVALS;
+  const int v = warp % NVALS, w = warp / NVALS;
+  double s = 0.0;
+  if (w < per) {
+#pragma unroll 4
+    for (long b = 32L * w + lane; b < nblocks; b += 32L * per) s += __ldcg(r.partials + b * NVALS + v);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) sh[warp] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < warps; w++) t += sh[w];
-      r.out[v] = t;
-    }
-    __syncthreads();
+  }
+  __syncthreads();
+  if (threadIdx.x < NVALS) {
+    double t = 0.0;
+    for (int k = 0; k < per; k++) t += sh[k * NVALS + threadIdx.x];
+    r.out[threadIdx.x] = t;
   }
   if (threadIdx.x == 0) *r.count = 0;
 }
@@ -205,33 +208,35 @@ int penrose_norm_blocks(int n);
 cudaError_t launch_penrose_norms(const Planes<const double>& R, int n, double sr, const Reduce& r, cudaStream_t st);
 cudaError_t launch_init_x0(const Planes<const double>& A, int m, int n, double alpha, const Planes<double>& X,
                            cudaStream_t st);
-// Column exponents e (|v| < 2^e over the four planes); `scratch`: COL_SCRATCH(cols) ints
-cudaError_t launch_maxexp(const Planes<const float>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st);
 // D = S (FP64 planes, any strides)
 cudaError_t launch_copy_planes(const Planes<const double>& S, int rows, int cols, const Planes<double>& D,
                                cudaStream_t st);
 cudaError_t launch_f64_to_f32(const Planes<const double>& src, int rows, int cols, const Planes<float>& dst,
                               cudaStream_t st);
-cudaError_t launch_maxexp(const Planes<const double>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st);
 cudaError_t launch_f32_to_f64(const Planes<const float>& src, int rows, int cols,
                               const Planes<double>& dst, cudaStream_t st);
 
-// Exact slices for the eight-product exact-slice GEMM (qgemm_emu.cu): S
-// balanced 7-bit digits of v * 2^-e per component (slice s an integer in
-// [-64, 63], [-128, 128] for s = 0, of weight 2^-7(s+1)), stored as the BF16
-// digit sums of products p0 .. p0 + np - 1: dst [S][np][rows][ld].
-// Rows: A-form with the left combinations; the row exponents are found and
-// written to e.  Cols: the transposed B-form, dst [S][np][cols][ld], with the
-// right combinations and given column exponents (launch_maxexp).  Padding up
-// to the next multiple of 8 along the slice rows is written as 0.
-cudaError_t launch_slice_rows(const Planes<const double>& A, int rows, int cols, int* e, int S, int p0, int np,
-                              bf16* dst, long ld, long ps, cudaStream_t st);
-cudaError_t launch_slice_rows(const Planes<const float>& A, int rows, int cols, int* e, int S, int p0, int np,
-                              bf16* dst, long ld, long ps, cudaStream_t st);
-cudaError_t launch_slice_cols(const Planes<const double>& A, int rows, int cols, const int* e, int S, int p0, int np,
-                              bf16* dst, long ld, long ps, cudaStream_t st);
-cudaError_t launch_slice_cols(const Planes<const float>& A, int rows, int cols, const int* e, int S, int p0, int np,
-                              bf16* dst, long ld, long ps, cudaStream_t st);
+// Exact slices of a product's operands for the eight-product exact-slice GEMM
+// (qgemm_emu.cu): S balanced 7-bit digits of v * 2^-e per component (slice s
+// an integer in [-64, 63], [-128, 128] for s = 0, of weight 2^-7(s+1)), stored
+// as the BF16 digit sums of products p0 .. p0 + np - 1.  P (M x K): A-form with
+// the left combinations, za [S][np][M][lda], row exponents eP; Q (K x N): the
+// transposed B-form with the right combinations, zb [S][np][N][ldb], column
+// exponents eQ.  A null za or zb leaves that operand out.  Padding up to the
+// next multiple of 8 along the slice rows is written as 0.
+struct SliceArgs {
+  int M = 0, N = 0, K = 0, S = 0, p0 = 0, np = 8;
+  int *eP = nullptr, *eQ = nullptr;
+  int* scratch = nullptr;  // COL_SCRATCH(N) ints, kept between the groups of one product
+  bf16* za = nullptr;
+  long lda = 0, psa = 0;
+  bf16* zb = nullptr;
+  long ldb = 0, psb = 0;
+};
+cudaError_t launch_slices(const SliceArgs& a, const Planes<const double>& P, const Planes<const double>& Q,
+                          cudaStream_t st);
+cudaError_t launch_slices(const SliceArgs& a, const Planes<const float>& P, const Planes<const float>& Q,
+                          cudaStream_t st);
 
 cudaError_t launch_qgemm_f64(int M, int K, int N, const Planes<const double>& A,
                              const Planes<const double>& B, const Planes<double>& C,

@@ -442,10 +442,44 @@ __device__ __forceinline__ void slices_store(bf16* dst, long ps, int S, int p0, 
 // A-form: WPR warps per row find the row's exponent (one read of the row),
 // then slice it (the second read hits L1 / L2: a row is at most a few
 // hundred KB), so no separate exponent pass is needed.
+//
+// Blocks past the slicing (blockIdx.x >= cx.first) find the column exponents'
+// partial maxima of the product's other operand: both are needed before the
+// columns can be sliced, and neither depends on the other (one launch less).
+template <typename T>
+struct ColExp {
+  Planes<const T> A;
+  int rows = 0, cols = 0, chunk_rows = 0, colblocks = 0, first = 0x7fffffff;
+  int* part = nullptr;  // [chunk][cols]
+};
+template <typename T>
+__device__ __forceinline__ void col_maxexp_block(const ColExp<T>& cx, int blk, int (*sh)[32]) {
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int j = (blk % cx.colblocks) * 32 + tx, ch = blk / cx.colblocks;
+  const int r0 = ch * cx.chunk_rows, r1 = min(cx.rows, r0 + cx.chunk_rows);
+  int mx = -100000;
+  if (j < cx.cols)
+#pragma unroll 2
+    for (int i = r0 + ty; i < r1; i += 8)
+#pragma unroll
+      for (int c = 0; c < 4; c++) mx = max(mx, exp_of(cx.A.p[c * cx.A.ps + (long)i * cx.A.ld + j]));
+  sh[ty][tx] = mx;
+  __syncthreads();
+  if (ty == 0 && j < cx.cols) {
+#pragma unroll
+    for (int t = 1; t < 8; t++) mx = max(mx, sh[t][tx]);
+    cx.part[(long)ch * cx.cols + j] = mx;
+  }
+}
 template <typename T, int WPR>
 __global__ void __launch_bounds__(256, 2) k_slice_rows(Planes<const T> A, int rows, int cols, int* __restrict__ e_out,
-                                                    int S, int p0, int np, bf16* dst, long ld, long ps) {
-  __shared__ int sh[8];
+                                                    int S, int p0, int np, bf16* dst, long ld, long ps, ColExp<T> cx) {
+  __shared__ int sh2[8][32];
+  if ((int)blockIdx.x >= cx.first) {
+    col_maxexp_block<T>(cx, blockIdx.x - cx.first, sh2);
+    return;
+  }
+  int* sh = sh2[0];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * (8 / WPR) + warp / WPR, tr = (warp % WPR) * 32 + lane;
   const bool ok = i < rows;
@@ -483,15 +517,17 @@ __global__ void __launch_bounds__(256, 2) k_slice_rows(Planes<const T> A, int ro
   }
 }
 
-// B-form (the plane-wise transpose; column exponents e[j]): a block takes 64
-// rows x 32 columns of the four planes through shared memory, then each
-// thread slices 8 consecutive rows of one column (a warp's stores cover 128
+// B-form (the plane-wise transpose): a block takes 64
+// rows x 32 columns of the four planes through shared memory (and finishes its
+// columns' exponents from the chunk maxima), then each thread slices 8 consecutive rows of one column (a warp's stores cover 128
 // bytes of each of 4 slice rows).  Rows past `rows` up to the padded pitch are 0.
 constexpr int SC_ROWS = 64, SC_COLS = 32;
 template <typename T>
-__global__ void __launch_bounds__(256, 2) k_slice_cols(Planes<const T> A, int rows, int cols, const int* __restrict__ e,
-                                                    int S, int p0, int np, bf16* dst, long ld, long ps) {
+__global__ void __launch_bounds__(256, 2) k_slice_cols(Planes<const T> A, int rows, int cols, const int* __restrict__ part,
+                                                       int chunks, int* __restrict__ e, int S, int p0, int np,
+                                                       bf16* dst, long ld, long ps) {
   extern __shared__ __align__(16) unsigned char sc_smem[];
+  __shared__ int ecol[SC_COLS];
   T(*tile)[SC_COLS][SC_ROWS + 1] = reinterpret_cast<T(*)[SC_COLS][SC_ROWS + 1]>(sc_smem);
   const int i0 = blockIdx.y * SC_ROWS, j0 = blockIdx.x * SC_COLS;
   {
@@ -503,11 +539,20 @@ __global__ void __launch_bounds__(256, 2) k_slice_cols(Planes<const T> A, int ro
       for (int c = 0; c < 4; c++) tile[c][jl][il] = in ? A.p[c * A.ps + (long)(i0 + il) * A.ld + j0 + jl] : (T)0;
     }
   }
+  if (threadIdx.x < SC_COLS) {  // the columns' exponents from their chunks' maxima
+    const int j = j0 + threadIdx.x;
+    int mx = -100000;
+    if (j < cols)
+      for (int ch = 0; ch < chunks; ch++) mx = max(mx, part[(long)ch * cols + j]);
+    mx = mx == -100000 ? 0 : mx;
+    ecol[threadIdx.x] = mx;
+    if (blockIdx.y == 0 && j < cols) e[j] = mx;
+  }
   __syncthreads();
   const int jl = threadIdx.x >> 3, ig = (threadIdx.x & 7) * 8;
   const int j = j0 + jl;
   if (j < cols && i0 + ig < ((rows + 7) / 8) * 8) {
-    const int ej = e[j];
+    const int ej = ecol[jl];
     long long G[4][8];
 #pragma unroll
     for (int c = 0; c < 4; c++) {
@@ -711,33 +756,6 @@ __global__ void __launch_bounds__(256) k_init_x0(Planes<const double> A, int m, 
   }
 }
 
-// Exponent e with |v| < 2^e for every v of a column, over all four planes;
-// integer ops on the bits.
-template <typename T>
-__global__ void k_col_maxexp_part(Planes<const T> A, int rows, int cols, int chunk_rows, int* part) {
-  __shared__ int sh[CR_ROWS][CR_COLS];
-  const int j = blockIdx.x * CR_COLS + threadIdx.x;
-  const int r0 = blockIdx.y * chunk_rows, r1 = min(rows, r0 + chunk_rows);
-  int mx = -100000;
-  if (j < cols)
-    for (int i = r0 + threadIdx.y; i < r1; i += CR_ROWS)
-      for (int c = 0; c < 4; c++) mx = max(mx, exp_of(A.p[c * A.ps + (long)i * A.ld + j]));
-  sh[threadIdx.y][threadIdx.x] = mx;
-  __syncthreads();
-  if (threadIdx.y == 0 && j < cols) {
-    for (int t = 1; t < CR_ROWS; t++) mx = max(mx, sh[t][threadIdx.x]);
-    part[(long)blockIdx.y * cols + j] = mx;
-  }
-}
-
-__global__ void k_col_maxexp_finish(const int* part, int chunks, int cols, int* e) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= cols) return;
-  int mx = -100000;
-  for (int ch = 0; ch < chunks; ch++) mx = max(mx, part[(long)ch * cols + j]);
-  e[j] = mx == -100000 ? 0 : mx;
-}
-
 // Row chunks of a column reduction: about four blocks per SM of a 152-SM
 // part in total, at least 64 rows per chunk.
 static int col_chunks(int rows, int cols) {
@@ -853,22 +871,6 @@ cudaError_t launch_init_x0(const Planes<const double>& A, int m, int n, double a
   return cudaGetLastError();
 }
 
-template <typename T>
-static cudaError_t maxexp_t(const Planes<const T>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st) {
-  const int ch = col_chunks(rows, cols), chunk_rows = (rows + ch - 1) / ch;
-  k_col_maxexp_part<T><<<dim3((cols + CR_COLS - 1) / CR_COLS, ch), dim3(CR_COLS, CR_ROWS), 0, st>>>(
-      A, rows, cols, chunk_rows, scratch);
-  k_col_maxexp_finish<<<(cols + 255) / 256, 256, 0, st>>>(scratch, ch, cols, e);
-  g_kernel_launches += 2;
-  return cudaGetLastError();
-}
-cudaError_t launch_maxexp(const Planes<const double>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st) {
-  return maxexp_t<double>(A, rows, cols, e, scratch, st);
-}
-cudaError_t launch_maxexp(const Planes<const float>& A, int rows, int cols, int* e, int* scratch, cudaStream_t st) {
-  return maxexp_t<float>(A, rows, cols, e, scratch, st);
-}
-
 cudaError_t launch_copy_planes(const Planes<const double>& S, int rows, int cols, const Planes<double>& D,
                                cudaStream_t st) {
   if (rows <= 0 || cols <= 0) return cudaSuccess;
@@ -892,49 +894,59 @@ cudaError_t launch_f64_to_f32(const Planes<const double>& src, int rows, int col
 }
 
 
+// See common.cuh.  The row-slicing blocks of P and the exponent blocks of Q
+// share a launch; either part may be absent.
 template <typename T>
-static cudaError_t slice_rows_t(const Planes<const T>& A, int rows, int cols, int* e, int S, int p0, int np, bf16* dst,
-                                long ld, long ps, cudaStream_t st) {
-  if (rows <= 0 || cols <= 0) return cudaSuccess;
-  if ((ld & 7) || (ps & 7) || (reinterpret_cast<uintptr_t>(dst) & 15) || ld < ((cols + 7) / 8) * 8)
-    return cudaErrorInvalidValue;
+static cudaError_t slice_t(const SliceArgs& a, const Planes<const T>& P, const Planes<const T>& Q, cudaStream_t st) {
+  auto bad = [](long ld, long ps, const bf16* dst, int k) {
+    return (ld & 7) || (ps & 7) || (reinterpret_cast<uintptr_t>(dst) & 15) || ld < ((k + 7) / 8) * 8;
+  };
+  if (a.M <= 0 || a.N <= 0 || a.K <= 0) return cudaSuccess;
+  if ((a.za && bad(a.lda, a.psa, a.za, a.K)) || (a.zb && bad(a.ldb, a.psb, a.zb, a.K))) return cudaErrorInvalidValue;
   // four warps per row once a row is more than two iterations of one warp
-  if (cols > 512)
-    k_slice_rows<T, 4><<<(rows + 1) / 2, 256, 0, st>>>(A, rows, cols, e, S, p0, np, dst, ld, ps);
-  else
-    k_slice_rows<T, 1><<<(rows + 7) / 8, 256, 0, st>>>(A, rows, cols, e, S, p0, np, dst, ld, ps);
-  ++g_kernel_launches;
+  const int wpr = a.K > 512 ? 4 : 1;
+  const int row_blocks = a.za ? (wpr == 4 ? (a.M + 1) / 2 : (a.M + 7) / 8) : 0;
+  const int chunks = col_chunks(a.K, a.N);
+  ColExp<T> cx;
+  int col_blocks = 0;
+  if (a.zb && a.p0 == 0) {  // the exponents serve every group of products
+    cx.A = Q;
+    cx.rows = a.K;
+    cx.cols = a.N;
+    cx.chunk_rows = (a.K + chunks - 1) / chunks;
+    cx.colblocks = (a.N + 31) / 32;
+    cx.first = row_blocks;
+    cx.part = a.scratch;
+    col_blocks = cx.colblocks * chunks;
+  }
+  if (row_blocks + col_blocks > 0) {
+    if (wpr == 4)
+      k_slice_rows<T, 4><<<row_blocks + col_blocks, 256, 0, st>>>(P, a.M, a.K, a.eP, a.S, a.p0, a.np, a.za, a.lda,
+                                                                  a.psa, cx);
+    else
+      k_slice_rows<T, 1><<<row_blocks + col_blocks, 256, 0, st>>>(P, a.M, a.K, a.eP, a.S, a.p0, a.np, a.za, a.lda,
+                                                                  a.psa, cx);
+    ++g_kernel_launches;
+    if (cudaError_t err = cudaGetLastError()) return err;
+  }
+  if (a.zb) {
+    constexpr int smem = (int)sizeof(T) * 4 * SC_COLS * (SC_ROWS + 1);
+    static std::atomic<unsigned long long> attr_done{0};
+    if (cudaError_t err = ensure_smem_attr(k_slice_cols<T>, smem, attr_done)) return err;
+    dim3 grid((a.N + SC_COLS - 1) / SC_COLS, (a.K + SC_ROWS - 1) / SC_ROWS);
+    k_slice_cols<T><<<grid, 256, smem, st>>>(Q, a.K, a.N, a.scratch, chunks, a.eQ, a.S, a.p0, a.np, a.zb, a.ldb,
+                                             a.psb);
+    ++g_kernel_launches;
+  }
   return cudaGetLastError();
 }
-template <typename T>
-static cudaError_t slice_cols_t(const Planes<const T>& A, int rows, int cols, const int* e, int S, int p0, int np,
-                                bf16* dst, long ld, long ps, cudaStream_t st) {
-  if (rows <= 0 || cols <= 0) return cudaSuccess;
-  if ((ld & 7) || (ps & 7) || (reinterpret_cast<uintptr_t>(dst) & 15) || ld < ((rows + 7) / 8) * 8)
-    return cudaErrorInvalidValue;
-  constexpr int smem = (int)sizeof(T) * 4 * SC_COLS * (SC_ROWS + 1);
-  static std::atomic<unsigned long long> attr_done{0};
-  if (cudaError_t err = ensure_smem_attr(k_slice_cols<T>, smem, attr_done)) return err;
-  dim3 grid((cols + SC_COLS - 1) / SC_COLS, (rows + SC_ROWS - 1) / SC_ROWS);
-  k_slice_cols<T><<<grid, 256, smem, st>>>(A, rows, cols, e, S, p0, np, dst, ld, ps);
-  ++g_kernel_launches;
-  return cudaGetLastError();
+cudaError_t launch_slices(const SliceArgs& a, const Planes<const double>& P, const Planes<const double>& Q,
+                          cudaStream_t st) {
+  return slice_t<double>(a, P, Q, st);
 }
-cudaError_t launch_slice_rows(const Planes<const double>& A, int rows, int cols, int* e, int S, int p0, int np,
-                              bf16* dst, long ld, long ps, cudaStream_t st) {
-  return slice_rows_t<double>(A, rows, cols, e, S, p0, np, dst, ld, ps, st);
-}
-cudaError_t launch_slice_rows(const Planes<const float>& A, int rows, int cols, int* e, int S, int p0, int np,
-                              bf16* dst, long ld, long ps, cudaStream_t st) {
-  return slice_rows_t<float>(A, rows, cols, e, S, p0, np, dst, ld, ps, st);
-}
-cudaError_t launch_slice_cols(const Planes<const double>& A, int rows, int cols, const int* e, int S, int p0, int np,
-                              bf16* dst, long ld, long ps, cudaStream_t st) {
-  return slice_cols_t<double>(A, rows, cols, e, S, p0, np, dst, ld, ps, st);
-}
-cudaError_t launch_slice_cols(const Planes<const float>& A, int rows, int cols, const int* e, int S, int p0, int np,
-                              bf16* dst, long ld, long ps, cudaStream_t st) {
-  return slice_cols_t<float>(A, rows, cols, e, S, p0, np, dst, ld, ps, st);
+cudaError_t launch_slices(const SliceArgs& a, const Planes<const float>& P, const Planes<const float>& Q,
+                          cudaStream_t st) {
+  return slice_t<float>(a, P, Q, st);
 }
 
 }  // namespace qp

@@ -317,6 +317,7 @@ struct Solver {
   long long gemms = 0;
   QMat A, X[2];
   int cur = 0;
+  bool x_forms = true;  // X[cur] has its operand forms (its last step's X-products ran on BF16 splits)
 
   // ---------------- products ----------------
   struct Acc {
@@ -510,22 +511,24 @@ struct Solver {
     g.A = &za;
     g.B = &zb;
     g.np = np;
+    SliceArgs z;
+    z.M = M;
+    z.N = N;
+    z.K = K;
+    z.S = S;
+    z.np = np;
+    z.eP = eP;
+    z.eQ = eQ;
+    z.scratch = eS;
+    if (!skipP) z.za = za.a, z.lda = za.lda, z.psa = za.psa;
+    if (!skipQ) z.zb = zb.b, z.ldb = zb.ldb, z.psb = zb.psb;
     const double ms = dbl ? 32.0 : 16.0, sbytes = 2.0 * S * np;
-    if (!skipQ)
-      timed(c, EV_EW, 0, 0, ms * K * N, [&] {
-        return dbl ? launch_maxexp(dview(Q), K, N, eQ, eS, c->st) : launch_maxexp(fview(Q), K, N, eQ, eS, c->st);
-      });
+    const double bytes = (skipP ? 0.0 : (ms + sbytes) * M * K) + (skipQ ? 0.0 : (2 * ms + sbytes) * K * N);
     for (int p0 = 0; p0 < 8; p0 += np) {
-      g.p0 = p0;
-      if (!skipP)
-        timed(c, EV_EW, 0, 0, (ms + sbytes) * M * K, [&] {
-          return dbl ? launch_slice_rows(dview(P), M, K, eP, S, p0, np, za.a, za.lda, za.psa, c->st)
-                     : launch_slice_rows(fview(P), M, K, eP, S, p0, np, za.a, za.lda, za.psa, c->st);
-        });
-      if (!skipQ)
-        timed(c, EV_EW, 0, 0, (ms + sbytes) * K * N, [&] {
-          return dbl ? launch_slice_cols(dview(Q), K, N, eQ, S, p0, np, zb.b, zb.ldb, zb.psb, c->st)
-                     : launch_slice_cols(fview(Q), K, N, eQ, S, p0, np, zb.b, zb.ldb, zb.psb, c->st);
+      g.p0 = z.p0 = p0;
+      if (!skipP || !skipQ)
+        timed(c, EV_EW, 0, 0, bytes, [&] {
+          return dbl ? launch_slices(z, dview(P), dview(Q), c->st) : launch_slices(z, fview(P), fview(Q), c->st);
         });
       // 8 real products of 2 M K N flops per slice pair: half of the 16-product form
       timed(c, EV_EMU, flops * np / 8, flops * np / 8 * S * (S + 1) / 4, 0,
@@ -568,8 +571,18 @@ struct Solver {
       a.ps_aux[t] = M.f.ps;
     }
   }
-  // Adds an output; forms: 'f' master of the phase type, 'a' A-form, 'b' B-form.
-  OutSpec& out(CombineArgs& a, const QMat& M, const char* forms, double cacc, double diag = 0.0) {
+  // Split terms of the operand forms an R-product / X-product of this step
+  // reads (0: it works from the masters), and the outputs an operand then
+  // needs: its forms, or its master.  Writing every form at the widest split
+  // and every master doubled what the fused epilogues and combine passes store.
+  bool r_tc() const { return L > 0 && (rmode < 0 || rmode == PM_TC); }
+  int lv_r() const { return r_tc() ? Lr : 0; }
+  int lv_x() const { return L > 0 && xmode == PM_TC ? Lx : 0; }
+  const char* rop(const char* ab) const { return r_tc() ? ab : "f"; }
+  const char* tform() const { return lv_x() ? (left ? "a" : "b") : "f"; }
+  // Adds an output; forms: 'f' master of the phase type, 'a' A-form, 'b'
+  // B-form of `lv` split terms (0: none).
+  OutSpec& out(CombineArgs& a, const QMat& M, const char* forms, int lv, double cacc, double diag = 0.0) {
     OutSpec& o = a.out[a.nout++];
     o = OutSpec();
     if (strchr(forms, 'f')) {
@@ -583,8 +596,8 @@ struct Solver {
         o.mps = M.f.ps;
       }
     }
-    if (L > 0) {
-      o.s16.levels = L;
+    if (L > 0 && lv > 0) {
+      o.s16.levels = lv;
       if (strchr(forms, 'a')) {
         o.s16.a = M.s16.a;
         o.s16.lda = M.s16.lda;
@@ -642,7 +655,6 @@ struct Solver {
     else prod_run(Y, T, xmode, a, with_partials);
     xS = save;
   }
-  const char* tform() const { return left ? "fa" : "fb"; }
   QMat sq(const char* name, bool a, bool b) { return mat(c, name, s, s, MST_F | MST_D, a, b); }
   QMat big(const char* name) { return mat(c, name, n, m, MST_F | MST_D, true, true); }
 
@@ -655,7 +667,7 @@ struct Solver {
     }
     QMat R = sq(name, strchr(forms, 'a') != nullptr, strchr(forms, 'b') != nullptr);
     CombineArgs a = base_args(s, s, nullptr);
-    out(a, R, forms, -1.0, 1.0);
+    out(a, R, forms, std::max(lv_r(), lv_x()), -1.0, 1.0);
     res_run(Y, a, norm, 4);
     if (strcmp(name, "R") == 0) {
       const bool exact = dbl && (xmode == PM_F64 || (xmode == PM_EMU && xS >= 8));
@@ -672,32 +684,34 @@ struct Solver {
     CombineArgs a = base_args(n, m, nullptr);
     aux(a, 0, X[cur]);
     aux(a, 1, base);
-    OutSpec& o = out(a, Xn, "fab", 1.0);
+    x_forms = lv_x() > 0;
+    OutSpec& o = out(a, Xn, "fab", lv_x(), 1.0);
     o.caux[1] = 1.0;  // + base (aux 0 = X_j is only the reference of the norm)
     apply_run(Y, T, a, true);
   }
 
   // ---------------- one iteration of each method ----------------
   void step_ns() {
-    QMat R = residual(X[cur], "R", tform(), true);
+    QMat R = residual(X[cur], "R", lv_x() ? (left ? "fa" : "fb") : "f", true);
     apply_update(X[cur], R, X[cur]);
   }
 
   void step_qsai(double b1, double b2) {
     QMat R = residual(X[cur], "R", "fab", true);
     QMat R2 = sq("R2", true, true);
+    const int lr = lv_r();
     {
       CombineArgs a = base_args(s, s, nullptr);
-      out(a, R2, "fab", 1.0);
+      out(a, R2, "fab", lr, 1.0);
       rprod_run(R, R, a);
     }
     QMat R4 = sq("R4", false, false), Fa = sq("Fa", true, false), Fb = sq("Fb", false, true);
     {
       CombineArgs a = base_args(s, s, nullptr);
       aux(a, 0, R2);
-      out(a, R4, "f", 1.0);
-      out(a, Fa, "fa", 1.0).caux[0] = b1;
-      out(a, Fb, "fb", 1.0).caux[0] = b2;
+      out(a, R4, "f", 0, 1.0);
+      out(a, Fa, rop("a"), lr, 1.0).caux[0] = b1;
+      out(a, Fb, rop("b"), lr, 1.0).caux[0] = b2;
       rprod_run(R2, R2, a);
     }
     QMat q = sq("q", false, true);
@@ -705,7 +719,7 @@ struct Solver {
       CombineArgs a = base_args(s, s, nullptr);
       aux(a, 0, R2);
       aux(a, 1, R4);
-      OutSpec& o = out(a, q, "fb", 1.0);
+      OutSpec& o = out(a, q, "fb", lr, 1.0);
       o.caux[0] = b1 + b2;
       o.caux[1] = 2.0;
       rprod_run(Fa, Fb, a);
@@ -715,7 +729,7 @@ struct Solver {
       CombineArgs a = base_args(s, s, nullptr);
       aux(a, 0, R);
       aux(a, 1, q);
-      OutSpec& o = out(a, t, tform(), 1.0);
+      OutSpec& o = out(a, t, tform(), lv_x(), 1.0);
       o.caux[0] = 1.0;
       o.caux[1] = 1.0;
       rprod_run(R, q, a);
@@ -728,20 +742,21 @@ struct Solver {
     const double c1 = k[5], c2 = k[6], d1 = k[7], d2 = k[8], d3 = k[9], e1 = k[10], e2 = k[11];
     QMat R = residual(X[cur], "R", "fab", true);
     QMat R2 = sq("R2", true, true), S = sq("S", true, false);
+    const int lr = lv_r();
     {
       CombineArgs a = base_args(s, s, nullptr);
       aux(a, 0, R);
-      out(a, R2, "fab", 1.0);
-      out(a, S, "fa", 1.0).caux[0] = 1.0;
+      out(a, R2, "fab", lr, 1.0);
+      out(a, S, "fa", lr, 1.0).caux[0] = 1.0;
       rprod_run(R, R, a);
     }
     QMat R4 = sq("R4", false, false), Fa = sq("Fa", true, false), Fb = sq("Fb", false, true);
     {
       CombineArgs a = base_args(s, s, nullptr);
       aux(a, 0, R2);
-      out(a, R4, "f", 1.0);
-      out(a, Fa, "fa", 1.0).caux[0] = d1;
-      out(a, Fb, "fb", 1.0).caux[0] = d2;
+      out(a, R4, "f", 0, 1.0);
+      out(a, Fa, rop("a"), lr, 1.0).caux[0] = d1;
+      out(a, Fb, rop("b"), lr, 1.0).caux[0] = d2;
       rprod_run(R2, R2, a);
     }
     QMat u = sq("u", false, false), v = sq("v", true, false), w = sq("w", false, true);
@@ -749,13 +764,13 @@ struct Solver {
       CombineArgs a = base_args(s, s, nullptr);
       aux(a, 0, R2);
       aux(a, 1, R4);
-      OutSpec& ou = out(a, u, "f", 1.0);
+      OutSpec& ou = out(a, u, "f", 0, 1.0);
       ou.caux[0] = d1 + d2;
       ou.caux[1] = 2.0;
-      OutSpec& ov = out(a, v, "fa", 1.0);
+      OutSpec& ov = out(a, v, rop("a"), lr, 1.0);
       ov.caux[0] = d1 + d2 + d3;
       ov.caux[1] = 2.0;
-      OutSpec& ow = out(a, w, "fb", 1.0);
+      OutSpec& ow = out(a, w, rop("b"), lr, 1.0);
       ow.caux[0] = d1 + d2 + e1;
       ow.caux[1] = 2.0 + e2;
       rprod_run(Fa, Fb, a);
@@ -766,7 +781,7 @@ struct Solver {
       aux(a, 0, u);
       aux(a, 1, R2);
       aux(a, 2, R4);
-      OutSpec& o = out(a, g, "fb", 1.0);
+      OutSpec& o = out(a, g, rop("b"), lr, 1.0);
       o.caux[0] = 2.0;
       o.caux[1] = d3 + e1 + c1;
       o.caux[2] = e2 + c2;
@@ -776,7 +791,7 @@ struct Solver {
     {
       CombineArgs a = base_args(s, s, nullptr);
       aux(a, 0, S);
-      out(a, t, tform(), 1.0).caux[0] = 1.0;
+      out(a, t, tform(), lv_x(), 1.0).caux[0] = 1.0;
       rprod_run(S, g, a);
     }
     apply_update(X[cur], t, X[cur]);
@@ -787,14 +802,15 @@ struct Solver {
   // by Horner's rule h <- R + R h from h = R: k - 2 R-products, then the
   // update; k products per iteration with the residual.
   void step_qhpim(int k) {
-    QMat R = residual(X[cur], "R", k == 2 ? tform() : "fab", true);
+    QMat R = residual(X[cur], "R", "fab", true);
     QMat H[2] = {sq("h0", true, true), sq("h1", true, true)};
     const QMat* h = &R;
     for (int i = 2; i < k; i++) {
       QMat& hn = H[i & 1];
       CombineArgs a = base_args(s, s, nullptr);
       aux(a, 0, R);
-      out(a, hn, i == k - 1 ? tform() : "fb", 1.0).caux[0] = 1.0;
+      const bool last = i == k - 1;
+      out(a, hn, last ? tform() : rop("b"), last ? lv_x() : lv_r(), 1.0).caux[0] = 1.0;
       rprod_run(R, *h, a);
       h = &hn;
     }
@@ -803,14 +819,14 @@ struct Solver {
 
   // QRAPID correction  W + Y (I - A W)  (right) / W + (I - W A) Y (left) into Z.
   void rapid_correct(const QMat& W, const QMat& Y, QMat& Z, bool is_final) {
-    QMat E = residual(W, "E", tform());
+    QMat E = residual(W, "E", tform());  // an operand of the correction only
     if (is_final) {
       apply_update(Y, E, W);
       return;
     }
     CombineArgs a = base_args(n, m, nullptr);
     aux(a, 0, W);
-    out(a, Z, "fab", 1.0).caux[0] = 1.0;
+    out(a, Z, "fab", lv_x(), 1.0).caux[0] = 1.0;
     apply_run(Y, E, a);
   }
 
@@ -819,7 +835,7 @@ struct Solver {
     QMat R2 = sq("R2", false, true);
     {
       CombineArgs a = base_args(s, s, nullptr);
-      out(a, R2, "fb", 1.0);
+      out(a, R2, "fb", lv_r(), 1.0);
       rprod_run(R, R, a);
     }
     QMat tU = sq("t", left, !left);
@@ -827,7 +843,7 @@ struct Solver {
       CombineArgs a = base_args(s, s, nullptr);
       aux(a, 0, R);
       aux(a, 1, R2);
-      OutSpec& o = out(a, tU, tform(), 0.25);
+      OutSpec& o = out(a, tU, tform(), lv_x(), 0.25);
       o.caux[0] = 1.0;
       o.caux[1] = 1.0;
       rprod_run(R, R2, a);
@@ -836,7 +852,7 @@ struct Solver {
     {  // U = X + X tU
       CombineArgs a = base_args(n, m, nullptr);
       aux(a, 0, X[cur]);
-      out(a, Zb[0], "fab", 1.0).caux[0] = 1.0;
+      out(a, Zb[0], "fab", lv_x(), 1.0).caux[0] = 1.0;
       apply_run(X[cur], tU, a);
     }
     rapid_correct(Zb[0], X[cur], Zb[1], false);  // V = U + X (I - A U)
@@ -871,12 +887,12 @@ struct Solver {
     {
       Acc g = tall ? prod(X[cur], XH, PM_EMU) : prod(XH, X[cur], PM_EMU);
       CombineArgs a = base_args(k, k, &g);
-      out(a, G, "f", 1.0);
+      out(a, G, "f", 0, 1.0);
       run(a);
     }
     Acc y = tall ? prod(G, AH, PM_EMU) : prod(AH, G, PM_EMU);
     CombineArgs a = base_args(n, m, &y);
-    out(a, X[cur ^ 1], "f", 1.0);
+    out(a, X[cur ^ 1], "f", 0, 1.0);
     run(a);
     cur ^= 1;
     L = L0;
@@ -889,7 +905,7 @@ struct Solver {
     if (L == 0) return;
     CombineArgs args = base_args(M.rows, M.cols, nullptr);
     aux(args, 0, M);
-    OutSpec& o = out(args, M, a && b ? "ab" : (a ? "a" : "b"), 0.0);
+    OutSpec& o = out(args, M, a && b ? "ab" : (a ? "a" : "b"), L, 0.0);
     o.caux[0] = 1.0;
     run(args);
   }
@@ -1036,7 +1052,7 @@ void penrose(qpinv_ctx* c, const QMat& A, const QMat& X, int mode, double* E, do
     S.xS = slices;
     Solver::Acc acc = S.prod(P, Q, mode);
     CombineArgs a = S.base_args(Out.rows, Out.cols, &acc);
-    S.out(a, Out, "f", 1.0, diag);
+    S.out(a, Out, "f", 0, 1.0, diag);
     S.run(a);
   };
   double sr = 1.0, sl = 1.0;  // Rr = sr (AX - I), Rl = sl (XA - I)
@@ -1357,7 +1373,7 @@ int qpinv_solve(qpinv_ctx* c, void* stream, int m, int n, const double* const A[
         const double nv = std::sqrt(fro2(c, dview(v), nullptr, n, 1));
         CombineArgs ca = P.base_args(n, 1, nullptr);
         P.aux(ca, 0, v);
-        P.out(ca, v, "f", 0.0).caux[0] = 1.0 / nv;
+        P.out(ca, v, "f", 0, 0.0).caux[0] = 1.0 / nv;
         P.run(ca);
         timed(c, EV_F64, 32.0 * m * n, 32.0 * m * n, 0,
               [&] { return launch_qgemm_f64(m, n, 1, a, dview(v), w.d, c->st); });
@@ -1422,6 +1438,10 @@ int qpinv_solve(qpinv_ctx* c, void* stream, int m, int n, const double* const A[
           S.xS = 4;
         } else {
           S.xmode = PM_TC;
+          if (!S.x_forms) {  // back below the threshold after a step on exact slices
+            S.forms(S.X[S.cur], true, true);
+            S.x_forms = true;
+          }
         }
       }
       // R-products on single BF16 terms while the residual still has
@@ -1688,7 +1708,7 @@ int qpinv_qgemm(qpinv_ctx* c, void* stream, int m, int k, int n, const double* c
       }
       S.L = 0;
       CombineArgs args = S.base_args(m, n, nullptr);
-      S.out(args, cc, "f", 1.0);
+      S.out(args, cc, "f", 0, 1.0);
       S.prod_run(a, b, precision == QPINV_PREC_TC ? PM_TC : PM_EMU, args);
     }
     if (!in_place) store_planes(c, cc, C, ldc, m, n);
@@ -1785,7 +1805,7 @@ int qpinv_cur_complete(qpinv_ctx* c, void* stream, int m, int n, const double* c
       S.xS = 8;
       Solver::Acc acc = S.prod(P, Q, fp64 ? PM_F64 : PM_EMU);
       CombineArgs a = S.base_args(R.rows, R.cols, &acc);
-      S.out(a, R, "f", 1.0);
+      S.out(a, R, "f", 0, 1.0);
       S.run(a);
     };
     auto planes = [](const QMat& Q, double* p[4]) {
@@ -1884,7 +1904,7 @@ int qpinv_toeplitz_filter(qpinv_ctx* c, void* stream, int N, const double* const
       S2.xS = 8;
       Solver::Acc acc = S2.prod(P, Q, fp64 ? PM_F64 : PM_EMU);
       CombineArgs ca = S2.base_args(R.rows, R.cols, &acc);
-      S2.out(ca, R, "f", 1.0);
+      S2.out(ca, R, "f", 0, 1.0);
       S2.run(ca);
       if (!fp64) read_status(c);
     };
