@@ -112,10 +112,6 @@ struct DM {
   __device__ dfv& at(int c, int i, int j) const { return p[c * ps() + (long)i * cols + j]; }
 };
 
-struct Coef {
-  dfv v;
-};
-
 // Output of a fused CTA GEMM pass: out = ca * (P Q) + sum_t ct * aux_t + diag * I,
 // and up to two more outputs formed from it: xo_k = out + sum_t cx_k,t * aux_t
 // (the polynomial blocks that would otherwise take their own elementwise

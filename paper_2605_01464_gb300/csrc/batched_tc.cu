@@ -28,8 +28,8 @@
 // (about 2^-46), which rank-deficient blocks need: rounding that reaches the
 // complement of the range is multiplied by the method's order every step.
 //
-// Roles inside a product (352 threads): warp 0 lane 0 TMA, warps 1-2 lane 0
-// MMA (components 0-1 and 2-3; warp 1 owns TMEM: 512 columns, two FP32 chunk
+// Roles inside a product (352 threads): warp 0 lane 0 TMA, warps 1-2 (one
+// elected lane each) MMA (components 0-1 and 2-3; warp 1 owns TMEM: 512 columns, two FP32 chunk
 // buffers), warps 3-10 the TMEM epilogue (TMEM lane quarter = warp % 4,
 // column half = (warp - 3) / 4); exponents, slicing and the combine use all
 // warps.  mbarrier phases continue across products.  Every wait is bounded
@@ -151,6 +151,24 @@ __device__ __forceinline__ void slice8(bf16* base, long lstride, const dfv* v, f
 #pragma unroll
   for (int q = 0; q < 8; q++) G[q] = biased_fixed(v[q], s1, s2);
   store_planes8<0>(base, lstride, G);
+}
+
+// The 16 signed MMAs of one stage (BK / 16 steps) into components C0, C0 + 1.
+constexpr uint32_t TDESC_HI = ((8 * TSWB) >> 4) | (1u << 14) | (4u << 29);
+__device__ __forceinline__ uint32_t tdesc_lo(uint32_t addr) { return ((addr & 0x3FFFFu) >> 4) | (1u << 16); }
+template <int C0>
+__device__ __forceinline__ void tstage_mmas(uint32_t d, uint32_t ad, uint32_t bd, uint32_t acc) {
+  constexpr uint32_t NEG_A = 1u << 13;
+  const uint64_t hi = (uint64_t)TDESC_HI << 32;
+#pragma unroll
+  for (int kk = 0; kk < TBK / 16; kk++)
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+      for (int c = C0; c < C0 + 2; c++)
+        mma_bf16(d + c * TBN, hi | (ad + ((r * TA_PLANE) >> 4) + kk * 2),
+                 hi | (bd + (((r ^ c) * TB_PLANE) >> 4) + kk * 2), qsign_neg(r, c) ? TIDESC | NEG_A : TIDESC,
+                 (kk || r) ? 1u : acc);
 }
 
 // Epilogue: drain FP32 chunk w (TMEM buffer w % 2) into the thread's int32
@@ -359,10 +377,8 @@ __device__ __noinline__ void TcGemm::products(int M, int N, int K, int u0, int w
                   const uint32_t fb = smem_u32(&ts->full[st]);
                   mbar_expect_tx(fb, TSTAGE);
                   uint8_t* sp = smem + (size_t)st * TSTAGE;
-                  for (int c = 0; c < 4; c++)
-                    tma_load_3d(smem_u32(sp + c * TA_PLANE), mapA, kb * TBK, m0, s * 4 + c, fb);
-                  for (int c = 0; c < 4; c++)
-                    tma_load_3d(smem_u32(sp + 4 * TA_PLANE + c * TB_PLANE), mapB, kb * TBK, n0, (d - s) * 4 + c, fb);
+                  tma_load_3d(smem_u32(sp), mapA, kb * TBK, m0, s * 4, fb);  // four planes per copy
+                  tma_load_3d(smem_u32(sp + 4 * TA_PLANE), mapB, kb * TBK, n0, (d - s) * 4, fb);
                   ts->issued = u + 1;
                 }
               }
@@ -373,52 +389,51 @@ __device__ __noinline__ void TcGemm::products(int M, int N, int K, int u0, int w
       }
     } else if (warp < TEPI0) {
       // ---------------- MMA issuers: warp 1 components 0, 1; warp 2 components 2, 3 ----------------
-      if (lane == 0) {
-        const bool lo = warp == 1;
-        int u = u0, w = w0;
-        bool ok = true;
-        for (int tile = 0; tile < Mt * Nt && ok; tile++) {
-          for (int d = TS - 1; d >= 0 && ok; d--) {
-            for (int k0 = 0; k0 < K && ok; k0 += kc[d], w++) {
-              const int b = w & 1;  // FP32 buffer of this chunk, free once chunk w - 2 was drained
-              if (w >= 2 && !mbar_wait(smem_u32(&ts->acc_empty[b]), ((w >> 1) - 1) & 1, &ts->abort_flag, err, 22)) {
-                ok = false;
-                break;
-              }
-              fence_after();
-              const uint32_t dacc = ts->tmem + b * 256;
-              const int kb0 = k0 / TBK, kb1 = (min(K, k0 + kc[d]) + TBK - 1) / TBK;
-              bool first = true;
-              for (int kb = kb0; kb < kb1 && ok; kb++) {
-                for (int s = 0; s <= d; s++, u++) {
-                  const int st = u % TSTAGES;
-                  if (!mbar_wait(smem_u32(&ts->full[st]), (u / TSTAGES) & 1, &ts->abort_flag, err, 23)) {
-                    ok = false;
-                    break;
-                  }
-                  fence_after();
-                  uint8_t* sp = smem + (size_t)st * TSTAGE;
-                  const uint64_t ad0 = smem_desc_sw<TSWB>(smem_u32(sp)),
-                                 bd0 = smem_desc_sw<TSWB>(smem_u32(sp + 4 * TA_PLANE));
-#pragma unroll
-                  for (int kk = 0; kk < TBK / 16; kk++) {
-                    if (lo)
-                      qmma_k16_half<TA_PLANE, TB_PLANE, 0>(dacc, TBN, ad0 + kk * 2, bd0 + kk * 2, TIDESC,
-                                                          first && kk == 0);
-                    else
-                      qmma_k16_half<TA_PLANE, TB_PLANE, 2>(dacc, TBN, ad0 + kk * 2, bd0 + kk * 2, TIDESC,
-                                                          first && kk == 0);
-                  }
-                  first = false;
+      // warp-uniform loops, one elected lane issues (see elect_one)
+      const bool lo = warp == 1;
+      const uint32_t a_lo = tdesc_lo(smem_u32(smem)), b_lo = tdesc_lo(smem_u32(smem + 4 * TA_PLANE));
+      int w = w0, st = u0 % TSTAGES;
+      uint32_t ph = (uint32_t)(u0 / TSTAGES) & 1u;
+      bool ok = true;
+      for (int tile = 0; tile < Mt * Nt && ok; tile++) {
+        for (int d = TS - 1; d >= 0 && ok; d--) {
+          for (int k0 = 0; k0 < K && ok; k0 += kc[d], w++) {
+            const int b = w & 1;  // FP32 buffer of this chunk, free once chunk w - 2 was drained
+            if (w >= 2 && !mbar_wait(smem_u32(&ts->acc_empty[b]), ((w >> 1) - 1) & 1, &ts->abort_flag, err, 22)) {
+              ok = false;
+              break;
+            }
+            fence_after();
+            const uint32_t dacc = ts->tmem + b * 256;
+            const int kb0 = k0 / TBK, kb1 = (min(K, k0 + kc[d]) + TBK - 1) / TBK;
+            uint32_t acc = 0u;
+            for (int kb = kb0; kb < kb1 && ok; kb++) {
+              for (int s = 0; s <= d; s++) {
+                if (!mbar_wait(smem_u32(&ts->full[st]), ph, &ts->abort_flag, err, 23)) {
+                  ok = false;
+                  break;
+                }
+                fence_after();
+                const uint32_t ad = a_lo + st * (TSTAGE >> 4), bd = b_lo + st * (TSTAGE >> 4);
+                if (elect_one()) {
+                  if (lo) tstage_mmas<0>(dacc, ad, bd, acc);
+                  else tstage_mmas<2>(dacc, ad, bd, acc);
                   mma_commit(smem_u32(&ts->empty[st]));
                 }
+                __syncwarp();
+                acc = 1u;
+                if (++st == TSTAGES) {
+                  st = 0;
+                  ph ^= 1u;
+                }
               }
-              if (ok) mma_commit(smem_u32(&ts->acc_full[b]));
             }
+            if (ok && elect_one()) mma_commit(smem_u32(&ts->acc_full[b]));
+            __syncwarp();
           }
         }
-        if (ok && lo) ts->w = w;
       }
+      if (ok && lo && lane == 0) ts->w = w;
     } else {
       // ---------------- epilogue: FP32 chunk -> int32 level sums (registers) -> int64 (global) -> C ----------------
       // Warp e = warp - TEPI0 reads TMEM lane quarter warp % 4 and column half e / 4
@@ -632,8 +647,8 @@ cudaError_t batched_tc_maps(char* tc_ws, int slots, CUtensorMap* host_maps, void
     char* slot = tc_ws + (size_t)s * TC_SLOT_BYTES;
     const bf16* sa = reinterpret_cast<const bf16*>(slot);
     const bf16* sb = reinterpret_cast<const bf16*>(slot + TC_SLICE_BYTES);
-    if (!make_map(&host_maps[2 * s], sa, TKP, MAXD, 4 * TMAXS, TKP, (long)MAXD * TKP, TBM, TBK) ||
-        !make_map(&host_maps[2 * s + 1], sb, TKP, MAXD, 4 * TMAXS, TKP, (long)MAXD * TKP, TBN, TBK))
+    if (!make_map(&host_maps[2 * s], sa, TKP, MAXD, 4 * TMAXS, TKP, (long)MAXD * TKP, TBM, TBK, 4) ||
+        !make_map(&host_maps[2 * s + 1], sb, TKP, MAXD, 4 * TMAXS, TKP, (long)MAXD * TKP, TBN, TBK, 4))
       return cudaErrorInvalidValue;
   }
   return cudaMemcpyAsync(dev_maps, host_maps, sizeof(CUtensorMap) * 2 * (size_t)slots, cudaMemcpyHostToDevice, st);
