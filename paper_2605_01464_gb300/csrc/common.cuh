@@ -189,10 +189,11 @@ namespace qp {
 // blocks (and partials) launch_combine will use for these arguments
 int combine_blocks(const CombineArgs& a);
 cudaError_t launch_combine(const CombineArgs& a, cudaStream_t st);
-// colsum needs `scratch` of COL_SCRATCH(n) doubles
-cudaError_t launch_abs_sums(const Planes<const double>& A, int m, int n, double* rowsum,
-                            double* colsum, double* scratch, cudaStream_t st);
-cudaError_t launch_max(const double* v, int n, double* out, cudaStream_t st);
+// ||A||_F^2, the non-finite count, the largest row and column modulus sums into
+// out[0..3]; scratch: norms_scratch(m, n) doubles
+long norms_scratch(int m, int n);
+cudaError_t launch_matrix_norms(const Planes<const double>& A, int m, int n, double* scratch, double* out,
+                                unsigned int* count, cudaStream_t st);
 // scratch entries of a column reduction over `cols` columns
 inline long COL_SCRATCH(long cols) { return 64 * cols; }
 // ||A - B||_F^2 (B optional) and the non-finite count of A into r.out[0..1];
@@ -207,6 +208,8 @@ cudaError_t launch_fro2(const Planes<const double>& A, const Planes<const double
 int penrose_norm_blocks(int n);
 cudaError_t launch_penrose_norms(const Planes<const double>& R, int n, double sr, const Reduce& r, cudaStream_t st);
 cudaError_t launch_init_x0(const Planes<const double>& A, int m, int n, double alpha, const Planes<double>& X,
+                           cudaStream_t st);
+cudaError_t launch_init_x0(const Planes<const double>& A, int m, int n, double alpha, const Planes<float>& X,
                            cudaStream_t st);
 // D = S (FP64 planes, any strides)
 cudaError_t launch_copy_planes(const Planes<const double>& S, int rows, int cols, const Planes<double>& D,

@@ -390,6 +390,21 @@ static int combine_groups(const CombineArgs& a) {
 // conversions (exact: the sums are integers of at most 8 bits).
 // Bound: HBM writes, 16 S bytes per entry (double the four-plane form's; the
 // product it feeds does half the tensor work).
+//
+// Up to four slices of FP32 values (28 bits and the bias) are 32-bit integers:
+// half the integer instructions, which bound the FP32 phase's slicing.
+__device__ __forceinline__ int to_fixed32(float v, int sh) {  // as to_fixed, |v 2^sh| <= 2^28
+  const unsigned b = __float_as_uint(v);
+  const int ex = (int)((b >> 23) & 0xFF);
+  const int mant = (int)((b & 0x7FFFFFu) | (1u << 23));
+  const int k = ex - 150 + sh;
+  int F;
+  if (k >= 0) F = mant << k;
+  else if (k <= -26) F = 0;
+  else F = (mant + (1 << (-k - 1))) >> (-k);
+  if (ex == 0) F = 0;
+  return (b >> 31) ? -F : F;
+}
 template <typename T>
 __device__ __forceinline__ void slice_bias(const T* v, int S, int e, long long* G) {
   long long bias = 0;
@@ -397,7 +412,14 @@ __device__ __forceinline__ void slice_bias(const T* v, int S, int e, long long* 
 #pragma unroll
   for (int t = 0; t < 8; t++) G[t] = to_fixed(v[t], 7 * S - e) + bias;
 }
-__device__ __forceinline__ float digit_of(long long G, int sh, bool top) {
+__device__ __forceinline__ void slice_bias(const float* v, int S, int e, int* G) {
+  int bias = 0;
+  for (int q = 0; q < S - 1; q++) bias = (bias << 7) + 64;
+#pragma unroll
+  for (int t = 0; t < 8; t++) G[t] = to_fixed32(v[t], 7 * S - e) + bias;
+}
+template <typename I>
+__device__ __forceinline__ float digit_of(I G, int sh, bool top) {
   if (top) return (float)(int)(G >> sh);
   return __uint_as_float(0x4B000000u | ((unsigned)(G >> sh) & 127u)) - 8388672.0f;
 }
@@ -413,8 +435,8 @@ __device__ __forceinline__ void digit_sums(float w, float x, float y, float z, f
   }
 }
 // dst: the entries' place in slice 0, product p0; planes ps apart, slices np ps apart.
-template <bool LEFT>
-__device__ __forceinline__ void slices_store(bf16* dst, long ps, int S, int p0, int np, const long long (*G)[8]) {
+template <bool LEFT, typename I>
+__device__ __forceinline__ void slices_store(bf16* dst, long ps, int S, int p0, int np, const I (*G)[8]) {
   for (int l = 0; l < S; l++) {
     const int sh = 7 * (S - 1 - l);
     uint32_t pk[8][4];
@@ -471,7 +493,7 @@ __device__ __forceinline__ void col_maxexp_block(const ColExp<T>& cx, int blk, i
     cx.part[(long)ch * cx.cols + j] = mx;
   }
 }
-template <typename T, int WPR>
+template <typename T, int WPR, typename I>
 __global__ void __launch_bounds__(256, 2) k_slice_rows(Planes<const T> A, int rows, int cols, int* __restrict__ e_out,
                                                     int S, int p0, int np, bf16* dst, long ld, long ps, ColExp<T> cx) {
   __shared__ int sh2[8][32];
@@ -504,16 +526,16 @@ __global__ void __launch_bounds__(256, 2) k_slice_rows(Planes<const T> A, int ro
   if (tr == 0) e_out[i] = e;
   const int g8 = (cols + 7) / 8;
   for (int g = tr; g < g8; g += 32 * WPR) {
-    long long G[4][8];
+    I G[4][8];
 #pragma unroll
     for (int c = 0; c < 4; c++) {
       const T* src = row + c * A.ps + 8 * g;
       T v[8];
 #pragma unroll
       for (int q = 0; q < 8; q++) v[q] = 8 * g + q < cols ? src[q] : (T)0;
-      slice_bias<T>(v, S, e, G[c]);
+      slice_bias(v, S, e, G[c]);
     }
-    slices_store<true>(dst + (long)i * ld + 8 * g, ps, S, p0, np, G);
+    slices_store<true, I>(dst + (long)i * ld + 8 * g, ps, S, p0, np, G);
   }
 }
 
@@ -522,7 +544,7 @@ __global__ void __launch_bounds__(256, 2) k_slice_rows(Planes<const T> A, int ro
 // columns' exponents from the chunk maxima), then each thread slices 8 consecutive rows of one column (a warp's stores cover 128
 // bytes of each of 4 slice rows).  Rows past `rows` up to the padded pitch are 0.
 constexpr int SC_ROWS = 64, SC_COLS = 32;
-template <typename T>
+template <typename T, typename I>
 __global__ void __launch_bounds__(256, 2) k_slice_cols(Planes<const T> A, int rows, int cols, const int* __restrict__ part,
                                                        int chunks, int* __restrict__ e, int S, int p0, int np,
                                                        bf16* dst, long ld, long ps) {
@@ -553,82 +575,109 @@ __global__ void __launch_bounds__(256, 2) k_slice_cols(Planes<const T> A, int ro
   const int j = j0 + jl;
   if (j < cols && i0 + ig < ((rows + 7) / 8) * 8) {
     const int ej = ecol[jl];
-    long long G[4][8];
+    I G[4][8];
 #pragma unroll
     for (int c = 0; c < 4; c++) {
       T v[8];
 #pragma unroll
       for (int q = 0; q < 8; q++) v[q] = tile[c][jl][ig + q];
-      slice_bias<T>(v, S, ej, G[c]);
+      slice_bias(v, S, ej, G[c]);
     }
-    slices_store<false>(dst + (long)j * ld + i0 + ig, ps, S, p0, np, G);
+    slices_store<false, I>(dst + (long)j * ld + i0 + ig, ps, S, p0, np, G);
   }
 }
 
-__global__ void k_row_abs_sums(Planes<const double> A, int m, int n, double* rowsum) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= m) return;
-  double s = 0.0;
-  for (int j = lane; j < n; j += 32) {
-    double q = 0.0;
-    for (int c = 0; c < 4; c++) {
-      const double x = A.p[c * A.ps + (long)warp * A.ld + j];
-      q += x * x;
-    }
-    s += sqrt(q);
-  }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) rowsum[warp] = s;
-}
-
-// Column reductions: blocks of 32 columns x one row chunk (a warp reads 32
-// consecutive entries of a row) write one partial per (chunk, column); the
-// finishing kernel combines the partials in chunk order, so the result does
-// not depend on scheduling.
-constexpr int CR_COLS = 32, CR_ROWS = 8, CR_MAX_CHUNKS = 64;
-
-__global__ void k_col_abs_part(Planes<const double> A, int m, int n, int chunk_rows, double* part) {
-  __shared__ double sh[CR_ROWS][CR_COLS];
-  const int j = blockIdx.x * CR_COLS + threadIdx.x;
-  const int r0 = blockIdx.y * chunk_rows, r1 = min(m, r0 + chunk_rows);
-  double s = 0.0;
-  if (j < n)
-    for (int i = r0 + threadIdx.y; i < r1; i += CR_ROWS) {
-      double q = 0.0;
-      for (int c = 0; c < 4; c++) {
-        const double x = A.p[c * A.ps + (long)i * A.ld + j];
-        q += x * x;
-      }
-      s += sqrt(q);
-    }
-  sh[threadIdx.y][threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.y == 0 && j < n) {
-    for (int t = 1; t < CR_ROWS; t++) s += sh[t][threadIdx.x];
-    part[(long)blockIdx.y * n + j] = s;
-  }
-}
-
-__global__ void k_col_abs_finish(const double* part, int chunks, int n, double* colsum) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  double s = 0.0;
-  for (int ch = 0; ch < chunks; ch++) s += part[(long)ch * n + j];
-  colsum[j] = s;
-}
-
-__global__ void k_max(const double* v, int n, double* out) {
+// ||A||_F^2, the non-finite count and the modulus sums of A's rows and columns
+// in one read: a block takes 64 rows x 32 columns and writes one partial sum
+// per row and per column of its tile (the moduli meet in shared memory).
+// Bound: the FP64 pipe's square roots (about 15 instructions each), so they
+// are taken once per entry: a pass each for the norm, the row sums and the
+// column sums, and three more launches for their ends, took 340 us at 2048^2.
+constexpr int MN_ROWS = 64, MN_COLS = 32;
+__global__ void __launch_bounds__(256) k_matrix_norms(Planes<const double> A, int m, int n, double* rowpart,
+                                                      double* colpart, Reduce r) {
+  __shared__ double mod[MN_ROWS][MN_COLS + 1];
   __shared__ double sh[256];
-  double mx = 0.0;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) mx = fmax(mx, v[t]);
-  sh[threadIdx.x] = mx;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int j = blockIdx.x * MN_COLS + tx, r0 = blockIdx.y * MN_ROWS;
+  double s = 0.0, col = 0.0;
+  int bad = 0;
+#pragma unroll 2
+  for (int il = ty; il < MN_ROWS; il += 8) {
+    const int i = r0 + il;
+    double x[4] = {0.0, 0.0, 0.0, 0.0};
+    if (i < m && j < n) {
+#pragma unroll
+      for (int c = 0; c < 4; c++) x[c] = A.p[c * A.ps + (long)i * A.ld + j];
+    }
+    const double q = fma(x[3], x[3], fma(x[2], x[2], fma(x[1], x[1], x[0] * x[0])));
+#pragma unroll
+    for (int c = 0; c < 4; c++) bad += nonfinite_bits(x[c]);
+    const double d = sqrt(q);
+    s += q;
+    col += d;
+    mod[il][tx] = d;
+  }
+  const double t0 = block_sum(s, sh);
+  const double t1 = block_count(bad, sh);
+  if (threadIdx.x == 0) {
+    double* p = r.partials + 2 * ((long)blockIdx.y * gridDim.x + blockIdx.x);
+    p[0] = t0;
+    p[1] = t1;
+  }
   __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + s]);
+  sh[threadIdx.x] = col;
+  __syncthreads();
+  if (ty == 0 && j < n) {
+#pragma unroll
+    for (int k = 1; k < 8; k++) col += sh[tx + 32 * k];
+    colpart[(long)blockIdx.y * n + j] = col;
+  }
+  if (threadIdx.x >= 64 && threadIdx.x < 64 + MN_ROWS) {
+    const int il = threadIdx.x - 64;
+    double t = 0.0;
+    for (int k = 0; k < MN_COLS; k++) t += mod[il][k];
+    if (r0 + il < m) rowpart[(long)blockIdx.x * m + r0 + il] = t;
+  }
+  reduce_last_block<2>(r, (long)gridDim.x * gridDim.y, sh);
+}
+
+// The largest row sum and column sum from the partials (summed in block
+// order); the last block takes the maximum over the blocks.
+__global__ void __launch_bounds__(256) k_norms_finish(const double* rowpart, int cb, int m, const double* colpart,
+                                                      int rb, int n, int row_blocks, Reduce r) {
+  __shared__ double sh[256];
+  __shared__ int last;
+  const bool rows = (int)blockIdx.x < row_blocks;
+  const int idx = (rows ? blockIdx.x : blockIdx.x - row_blocks) * 256 + threadIdx.x, len = rows ? m : n;
+  const double* p = rows ? rowpart : colpart;
+  const int parts = rows ? cb : rb;
+  double s = 0.0;
+  if (idx < len)
+#pragma unroll 4
+    for (int k = 0; k < parts; k++) s += p[(long)k * len + idx];
+  sh[threadIdx.x] = s;
+  __syncthreads();
+  for (int k = 128; k > 0; k >>= 1) {
+    if ((int)threadIdx.x < k) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + k]);
     __syncthreads();
   }
-  if (threadIdx.x == 0) out[0] = sh[0];
+  if (threadIdx.x == 0) {
+    r.partials[blockIdx.x] = sh[0];
+    __threadfence();
+    last = atomicAdd(r.count, 1u) == gridDim.x - 1 ? 1 : 0;
+  }
+  __syncthreads();
+  if (!last || threadIdx.x >= 2) return;
+  __threadfence();
+  double mx = 0.0;
+  const int b0 = threadIdx.x == 0 ? 0 : row_blocks, b1 = threadIdx.x == 0 ? row_blocks : (int)gridDim.x;
+  for (int b = b0; b < b1; b++) mx = fmax(mx, __ldcg(r.partials + b));
+  r.out[2 + threadIdx.x] = mx;
+  if (threadIdx.x == 0) *r.count = 0;
 }
+
+constexpr int CR_COLS = 32, CR_MAX_CHUNKS = 64;  // column blocks and row chunks of the column exponents
 
 // ||A - B||_F^2 (B optional) and the non-finite count of A.  Work is split
 // into tasks of one row and FRO_COLS consecutive columns; a block takes tasks
@@ -735,8 +784,8 @@ __global__ void __launch_bounds__(256) k_penrose_norms(Planes<const double> R, i
 }
 
 // X (n x m) = alpha * A^H, A m x n: X[j][i] = alpha * conj(A[i][j]).
-__global__ void __launch_bounds__(256) k_init_x0(Planes<const double> A, int m, int n, double al,
-                                                 Planes<double> X) {
+template <typename T>
+__global__ void __launch_bounds__(256) k_init_x0(Planes<const double> A, int m, int n, double al, Planes<T> X) {
   __shared__ double t[4][TILE][TILE + 1];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int r0 = blockIdx.y * TILE, c0 = blockIdx.x * TILE;  // tile of A: rows r0.., cols c0..
@@ -751,7 +800,8 @@ __global__ void __launch_bounds__(256) k_init_x0(Planes<const double> A, int m, 
     if (i < m && j < n)
       for (int c = 0; c < 4; c++) {
         const double v = t[c][tx][ty + q * TROWS];
-        X.p[c * X.ps + (long)j * X.ld + i] = al * (c == 0 ? v : -v);
+        const double x = al * (c == 0 ? v : flip_sign(v));
+        X.p[c * X.ps + (long)j * X.ld + i] = sizeof(T) == 4 ? (T)narrow(x) : (T)x;
       }
   }
 }
@@ -822,22 +872,20 @@ cudaError_t launch_combine(const CombineArgs& args, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_abs_sums(const Planes<const double>& A, int m, int n, double* rowsum, double* colsum,
-                            double* scratch, cudaStream_t st) {
-  k_row_abs_sums<<<(m + 7) / 8, 256, 0, st>>>(A, m, n, rowsum);
-  ++g_kernel_launches;
-  const int ch = col_chunks(m, n), chunk_rows = (m + ch - 1) / ch;
-  k_col_abs_part<<<dim3((n + CR_COLS - 1) / CR_COLS, ch), dim3(CR_COLS, CR_ROWS), 0, st>>>(A, m, n, chunk_rows,
-                                                                                         scratch);
-  ++g_kernel_launches;
-  k_col_abs_finish<<<(n + 255) / 256, 256, 0, st>>>(scratch, ch, n, colsum);
-  ++g_kernel_launches;
-  return cudaGetLastError();
+long norms_scratch(int m, int n) {  // row and column partials, block partials of both launches
+  const long cb = (n + MN_COLS - 1) / MN_COLS, rb = (m + MN_ROWS - 1) / MN_ROWS;
+  return cb * m + rb * n + std::max(2 * cb * rb, (long)(m + 255) / 256 + (n + 255) / 256);
 }
-
-cudaError_t launch_max(const double* v, int n, double* out, cudaStream_t st) {
-  k_max<<<1, 256, 0, st>>>(v, n, out);
-  ++g_kernel_launches;
+cudaError_t launch_matrix_norms(const Planes<const double>& A, int m, int n, double* scratch, double* out,
+                                unsigned int* count, cudaStream_t st) {
+  const int cb = (n + MN_COLS - 1) / MN_COLS, rb = (m + MN_ROWS - 1) / MN_ROWS;
+  if (rb > 65535) return cudaErrorInvalidValue;  // 4 million rows
+  double *rowpart = scratch, *colpart = scratch + (long)cb * m;
+  const Reduce r{colpart + (long)rb * n, out, count};
+  k_matrix_norms<<<dim3(cb, rb), 256, 0, st>>>(A, m, n, rowpart, colpart, r);
+  const int row_blocks = (m + 255) / 256;
+  k_norms_finish<<<row_blocks + (n + 255) / 256, 256, 0, st>>>(rowpart, cb, m, colpart, rb, n, row_blocks, r);
+  g_kernel_launches += 2;
   return cudaGetLastError();
 }
 
@@ -863,12 +911,21 @@ cudaError_t launch_penrose_norms(const Planes<const double>& R, int n, double sr
   return cudaGetLastError();
 }
 
-cudaError_t launch_init_x0(const Planes<const double>& A, int m, int n, double alpha, const Planes<double>& X,
-                           cudaStream_t st) {
+template <typename T>
+static cudaError_t init_x0_t(const Planes<const double>& A, int m, int n, double alpha, const Planes<T>& X,
+                             cudaStream_t st) {
   dim3 grid((n + TILE - 1) / TILE, (m + TILE - 1) / TILE);
-  k_init_x0<<<grid, TILE * TROWS, 0, st>>>(A, m, n, alpha, X);
+  k_init_x0<T><<<grid, TILE * TROWS, 0, st>>>(A, m, n, alpha, X);
   ++g_kernel_launches;
   return cudaGetLastError();
+}
+cudaError_t launch_init_x0(const Planes<const double>& A, int m, int n, double alpha, const Planes<double>& X,
+                           cudaStream_t st) {
+  return init_x0_t<double>(A, m, n, alpha, X, st);
+}
+cudaError_t launch_init_x0(const Planes<const double>& A, int m, int n, double alpha, const Planes<float>& X,
+                           cudaStream_t st) {
+  return init_x0_t<float>(A, m, n, alpha, X, st);
 }
 
 cudaError_t launch_copy_planes(const Planes<const double>& S, int rows, int cols, const Planes<double>& D,
@@ -896,7 +953,7 @@ cudaError_t launch_f64_to_f32(const Planes<const double>& src, int rows, int col
 
 // See common.cuh.  The row-slicing blocks of P and the exponent blocks of Q
 // share a launch; either part may be absent.
-template <typename T>
+template <typename T, typename I>
 static cudaError_t slice_t(const SliceArgs& a, const Planes<const T>& P, const Planes<const T>& Q, cudaStream_t st) {
   auto bad = [](long ld, long ps, const bf16* dst, int k) {
     return (ld & 7) || (ps & 7) || (reinterpret_cast<uintptr_t>(dst) & 15) || ld < ((k + 7) / 8) * 8;
@@ -921,10 +978,10 @@ static cudaError_t slice_t(const SliceArgs& a, const Planes<const T>& P, const P
   }
   if (row_blocks + col_blocks > 0) {
     if (wpr == 4)
-      k_slice_rows<T, 4><<<row_blocks + col_blocks, 256, 0, st>>>(P, a.M, a.K, a.eP, a.S, a.p0, a.np, a.za, a.lda,
+      k_slice_rows<T, 4, I><<<row_blocks + col_blocks, 256, 0, st>>>(P, a.M, a.K, a.eP, a.S, a.p0, a.np, a.za, a.lda,
                                                                   a.psa, cx);
     else
-      k_slice_rows<T, 1><<<row_blocks + col_blocks, 256, 0, st>>>(P, a.M, a.K, a.eP, a.S, a.p0, a.np, a.za, a.lda,
+      k_slice_rows<T, 1, I><<<row_blocks + col_blocks, 256, 0, st>>>(P, a.M, a.K, a.eP, a.S, a.p0, a.np, a.za, a.lda,
                                                                   a.psa, cx);
     ++g_kernel_launches;
     if (cudaError_t err = cudaGetLastError()) return err;
@@ -932,9 +989,9 @@ static cudaError_t slice_t(const SliceArgs& a, const Planes<const T>& P, const P
   if (a.zb) {
     constexpr int smem = (int)sizeof(T) * 4 * SC_COLS * (SC_ROWS + 1);
     static std::atomic<unsigned long long> attr_done{0};
-    if (cudaError_t err = ensure_smem_attr(k_slice_cols<T>, smem, attr_done)) return err;
+    if (cudaError_t err = ensure_smem_attr(k_slice_cols<T, I>, smem, attr_done)) return err;
     dim3 grid((a.N + SC_COLS - 1) / SC_COLS, (a.K + SC_ROWS - 1) / SC_ROWS);
-    k_slice_cols<T><<<grid, 256, smem, st>>>(Q, a.K, a.N, a.scratch, chunks, a.eQ, a.S, a.p0, a.np, a.zb, a.ldb,
+    k_slice_cols<T, I><<<grid, 256, smem, st>>>(Q, a.K, a.N, a.scratch, chunks, a.eQ, a.S, a.p0, a.np, a.zb, a.ldb,
                                              a.psb);
     ++g_kernel_launches;
   }
@@ -942,11 +999,11 @@ static cudaError_t slice_t(const SliceArgs& a, const Planes<const T>& P, const P
 }
 cudaError_t launch_slices(const SliceArgs& a, const Planes<const double>& P, const Planes<const double>& Q,
                           cudaStream_t st) {
-  return slice_t<double>(a, P, Q, st);
+  return slice_t<double, long long>(a, P, Q, st);
 }
 cudaError_t launch_slices(const SliceArgs& a, const Planes<const float>& P, const Planes<const float>& Q,
                           cudaStream_t st) {
-  return slice_t<float>(a, P, Q, st);
+  return a.S <= 4 ? slice_t<float, int>(a, P, Q, st) : slice_t<float, long long>(a, P, Q, st);
 }
 
 }  // namespace qp

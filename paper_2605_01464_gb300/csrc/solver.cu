@@ -1022,6 +1022,14 @@ double fro2(qpinv_ctx* c, const Planes<const double>& P, const Planes<const doub
   return h[0];
 }
 
+// The four values of launch_matrix_norms (one host read).
+void matrix_norms(qpinv_ctx* c, const Planes<const double>& A, int m, int n, double* h) {
+  double* scratch = (double*)buf(c, "norms", sizeof(double) * (size_t)norms_scratch(m, n) + 64);
+  timed(c, EV_EW, 0, 0, 32.0 * m * n,
+        [&] { return launch_matrix_norms(A, m, n, scratch, c->d_red, c->d_count, c->st); });
+  read_status(c, 4, h);
+}
+
 // The four sums of launch_penrose_norms into dst.
 void penrose_norms_to(qpinv_ctx* c, const QMat& R, double sr, double* dst) {
   const Reduce r{(double*)buf(c, "ah_part", sizeof(double) * 4 * (size_t)penrose_norm_blocks(R.rows) + 64), dst,
@@ -1047,7 +1055,6 @@ void penrose(qpinv_ctx* c, const QMat& A, const QMat& X, int mode, double* E, do
   S.dbl = true;
   S.L = 0;
   QMat Rr = mat(c, "pRr", m, m, MST_D, false, false), Rl = mat(c, "pRl", n, n, MST_D, false, false);
-  QMat E1m = mat(c, "pE1", m, n, MST_D, false, false), E2m = mat(c, "pE2", n, m, MST_D, false, false);
   auto product = [&](const QMat& P, const QMat& Q, QMat& Out, int slices, double diag) {
     S.xS = slices;
     Solver::Acc acc = S.prod(P, Q, mode);
@@ -1082,18 +1089,28 @@ void penrose(qpinv_ctx* c, const QMat& A, const QMat& X, int mode, double* E, do
   // full-rank A) the product needs only a few digits relative to ||R|| ||Q||:
   // 6 slices are accepted when the result exceeds 1e3 times a bound on their
   // truncation error, 2^(10 - 7S) K ||R||_F ||Q||_F; otherwise 8 slices.
-  auto outer = [&](const QMat& R, const QMat& Q, QMat& Out, double fr, double fq) {
-    const int rows = R.rows, cols = Q.cols, K = R.cols;
-    if (mode == PM_EMU && fr <= 1e-3) {
-      product(R, Q, Out, 6, 0.0);
-      const double e = std::sqrt(fro2(c, dview(Out), nullptr, rows, cols));
-      if (e >= 1e3 * std::ldexp(1.0, 10 - 7 * 6) * K * fr * fq) return e;
-    }
-    product(R, Q, Out, 8, 0.0);
-    return std::sqrt(fro2(c, dview(Out), nullptr, rows, cols));
+  // The products themselves are not kept: the combine pass forms their entries
+  // and adds the squares.
+  auto outer_norm = [&](const QMat& R, const QMat& Q, int slices) {
+    S.xS = slices;
+    Solver::Acc acc = S.prod(R, Q, mode);
+    CombineArgs ca = S.base_args(R.rows, Q.cols, &acc);
+    QMat none;
+    S.out(ca, none, "", 0, 1.0);
+    S.run(ca, true, 0);
+    double s[3];
+    read_status(c, 3, s);
+    return std::sqrt(s[1]);
   };
-  E[0] = outer(Rr, A, E1m, std::sqrt(h[4] + h[5]), fa);
-  E[1] = outer(Rl, X, E2m, std::sqrt(h[8] + h[9]), fx);
+  auto outer = [&](const QMat& R, const QMat& Q, double fr, double fq) {
+    if (mode == PM_EMU && fr <= 1e-3) {
+      const double e = outer_norm(R, Q, 6);
+      if (e >= 1e3 * std::ldexp(1.0, 10 - 7 * 6) * R.cols * fr * fq) return e;
+    }
+    return outer_norm(R, Q, 8);
+  };
+  E[0] = outer(Rr, A, std::sqrt(h[4] + h[5]), fa);
+  E[1] = outer(Rl, X, std::sqrt(h[8] + h[9]), fx);
   if (gemms) *gemms += S.gemms;
   E[2] = std::sqrt(h[7]);
   E[3] = std::sqrt(h[11]);
@@ -1311,18 +1328,12 @@ int qpinv_solve(qpinv_ctx* c, void* stream, int m, int n, const double* const A[
     S.A = mat(c, "A", m, n, MST_F, !S.left, S.left);
     S.A.d = input_planes(c, A, lda, m, n, "A");
     Planes<const double> a = dview(S.A);
-    double bad = 0.0;
-    const double a_f2 = fro2(c, a, nullptr, m, n, &bad);
-    if (bad > 0.0 || !std::isfinite(a_f2)) return fail(c, QPINV_E_NONFINITE, "A contains NaN or Inf");
-    // ---- norms and alpha (Thm. 1) ----
-    double* rs = (double*)buf(c, "rowsum", sizeof(double) * (size_t)(m + n) + 64);
-    double* mx = (double*)buf(c, "maxes", sizeof(double) * 4);
-    timed(c, EV_EW, 0, 0, 64.0 * m * n, [&] { return launch_abs_sums(a, m, n, rs, rs + m, (double*)buf(c, "colpart", sizeof(double) * (size_t)COL_SCRATCH(n) + 64), c->st); });
-    timed(c, EV_EW, 0, 0, 8.0 * m, [&] { return launch_max(rs, m, mx, c->st); });
-    timed(c, EV_EW, 0, 0, 8.0 * n, [&] { return launch_max(rs + m, n, mx + 1, c->st); });
-    double hm[2];
-    read_back(c, mx, 2, hm);
-    const double norm_inf = hm[0], norm_1 = hm[1];
+    // ---- norms and alpha (Thm. 1): ||A||_F^2, non-finite count, ||A||_inf, ||A||_1 ----
+    double hn[4];
+    matrix_norms(c, a, m, n, hn);
+    const double a_f2 = hn[0];
+    if (hn[1] > 0.0 || !std::isfinite(a_f2)) return fail(c, QPINV_E_NONFINITE, "A contains NaN or Inf");
+    const double norm_inf = hn[2], norm_1 = hn[3];
     const double a2est = std::sqrt(norm_1 * norm_inf);  // >= sigma_1
     double alpha = 0.0;
     int amode = o.alpha_mode;
@@ -1394,10 +1405,10 @@ int qpinv_solve(qpinv_ctx* c, void* stream, int m, int n, const double* const A[
     S.X[0] = mat(c, "X0", n, m, MST_D | MST_F, true, true);
     S.X[1] = mat(c, "X1", n, m, MST_D | MST_F, true, true);
     S.cur = 0;
-    ck(c, launch_init_x0(a, m, n, alpha, S.X[0].d, c->st), "init X0");
     const int Lr = o.split_level ? o.split_level : 2;
     bool polish = fp64 || emu;  // these forms run in their final precision from the start
     if (fp64 || emu) {
+      ck(c, launch_init_x0(a, m, n, alpha, S.X[0].d, c->st), "init X0");
       S.dbl = true;
       S.L = 0;
       S.xmode = S.rmode = fp64 ? PM_F64 : PM_EMU;
@@ -1418,7 +1429,7 @@ int qpinv_solve(qpinv_ctx* c, void* stream, int m, int n, const double* const A[
       S.L = std::max(S.Lx, Lr);  // BF16 terms the operand forms need: no more are written
       S.xmode = PM_TC;
       ck(c, launch_f64_to_f32(a, m, n, S.A.f, c->st), "A to fp32");
-      ck(c, launch_f64_to_f32(dview(S.X[0]), n, m, S.X[0].f, c->st), "X0 to fp32");
+      ck(c, launch_init_x0(a, m, n, alpha, S.X[0].f, c->st), "init X0");
       S.forms(S.A, !S.left, S.left);
       S.forms(S.X[0], true, true);
     }
@@ -2295,19 +2306,12 @@ int qpinv_alpha_features(qpinv_ctx* c, void* stream, int m, int n, const double*
     QMat a = mat(c, "A", m, n, MST_F, false, false);
     a.d = input_planes(c, A, lda, m, n, "A");
     Planes<const double> av = dview(a);
-    double bad = 0.0;
-    const double f2 = fro2(c, av, nullptr, m, n, &bad);
-    if (bad > 0.0) return fail(c, QPINV_E_NONFINITE, "A contains NaN or Inf");
-    double* rs = (double*)buf(c, "rowsum", sizeof(double) * (size_t)(m + n) + 64);
-    double* mx = (double*)buf(c, "maxes", sizeof(double) * 4);
-    ck(c, launch_abs_sums(av, m, n, rs, rs + m, (double*)buf(c, "colpart", sizeof(double) * (size_t)COL_SCRATCH(n) + 64), c->st), "abs sums");
-    ck(c, launch_max(rs, m, mx, c->st), "max");
-    ck(c, launch_max(rs + m, n, mx + 1, c->st), "max");
-    double hm[2];
-    read_back(c, mx, 2, hm);
+    double hn[4];
+    matrix_norms(c, av, m, n, hn);
+    if (hn[1] > 0.0) return fail(c, QPINV_E_NONFINITE, "A contains NaN or Inf");
     ck(c, launch_f64_to_f32(av, m, n, a.f, c->st), "A to fp32");
     double t1 = 0.0;
-    features_of(c, a, f2, hm[1], hm[0], feat, &t1);
+    features_of(c, a, hn[0], hn[3], hn[2], feat, &t1);
     if (theta1) *theta1 = t1;
   } catch (const QpError& e) {
     cudaGetLastError();
