@@ -148,6 +148,8 @@ __global__ void __launch_bounds__(32 * PW_ROWS * PW_WARPS) k_power_step(Planes<c
                                                                         const float* yprev, const double* d2prev,
                                                                         float* y, double* part, unsigned int* count,
                                                                         double* d2) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double wsum[PW_ROWS * PW_WARPS];
   __shared__ float racc[PW_ROWS * PW_WARPS][4];
   __shared__ int last;
@@ -474,8 +476,10 @@ cudaError_t power_radius(const Planes<const float>& M, int s, int steps, float* 
   if ((e = cudaMemsetAsync(count, 0, sizeof(unsigned int), st)) != cudaSuccess) return e;
   float* buf2[2] = {v, y};
   for (int k = 0; k < steps; k++)
-    k_power_step<<<blocks, 32 * PW_ROWS * PW_WARPS, 0, st>>>(M, s, buf2[k & 1], k ? dscratch + k - 1 : nullptr,
-                                                    buf2[(k + 1) & 1], part, count, dscratch + k);
+    if ((e = launch_pdl(k_power_step, dim3(blocks), dim3(32 * PW_ROWS * PW_WARPS), 0, st, M, s,
+                        (const float*)buf2[k & 1], (const double*)(k ? dscratch + k - 1 : nullptr), buf2[(k + 1) & 1],
+                        part, count, dscratch + k)) != cudaSuccess)
+      return e;
   g_kernel_launches += steps;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = cudaMemcpyAsync(pin, dscratch, sizeof(double) * steps, cudaMemcpyDeviceToHost, st)) != cudaSuccess)

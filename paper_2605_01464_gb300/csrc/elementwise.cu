@@ -265,6 +265,8 @@ __device__ __forceinline__ void split_store2(bf16* base, long idx, long lstride,
 // instructions per value), conversions and sign flips are integer operations.
 template <typename T>
 __global__ void __launch_bounds__(256) k_combine(const __grid_constant__ CombineArgs a, int groups) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float stage[4][2 * TILE][TILE + 1];  // [plane][column][row]
   __shared__ double red[256];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -280,7 +282,8 @@ __global__ void __launch_bounds__(256) k_combine(const __grid_constant__ Combine
       T v[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
       const bool in0 = i < a.rows && j < a.cols, two = in0 && j + 1 < a.cols;
       if (in0) {
-        if (a.acc && O.kacc.kind != CK_ZERO) acc_pairs<T>(a, O.kacc, i, j, two, v);
+        const bool acc_in = a.acc && O.kacc.kind != CK_ZERO;
+        if (acc_in) acc_pairs<T>(a, O.kacc, i, j, two, v);
 #pragma unroll
         for (int t = 0; t < 4; t++) {
           if (!a.aux[t] || O.kaux[t].kind == CK_ZERO) continue;
@@ -289,6 +292,14 @@ __global__ void __launch_bounds__(256) k_combine(const __grid_constant__ Combine
           T u[4][2];
 #pragma unroll
           for (int c = 0; c < 4; c++) ld2(ap + c * a.ps_aux[t], two, u[c][0], u[c][1]);
+          if (t == 0 && !acc_in && O.kaux[0].kind == CK_ONE) {  // a plain copy takes no arithmetic
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+              v[c][0] = u[c][0];
+              v[c][1] = u[c][1];
+            }
+            continue;
+          }
 #pragma unroll
           for (int c = 0; c < 4; c++) {
             v[c][0] += ct * u[c][0];
@@ -496,6 +507,8 @@ __device__ __forceinline__ void col_maxexp_block(const ColExp<T>& cx, int blk, i
 template <typename T, int WPR, typename I>
 __global__ void __launch_bounds__(256, 2) k_slice_rows(Planes<const T> A, int rows, int cols, int* __restrict__ e_out,
                                                     int S, int p0, int np, bf16* dst, long ld, long ps, ColExp<T> cx) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ int sh2[8][32];
   if ((int)blockIdx.x >= cx.first) {
     col_maxexp_block<T>(cx, blockIdx.x - cx.first, sh2);
@@ -548,6 +561,8 @@ template <typename T, typename I>
 __global__ void __launch_bounds__(256, 2) k_slice_cols(Planes<const T> A, int rows, int cols, const int* __restrict__ part,
                                                        int chunks, int* __restrict__ e, int S, int p0, int np,
                                                        bf16* dst, long ld, long ps) {
+  pdl_wait();
+  pdl_trigger();
   extern __shared__ __align__(16) unsigned char sc_smem[];
   __shared__ int ecol[SC_COLS];
   T(*tile)[SC_COLS][SC_ROWS + 1] = reinterpret_cast<T(*)[SC_COLS][SC_ROWS + 1]>(sc_smem);
@@ -596,6 +611,8 @@ __global__ void __launch_bounds__(256, 2) k_slice_cols(Planes<const T> A, int ro
 constexpr int MN_ROWS = 64, MN_COLS = 32;
 __global__ void __launch_bounds__(256) k_matrix_norms(Planes<const double> A, int m, int n, double* rowpart,
                                                       double* colpart, Reduce r) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double mod[MN_ROWS][MN_COLS + 1];
   __shared__ double sh[256];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -646,6 +663,8 @@ __global__ void __launch_bounds__(256) k_matrix_norms(Planes<const double> A, in
 // order); the last block takes the maximum over the blocks.
 __global__ void __launch_bounds__(256) k_norms_finish(const double* rowpart, int cb, int m, const double* colpart,
                                                       int rb, int n, int row_blocks, Reduce r) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double sh[256];
   __shared__ int last;
   const bool rows = (int)blockIdx.x < row_blocks;
@@ -689,6 +708,8 @@ constexpr int FRO_COLS = 256, FRO_U = 2;
 template <bool HASB>
 __global__ void __launch_bounds__(FRO_COLS) k_fro2(Planes<const double> A, Planes<const double> B, int m, int n,
                                                    Reduce r) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double sh[256];
   const unsigned chunks = (n + FRO_COLS - 1) / FRO_COLS;
   const unsigned tasks = (unsigned)m * chunks;  // below 2^31 for any matrix that fits the device
@@ -735,6 +756,8 @@ __global__ void __launch_bounds__(FRO_COLS) k_fro2(Planes<const double> A, Plane
 // the norm of +-R + I, which differs on the diagonal's s plane only, and the
 // anti-Hermitian part) at 2 FP64 operations per value instead of 7.
 __global__ void __launch_bounds__(256) k_penrose_norms(Planes<const double> R, int n, int neg, Reduce r) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double t[4][TILE][TILE + 1];
   __shared__ double sh[256];
   // blockIdx.x = J (J + 1) / 2 + I
@@ -786,6 +809,8 @@ __global__ void __launch_bounds__(256) k_penrose_norms(Planes<const double> R, i
 // X (n x m) = alpha * A^H, A m x n: X[j][i] = alpha * conj(A[i][j]).
 template <typename T>
 __global__ void __launch_bounds__(256) k_init_x0(Planes<const double> A, int m, int n, double al, Planes<T> X) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double t[4][TILE][TILE + 1];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int r0 = blockIdx.y * TILE, c0 = blockIdx.x * TILE;  // tile of A: rows r0.., cols c0..
@@ -816,6 +841,8 @@ static int col_chunks(int rows, int cols) {
 }
 
 __global__ void k_f32_to_f64(Planes<const float> S, int rows, int cols, Planes<double> D) {
+  pdl_wait();
+  pdl_trigger();
   const long total = (long)rows * cols;
   for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
     const long i = t / cols, j = t % cols;
@@ -824,6 +851,8 @@ __global__ void k_f32_to_f64(Planes<const float> S, int rows, int cols, Planes<d
 }
 
 __global__ void k_f64_to_f32(Planes<const double> S, int rows, int cols, Planes<float> D) {
+  pdl_wait();
+  pdl_trigger();
   const long total = (long)rows * cols;
   for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
     const long i = t / cols, j = t % cols;
@@ -833,6 +862,8 @@ __global__ void k_f64_to_f32(Planes<const double> S, int rows, int cols, Planes<
 
 // D = S, four planes: a block takes 512 columns of a row (two per thread).
 __global__ void __launch_bounds__(256) k_copy_planes(Planes<const double> S, int rows, int cols, Planes<double> D) {
+  pdl_wait();
+  pdl_trigger();
   const int j = (blockIdx.x * 256 + threadIdx.x) * 2;
   if (j >= cols) return;
   for (int i = blockIdx.y; i < rows; i += gridDim.y) {
@@ -865,9 +896,9 @@ cudaError_t launch_combine(const CombineArgs& args, cudaStream_t st) {
   const int groups = combine_groups(a), rows = TROWS * groups;
   dim3 grid((a.cols + 2 * TILE - 1) / (2 * TILE), (a.rows + rows - 1) / rows);
   if (a.f64)
-    k_combine<double><<<grid, 256, 0, st>>>(a, groups);
+    QP_LAUNCH(k_combine<double>, grid, dim3(256), 0, st, a, groups);
   else
-    k_combine<float><<<grid, 256, 0, st>>>(a, groups);
+    QP_LAUNCH(k_combine<float>, grid, dim3(256), 0, st, a, groups);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
@@ -882,9 +913,10 @@ cudaError_t launch_matrix_norms(const Planes<const double>& A, int m, int n, dou
   if (rb > 65535) return cudaErrorInvalidValue;  // 4 million rows
   double *rowpart = scratch, *colpart = scratch + (long)cb * m;
   const Reduce r{colpart + (long)rb * n, out, count};
-  k_matrix_norms<<<dim3(cb, rb), 256, 0, st>>>(A, m, n, rowpart, colpart, r);
+  QP_LAUNCH(k_matrix_norms, dim3(cb, rb), dim3(256), 0, st, A, m, n, rowpart, colpart, r);
   const int row_blocks = (m + 255) / 256;
-  k_norms_finish<<<row_blocks + (n + 255) / 256, 256, 0, st>>>(rowpart, cb, m, colpart, rb, n, row_blocks, r);
+  QP_LAUNCH(k_norms_finish, dim3(row_blocks + (n + 255) / 256), dim3(256), 0, st, rowpart, cb, m, colpart, rb, n,
+            row_blocks, r);
   g_kernel_launches += 2;
   return cudaGetLastError();
 }
@@ -894,9 +926,9 @@ cudaError_t launch_fro2(const Planes<const double>& A, const Planes<const double
   const long tasks = (long)m * ((n + FRO_COLS - 1) / FRO_COLS);
   const int blocks = (int)std::max(1L, std::min<long>(tasks, kFroBlocks));
   if (B)
-    k_fro2<true><<<blocks, FRO_COLS, 0, st>>>(A, *B, m, n, r);
+    QP_LAUNCH(k_fro2<true>, dim3(blocks), dim3(FRO_COLS), 0, st, A, *B, m, n, r);
   else
-    k_fro2<false><<<blocks, FRO_COLS, 0, st>>>(A, A, m, n, r);
+    QP_LAUNCH(k_fro2<false>, dim3(blocks), dim3(FRO_COLS), 0, st, A, A, m, n, r);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
@@ -906,7 +938,7 @@ int penrose_norm_blocks(int n) {
   return t * (t + 1) / 2;
 }
 cudaError_t launch_penrose_norms(const Planes<const double>& R, int n, double sr, const Reduce& r, cudaStream_t st) {
-  k_penrose_norms<<<penrose_norm_blocks(n), TILE * TROWS, 0, st>>>(R, n, sr < 0 ? 1 : 0, r);
+  QP_LAUNCH(k_penrose_norms, dim3(penrose_norm_blocks(n)), dim3(TILE * TROWS), 0, st, R, n, sr < 0 ? 1 : 0, r);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
@@ -915,7 +947,7 @@ template <typename T>
 static cudaError_t init_x0_t(const Planes<const double>& A, int m, int n, double alpha, const Planes<T>& X,
                              cudaStream_t st) {
   dim3 grid((n + TILE - 1) / TILE, (m + TILE - 1) / TILE);
-  k_init_x0<T><<<grid, TILE * TROWS, 0, st>>>(A, m, n, alpha, X);
+  QP_LAUNCH(k_init_x0<T>, grid, dim3(TILE * TROWS), 0, st, A, m, n, alpha, X);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
@@ -931,21 +963,21 @@ cudaError_t launch_init_x0(const Planes<const double>& A, int m, int n, double a
 cudaError_t launch_copy_planes(const Planes<const double>& S, int rows, int cols, const Planes<double>& D,
                                cudaStream_t st) {
   if (rows <= 0 || cols <= 0) return cudaSuccess;
-  k_copy_planes<<<dim3((cols + 511) / 512, std::min(rows, 8192)), 256, 0, st>>>(S, rows, cols, D);
+  QP_LAUNCH(k_copy_planes, dim3((cols + 511) / 512, std::min(rows, 8192)), dim3(256), 0, st, S, rows, cols, D);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
 
 cudaError_t launch_f32_to_f64(const Planes<const float>& src, int rows, int cols, const Planes<double>& dst,
                               cudaStream_t st) {
-  k_f32_to_f64<<<grid_for((long)rows * cols), 256, 0, st>>>(src, rows, cols, dst);
+  QP_LAUNCH(k_f32_to_f64, dim3(grid_for((long)rows * cols)), dim3(256), 0, st, src, rows, cols, dst);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
 
 cudaError_t launch_f64_to_f32(const Planes<const double>& src, int rows, int cols, const Planes<float>& dst,
                               cudaStream_t st) {
-  k_f64_to_f32<<<grid_for((long)rows * cols), 256, 0, st>>>(src, rows, cols, dst);
+  QP_LAUNCH(k_f64_to_f32, dim3(grid_for((long)rows * cols)), dim3(256), 0, st, src, rows, cols, dst);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
@@ -978,11 +1010,11 @@ static cudaError_t slice_t(const SliceArgs& a, const Planes<const T>& P, const P
   }
   if (row_blocks + col_blocks > 0) {
     if (wpr == 4)
-      k_slice_rows<T, 4, I><<<row_blocks + col_blocks, 256, 0, st>>>(P, a.M, a.K, a.eP, a.S, a.p0, a.np, a.za, a.lda,
-                                                                  a.psa, cx);
+      QP_LAUNCH(k_slice_rows<T, 4, I>, dim3(row_blocks + col_blocks), dim3(256), 0, st, P, a.M, a.K, a.eP, a.S, a.p0,
+                a.np, a.za, a.lda, a.psa, cx);
     else
-      k_slice_rows<T, 1, I><<<row_blocks + col_blocks, 256, 0, st>>>(P, a.M, a.K, a.eP, a.S, a.p0, a.np, a.za, a.lda,
-                                                                  a.psa, cx);
+      QP_LAUNCH(k_slice_rows<T, 1, I>, dim3(row_blocks + col_blocks), dim3(256), 0, st, P, a.M, a.K, a.eP, a.S, a.p0,
+                a.np, a.za, a.lda, a.psa, cx);
     ++g_kernel_launches;
     if (cudaError_t err = cudaGetLastError()) return err;
   }
@@ -991,8 +1023,8 @@ static cudaError_t slice_t(const SliceArgs& a, const Planes<const T>& P, const P
     static std::atomic<unsigned long long> attr_done{0};
     if (cudaError_t err = ensure_smem_attr(k_slice_cols<T, I>, smem, attr_done)) return err;
     dim3 grid((a.N + SC_COLS - 1) / SC_COLS, (a.K + SC_ROWS - 1) / SC_ROWS);
-    k_slice_cols<T, I><<<grid, 256, smem, st>>>(Q, a.K, a.N, a.scratch, chunks, a.eQ, a.S, a.p0, a.np, a.zb, a.ldb,
-                                             a.psb);
+    QP_LAUNCH(k_slice_cols<T, I>, grid, dim3(256), smem, st, Q, a.K, a.N, a.scratch, chunks, a.eQ, a.S, a.p0, a.np,
+              a.zb, a.ldb, a.psb);
     ++g_kernel_launches;
   }
   return cudaGetLastError();

@@ -176,6 +176,8 @@ __global__ void __launch_bounds__(ETHREADS, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = tmem_slot;
+  pdl_wait();  // the setup above touches no global memory
+  pdl_trigger();
   int issued = 0;
 
   if (warp == 0) {
@@ -367,9 +369,8 @@ cudaError_t launch_bn(const EmuGemmArgs& a, EParams& P, int nsm, cudaStream_t st
   if (!make_map(&mB, a.B->b, a.K, a.N, a.np * a.S, a.B->ldb, a.B->psb, BN, EBK)) return cudaErrorInvalidValue;
   static std::atomic<unsigned long long> attr_done{0};
   if (cudaError_t e = ensure_smem_attr(k_qgemm_emu<BN>, C::SMEM, attr_done)) return e;
-  k_qgemm_emu<BN><<<std::min(P.items, nsm), ETHREADS, C::SMEM, st>>>(mA, mB, P);
   ++g_kernel_launches;
-  return cudaGetLastError();
+  return launch_pdl(k_qgemm_emu<BN>, dim3((unsigned)std::min(P.items, nsm)), dim3(ETHREADS), C::SMEM, st, mA, mB, P);
 }
 
 }  // namespace

@@ -326,6 +326,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = tmem_slot;
+  pdl_wait();  // the setup above touches no global memory
+  pdl_trigger();
   int issued = 0;
 
   // grouped rasterization: consecutive items walk the component groups of a
@@ -571,9 +573,8 @@ cudaError_t launch_cfg(const TcGemmArgs& a, KParams& P, cudaStream_t st) {
   const int nsm = sm_count();
   if (nsm < 1 || items > 0x7fffffffL) return cudaErrorInvalidValue;
   P.items = (int)items;
-  k_qgemm_tc<C><<<(int)std::min<long>(items, nsm), THREADS, C::SMEM, st>>>(mA, mB, P);
   ++g_kernel_launches;
-  return cudaGetLastError();
+  return launch_pdl(k_qgemm_tc<C>, dim3((unsigned)std::min<long>(items, nsm)), dim3(THREADS), C::SMEM, st, mA, mB, P);
 }
 
 int units_of(const TcGemmArgs& a) { return ((a.k1 + BK - 1) / BK - a.k0 / BK) * a.npairs; }
