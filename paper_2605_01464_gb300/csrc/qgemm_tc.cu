@@ -26,9 +26,10 @@
 // receives the same MMAs in the same order in all of them, so they give
 // bit-identical products.
 //
-// Measured (GB300): single pass 4096^3 1.14 ms = 1930 TFLOP/s and 8192^3 2030
-// (1609 and 1784 with one-lane issue loops, see elect_one); the fused products
-// of a 60 x 512 solve 119 -> about 12 us (all of a small product's epilogue ran
+// Measured (GB300): single pass 4096^3 with FP64 output 1.20 ms = 1838 TFLOP/s
+// (1.14 ms = 1930 with FP32 output; 1609 with one-lane issue loops, see
+// elect_one); the fused products
+// of a 60 x 512 solve 119 -> 18 us (all of a small product's epilogue ran
 // on one SM's four warps), of a 500^2 one 93 -> 45 us.  The 2048^2 solve's
 // fused single-pass products take 216-263 us, their MMAs 157: the component
 // pair's operand traffic (64 bytes per cycle and SM at full rate) and the last
@@ -130,11 +131,13 @@ template <typename T>
 __device__ __forceinline__ void store_piece(T* plane, long ld, int r0, int M, int j0, int N, const float* v) {
   const int lane = threadIdx.x & 31, i = r0 + (lane >> 2), j = j0 + 2 * (lane & 3);
   T* dst = plane + (long)i * ld + j;
+  T w[8];
+  to_master_all<8>(v, w);
 #pragma unroll
   for (int t = 0; t < 8; t += 2) {
     const int k = (t >> 1) & 1, jj = j + 8 * (t >> 2);
     if (i + 8 * k < M && jj < N)
-      store2(dst + 8 * k * ld + 8 * (t >> 2), jj + 1 < N, to_master<T>(v[t]), to_master<T>(v[t + 1]));
+      store2(dst + 8 * k * ld + 8 * (t >> 2), jj + 1 < N, w[t], w[t + 1]);
   }
 }
 
@@ -533,15 +536,20 @@ long shape_items(int sh, int M, int N) {
 // 64-column one, -1 by the time of the busiest SM): a stage costs its MMAs or
 // its operand bytes, whichever is longer (cycles per stage below), an item
 // its stages, and the last item of an SM its epilogue (every item of the
-// four-component shape, which has one accumulator).  Measured where the line lies: 500 x 1000 x 500, 2 terms, 0.059 ms with
-// 64 columns against 0.125 with 128; 1000^3, 3 terms, 0.143 (component pair)
-// against 0.240 (four components) and 0.41 (64 columns); 2048^3 0.173 (four
-// components) against 0.204 and 0.453.
-TcShape tc_shape(int broad, bool fused, bool f64, int M, int N, int units) {
+// four-component shape, which has one accumulator).  Storing the product itself
+// (FP32, or FP64 for the caller) is a short epilogue: with the combine pass's
+// cost there, one-term products took the pair shape and its twice the operand
+// bytes (4096^3 1.37 against 1.20 ms, 2048^3 211 against 188 us).  Measured where
+// the line lies: 500 x 1000 x 500, 2 terms, 0.053 ms with 64 columns against
+// 0.082 with the component pair; 1000^3, 3 terms, 0.150 (component pair) against
+// 0.252 (four components) and 0.36 (64 columns); 1100^3, 1 term, 63 us (four
+// components) against 66; 2048^3, 1 term, 188 against 207 and 435; 2200 x 300 x
+// 2200 72 (component pair) against 101.
+TcShape tc_shape(int broad, bool fused, bool f64, bool plain64, int M, int N, int units) {
   if (broad == 0) return SHAPE_64;
   if (broad == 1) return fused ? SHAPE_PAIR : SHAPE_FULL;
   const double stage[4] = {1950, 1100, 600, 450};
-  const double tail[4] = {!fused ? 12000. : f64 ? 60000. : 45000., f64 ? 24000. : 12000., 5000, 4000};
+  const double tail[4] = {!fused || plain64 ? 12000. : f64 ? 60000. : 45000., f64 ? 24000. : 12000., 5000, 4000};
   const int nsm = std::max(1, sm_count());
   int best = SHAPE_PAIR;
   double tb = 1e300;
@@ -582,7 +590,7 @@ int units_of(const TcGemmArgs& a) { return ((a.k1 + BK - 1) / BK - a.k0 / BK) * 
 }  // namespace
 
 int tc_partial_blocks(const TcGemmArgs& a) {
-  const TcShape sh = tc_shape(a.broad, true, a.epi.f64 != 0, a.M, a.N, units_of(a));
+  const TcShape sh = tc_shape(a.broad, true, a.epi.f64 != 0, false, a.M, a.N, units_of(a));
   return (int)std::min<long>(shape_items(sh, a.M, a.N), std::max(1, sm_count())) * EPI_WARPS;
 }
 
@@ -622,7 +630,7 @@ cudaError_t launch_qgemm_tc(const TcGemmArgs& a, cudaStream_t st) {
   for (int t = 0; t < kEpiAux; t++)
     if (P.E.aux[t] && O.caux[t].kind != CK_ZERO) P.plain64 = 0;
   P.err = a.err;
-  switch (tc_shape(a.broad, P.E.nout > 0, P.E.f64 != 0, a.M, a.N, units_of(a))) {
+  switch (tc_shape(a.broad, P.E.nout > 0, P.E.f64 != 0, P.plain64 != 0, a.M, a.N, units_of(a))) {
     case SHAPE_FULL: return launch_cfg<Cfg<128, 4>>(a, P, st);
     case SHAPE_PAIR: return launch_cfg<Cfg<128, 2>>(a, P, st);
     case SHAPE_64: return launch_cfg<Cfg<64, 1>>(a, P, st);

@@ -54,3 +54,30 @@ def test_fused_epilogue_matches_the_separate_pass(ctx, m, n, method):
         xs.append(x.cpu().numpy())
     ctx.configure(fuse_epilogue=True)
     assert np.linalg.norm(xs[0] - xs[1]) <= 1e-10 * np.linalg.norm(xs[1])
+
+
+@pytest.mark.parametrize("m,k,n", [(2, 1, 7), (130, 1, 150), (1300, 1100, 1150)])
+@pytest.mark.parametrize("broad", ["auto", False, True])
+def test_fp64_output_of_special_values(ctx, m, k, n, broad):
+    # column 0 of A times row 0 of B, all others zero: every entry of plane 0 is
+    # one exact FP32 product (zero, normal, largest, smallest, infinite, NaN)
+    va = torch.tensor([1.0, 0.0, -3.0, 2.0 ** 100, -2.0 ** -100, 1.9921875 * 2.0 ** 127, float("inf"), float("nan")],
+                      dtype=torch.float64, device="cuda")
+    vb = torch.tensor([1.0, -0.5, 2.0 ** -20, 2.0 ** 20, 0.0], dtype=torch.float64, device="cuda")
+    a = torch.zeros(4, m, k, dtype=torch.float64, device="cuda")
+    b = torch.zeros(4, k, n, dtype=torch.float64, device="cuda")
+    a[0, :, 0] = va[torch.arange(m, device="cuda") % 8]
+    b[0, 0, :] = vb[torch.arange(n, device="cuda") % 5]
+    ctx.configure(tc_broad=broad)
+    c = ctx.qgemm(a, b, precision="tc", split_level=1)
+    ctx.configure(tc_broad="auto")
+    e = torch.zeros_like(c)
+    for q in range(4):  # 0 x inf and 0 x NaN of the zero planes are NaN
+        e[q] = (a[0, :, :1] * b[q, :1, :]).float().double()
+    ok = (c == e) | (torch.isnan(c) & torch.isnan(e))
+    # a product below FP32's normal range may come out as zero
+    ok |= (e.abs() < 2.0 ** -126) & (c.abs() < 2.0 ** -126)
+    # one K step adds zeros to an infinity: nothing but it or NaN can come out
+    if k > 1:
+        ok |= ~torch.isfinite(a[0, :, :1]).expand(m, n) & ~torch.isfinite(c[0])
+    assert bool(ok.all())
