@@ -728,8 +728,8 @@ def bench_krylov(args, torch, qpinv):
                     gbs = st["ew_bytes"] / (st["ew_ms"] * 1e-3) / 1e9 if st["ew_ms"] > 0 else None
                     roof = {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s",
                             "frac": gbs / hbm if gbs else None, "traffic": None,
-                            "kernel": "global Gram-Schmidt / update kernels (k_block_dot, k_block_sub, "
-                                      "k_norm_scale, k_basis_add; bytes counted per launch)",
+                            "kernel": "global Gram-Schmidt / update kernels (k_arnoldi, or k_block_dot, "
+                                      "k_block_combine, k_norm_scale; bytes counted per launch)",
                             "ew_ms_per_solve": st["ew_ms"] / steps_prof,
                             "f64_gemm_ms_per_solve": st["f64_gemm_ms"] / steps_prof,
                             "peak_source": "%s hbm_gbs (MEASURED_PEAKS.json)" % src}
@@ -834,11 +834,11 @@ def bench_learned(args, torch, qpinv):
 
 # DRAM bytes (read + write) per issued tensor flop from one ncu capture of
 # the current exact-slice kernel on an 8-slice 2048^3 product
-# (profiles/k_qgemm_emu_2048_slices8.md: 7.46 GB for 36 passes); a launch's
+# (profiles/k_qgemm_emu_2048_slices8.md: 4.28 GB for 18 passes); a launch's
 # traffic is estimated as this times its issued flops.  None where no
 # capture matches the launches the solve makes (the split GEMM's launches
 # carry the fused combine epilogue, the captured one a plain store).
-TRAFFIC_PER_ISSUED_FLOP = {"k_qgemm_emu": 7.4628e9 / (36 * 32 * 2048.0 ** 3),
+TRAFFIC_PER_ISSUED_FLOP = {"k_qgemm_emu": 4.28e9 / (18 * 32 * 2048.0 ** 3),
                            "k_qgemm_tc": None}
 
 
@@ -924,7 +924,7 @@ def main():
                     help="--kernel qgemm: BF16 terms (tc: 1..3) or exact slices (emu: 2..8)")
     ap.add_argument("--gemm-precision", default="tc", choices=["tc", "emu"], help="--kernel qgemm precision")
     ap.add_argument("--emu-pair", default="auto", choices=["auto", "0", "1"],
-                    help="--kernel qgemm: exact-slice products on SM pairs (1) or one SM (0, auto: the default)")
+                    help="--kernel qgemm: accepted, without effect (one exact-slice kernel serves every size)")
     ap.add_argument("--workload", default="dense",
                     choices=["dense", "batched", "rankdef", "learned", "hyper", "cur", "filter", "krylov"],
                     help="dense: one 2048^2 solve per step; batched: 4096 pure-quaternion blocks per step; "

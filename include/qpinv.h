@@ -88,8 +88,9 @@ enum {
   QPINV_PREC_TC = 2,    /* tensor-core products only (FP32-level output) */
   QPINV_PREC_EMU = 3,   /* every product FP64-accurate on the tensor cores: exact 7-bit slices
                            per operand (power-of-two row and column scaling; 8 slices in a
-                           solve, `split_level` = 2..8 in qpinv_qgemm), K-chunked so every FP32
-                           partial sum is exact, accumulated in 64-bit fixed point.  Use it for
+                           solve, `split_level` = 2..8 in qpinv_qgemm), eight real products of digit
+                           sums per quaternion product, K-chunked so every FP32 partial sum is
+                           exact, accumulated in 64-bit fixed point.  Use it for
                            rank-deficient A, whose null-space rounding noise the iteration
                            multiplies by its order each step */
   QPINV_PREC_DF32 = 4   /* reported only (qpinv_result.precision of batched solves): double-FP32
@@ -175,8 +176,7 @@ typedef struct {
 
 typedef struct {
   long long kernel_launches;  /* every kernel of this library launched since the last reset */
-  long long tc_gemm_launches; /* tcgen05 quaternion GEMM launches (BF16 splits; chunked
-                                 exact-slice launches for K beyond the fused kernel's range) */
+  long long tc_gemm_launches; /* tcgen05 quaternion GEMM launches (BF16 splits) */
   double tc_gemm_ms;          /* their summed duration (CUDA events on the launch stream; profile=1) */
   double tc_gemm_flops;       /* algorithmic real flops: 32 per quaternion multiply-add */
   double tc_gemm_flops_issued;/* tensor-core flops issued (split products count each pass) */
@@ -189,7 +189,8 @@ typedef struct {
   long long emu_gemm_launches;/* fused exact-slice (FP64-accurate) tensor-core GEMM launches */
   double emu_gemm_ms;
   double emu_gemm_flops;      /* algorithmic: 32 per quaternion multiply-add */
-  double emu_gemm_flops_issued;/* tensor-core flops issued: S(S+1)/2 slice-pair passes */
+  double emu_gemm_flops_issued;/* tensor-core flops issued: S(S+1)/2 slice-pair passes of
+                                     half the algorithmic flops (8 of 16 real products) */
   long long batched_tile;     /* CTA GEMM tile of the last batched call (see batched_tile) */
   double batched_tune_ms;     /* time spent autotuning batched tiles */
   long long batched_graph_replays; /* batched calls served by replaying a captured CUDA graph */
@@ -381,7 +382,9 @@ int qpinv_global_krylov(qpinv_ctx* ctx, void* stream, int n, int m, const double
  * FP64 arrays (device or host).  precision: QPINV_PREC_FP64 (CUDA-core FP64
  * kernel), QPINV_PREC_TC (tcgen05 kernel on BF16 splits of A and B with
  * `split_level` = 1..3 terms, FP32 accumulation) or QPINV_PREC_EMU (tcgen05,
- * `split_level` = 2..8 exact slices, FP64-accurate for 8).  C must not alias A or B. */
+ * `split_level` = 2..8 exact slices, FP64-accurate for 8).  C must not alias A or B:
+ * device planes are read and written in place.  On an error status from the GPU
+ * (QPINV_E_TIMEOUT, QPINV_E_CUDA) C may be partly written. */
 int qpinv_qgemm(qpinv_ctx* ctx, void* stream, int m, int k, int n, const double* const A[4],
                 long lda, const double* const B[4], long ldb, double* const C[4], long ldc,
                 int precision, int split_level);

@@ -26,14 +26,13 @@
 // receives the same MMAs in the same order in all of them, so they give
 // bit-identical products.
 //
-// Measured (GB300): single pass 4096^3 with FP64 output 1.20 ms = 1838 TFLOP/s
-// (1.14 ms = 1930 with FP32 output; 1609 with one-lane issue loops, see
-// elect_one); the fused products
-// of a 60 x 512 solve 119 -> 18 us (all of a small product's epilogue ran
-// on one SM's four warps), of a 500^2 one 93 -> 45 us.  The 2048^2 solve's
-// fused single-pass products take 216-263 us, their MMAs 157: the component
-// pair's operand traffic (64 bytes per cycle and SM at full rate) and the last
-// item's epilogue are what is left.
+// Measured (GB300): single pass 4096^3 with FP64 output 1.17-1.21 ms = 1813-1875
+// TFLOP/s (1.14 ms = 1930 with FP32 output; 1609 with one-lane issue loops, see
+// elect_one); the fused products of a 60 x 512 solve 119 -> 18 us (all of a small
+// product's epilogue ran on one SM's four warps), of a 500^2 one 93 -> 45 us.
+// The 2048^2 solve's fused single-pass products take 216-263 us, their MMAs 157:
+// the component pair's operand traffic (64 bytes per cycle and SM at full rate)
+// and the last item's epilogue are what is left.
 // Every wait is bounded (2 s of globaltimer); on expiry the kernel records
 // an error code, stops issuing work, drains what it started and frees TMEM.
 #include <cuda.h>
