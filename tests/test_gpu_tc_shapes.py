@@ -81,3 +81,9 @@ def test_fp64_output_of_special_values(ctx, m, k, n, broad):
     if k > 1:
         ok |= ~torch.isfinite(a[0, :, :1]).expand(m, n) & ~torch.isfinite(c[0])
     assert bool(ok.all())
+
+
+@pytest.mark.parametrize("m,k,n", [(700, 90, 650), (1153, 33, 705)])
+def test_clustered_shapes_give_the_same_bits(ctx, m, k, n):
+    # enough items that the 64-column shape runs in clusters, odd tile counts
+    test_shapes_give_the_same_bits(ctx, m, k, n, 2)
