@@ -86,14 +86,37 @@ __device__ __forceinline__ long long to_fixed(float v, int sh) {
   return (b >> 31) ? -F : F;
 }
 
-// Binary exponent e with |v| < 2^e (0 for zero / subnormal), from the bits.
-__device__ __forceinline__ int exp_of(double v) {
-  const int ex = (int)(((unsigned long long)__double_as_longlong(v) >> 52) & 0x7FF);
-  return ex == 0 ? -100000 : ex - 1022;
+// Magnitudes as integers, in the order of the values: a maximum is taken over
+// these, and its exponent once at the end.
+template <typename T>
+struct Bits;
+template <>
+struct Bits<double> {
+  using U = unsigned long long;
+  static constexpr int MANT = 53, BIAS = 1022;
+};
+template <>
+struct Bits<float> {
+  using U = unsigned;
+  static constexpr int MANT = 24, BIAS = 126;
+};
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
 }
-__device__ __forceinline__ int exp_of(float v) {
-  const int ex = (int)((__float_as_uint(v) >> 23) & 0xFF);
-  return ex == 0 ? -100000 : ex - 126;
+__device__ __forceinline__ unsigned abs_bits(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
+
+// Binary exponent e of a slicing with S slices, from the largest magnitude:
+// |v| < 2^e for every v and for every v rounded to 7S bits (-100000 when all are
+// zero or subnormal).  Where 7S bits do not hold the mantissa, half of the last
+// kept bit carries a maximum that rounds up to its power of two into the next
+// exponent, so that no sliced entry reaches 1 in its row's or column's units: the
+// exact-slice GEMM's fixed point has no room for a component of 4K (see emu_plan).
+template <typename T>
+__device__ __forceinline__ int exp_of(typename Bits<T>::U mx, int S) {
+  using B = Bits<T>;
+  const typename B::U half = 7 * S < B::MANT ? (typename B::U)1 << (B::MANT - 1 - 7 * S) : 0;
+  const int ex = (int)((mx + half) >> (B::MANT - 1));
+  return ex == 0 ? -100000 : ex - B::BIAS;
 }
 
 // q 2^e rounded to nearest (ties to even) as a double or float, from the
@@ -136,7 +159,7 @@ __device__ __forceinline__ float i64_scaledf(long long q, int e) {
 
 // Twice the four components from the eight real products of the exact-slice
 // GEMM (see qgemm_emu.cu).  Wrapping arithmetic: a doubled component is below
-// 2^63 in modulus, the partial sums need not be.
+// 2^63 in modulus (emu_plan), the partial sums need not be.
 __device__ __forceinline__ void quad_of(const unsigned long long* p, long long* q) {
   const unsigned long long a = p[4] + p[5], b = p[4] - p[5], c = p[6] + p[7], d = p[6] - p[7];
   q[0] = (long long)(2 * p[1] - a + c);
@@ -483,6 +506,7 @@ template <typename T>
 struct ColExp {
   Planes<const T> A;
   int rows = 0, cols = 0, chunk_rows = 0, colblocks = 0, first = 0x7fffffff;
+  int S = 0;            // slices
   int* part = nullptr;  // [chunk][cols]
 };
 template <typename T>
@@ -490,12 +514,13 @@ __device__ __forceinline__ void col_maxexp_block(const ColExp<T>& cx, int blk, i
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int j = (blk % cx.colblocks) * 32 + tx, ch = blk / cx.colblocks;
   const int r0 = ch * cx.chunk_rows, r1 = min(cx.rows, r0 + cx.chunk_rows);
-  int mx = -100000;
+  typename Bits<T>::U top = 0;
   if (j < cx.cols)
 #pragma unroll 2
     for (int i = r0 + ty; i < r1; i += 8)
 #pragma unroll
-      for (int c = 0; c < 4; c++) mx = max(mx, exp_of(cx.A.p[c * cx.A.ps + (long)i * cx.A.ld + j]));
+      for (int c = 0; c < 4; c++) top = max(top, abs_bits(cx.A.p[c * cx.A.ps + (long)i * cx.A.ld + j]));
+  int mx = exp_of<T>(top, cx.S);
   sh[ty][tx] = mx;
   __syncthreads();
   if (ty == 0 && j < cx.cols) {
@@ -519,13 +544,14 @@ __global__ void __launch_bounds__(256, 2) k_slice_rows(Planes<const T> A, int ro
   const int i = blockIdx.x * (8 / WPR) + warp / WPR, tr = (warp % WPR) * 32 + lane;
   const bool ok = i < rows;
   const T* row = A.p + (long)(ok ? i : 0) * A.ld;
-  int mx = -100000;
+  typename Bits<T>::U top = 0;
   if (ok) {
 #pragma unroll 4
     for (int j = tr; j < cols; j += 32 * WPR)
 #pragma unroll
-      for (int c = 0; c < 4; c++) mx = max(mx, exp_of(row[c * A.ps + j]));
+      for (int c = 0; c < 4; c++) top = max(top, abs_bits(row[c * A.ps + j]));
   }
+  int mx = exp_of<T>(top, S);
   for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if (WPR > 1) {
     if (lane == 0) sh[warp] = mx;
@@ -1000,6 +1026,7 @@ static cudaError_t slice_t(const SliceArgs& a, const Planes<const T>& P, const P
   int col_blocks = 0;
   if (a.zb && a.p0 == 0) {  // the exponents serve every group of products
     cx.A = Q;
+    cx.S = a.S;
     cx.rows = a.K;
     cx.cols = a.N;
     cx.chunk_rows = (a.K + chunks - 1) / chunks;

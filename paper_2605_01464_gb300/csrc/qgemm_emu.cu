@@ -380,7 +380,12 @@ EmuPlan emu_plan(int M, int N, int K, int S) {
   EmuPlan p;
   int lg = 0;
   while ((1L << lg) < 4L * K) lg++;
-  p.F = 62 - lg;  // |product| <= 4K in normalised units: |acc| <= 2^62
+  // A product is at most 4K in normalised units: |acc| <= 2^62.  The combine pass
+  // forms twice a component, which has to stay below 2^63, a component below 4K:
+  // sliced entries are below 1 by at least 2^-7S (2^-53 where 8 slices hold an FP64
+  // mantissa), so twice a component leaves 2^11 units or more for the roundings (a
+  // few hundred) and for what the dropped levels would have subtracted.
+  p.F = 62 - lg;
   const int npairs = (S + 1) / 2;
   const int nsm = std::max(1, emu_sm_count());
   // Tile width and parts by the time of the busiest SM, in units of one
