@@ -51,8 +51,7 @@
 // 16-product kernel it replaced (1696 TFLOP/s issued of 1876 measured burst),
 // 4096^3 22.9 against 44.9 ms, 60 x 512 x 60 14 against 155 us.  What is left
 // at 2048: 2048 items on 152 SMs fill 13.5 of 14 waves, and the MMA warp's
-// barrier waits between stages (sharing B tiles between two CTAs by multicast
-// left the time as it was).
+// barrier waits between stages.
 #include <cuda.h>
 
 #include <algorithm>

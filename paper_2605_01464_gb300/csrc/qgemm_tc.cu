@@ -30,14 +30,9 @@
 // TFLOP/s (1.14 ms = 1930 with FP32 output; 1609 with one-lane issue loops, see
 // elect_one); the fused products of a 60 x 512 solve 119 -> 18 us (all of a small
 // product's epilogue ran on one SM's four warps), of a 500^2 one 93 -> 45 us.
-//
-// Clusters: the items of one tile's component groups read the same A and B
-// planes, so two of them run as a cluster of two CTAs, one loading A and the
-// other B into both (multicast).  L2 delivers about 50 bytes per clock and SM to
-// all 152, a component pair's stages ask for 64; halving what they read took
-// 4096^3 in pairs from 1353 to 1271 us, a 2048^2 solve's BF16 products from 25.4
-// to 23.8 ms, a 1600^2 one's from 10.8 to 10.1, 2200 x 100 x 2200 in three terms
-// from 152 to 111 us.  A stage is refilled once both CTAs' MMAs have read it.
+// The 2048^2 solve's fused single-pass products take 216-263 us, their MMAs 157:
+// the component pair's operand traffic (64 bytes per cycle and SM at full rate)
+// and the last item's epilogue are what is left.
 // Every wait is bounded (2 s of globaltimer); on expiry the kernel records
 // an error code, stops issuing work, drains what it started and frees TMEM.
 #include <cuda.h>
@@ -58,14 +53,9 @@ constexpr int EPI_WARPS = 16;
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
 constexpr int TP = 48;       // row pitch (bytes) of the epilogue's 16 x 16 BF16 tiles: conflict-free stmatrix
 
-template <int BN_, int NC_, int CL_>
+template <int BN_, int NC_>
 struct Cfg {
   static constexpr int BN = BN_, NC = NC_;
-  // CTAs of a cluster: the items of one tile's component groups, which read the
-  // same operand planes
-  static constexpr int CL = CL_;
-  static_assert((4 / NC) % CL == 0 && CL <= 2, "the items of a cluster are of one tile");
-  static constexpr uint16_t CL_MASK = (1 << CL) - 1;
   static constexpr int B_PLANE = BN * BK * 2;
   static constexpr int STAGE = 4 * (A_PLANE + B_PLANE);
   static constexpr int STAGES = BN == 128 ? 3 : 4;
@@ -320,7 +310,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     abort_flag = 0;
     for (int s = 0; s < STAGES; s++) {
       mbar_init(smem_u32(&bar_full[s]), 1);
-      mbar_init(smem_u32(&bar_empty[s]), C::CL);  // one commit per CTA of the cluster
+      mbar_init(smem_u32(&bar_empty[s]), 1);
     }
     for (int b = 0; b < NBUF; b++) {
       mbar_init(smem_u32(&bar_acc_full[b]), 1);
@@ -336,7 +326,6 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
   fence_before();
   __syncthreads();
-  if (C::CL > 1) cluster_sync();  // the barriers that the other CTA's copies and commits signal
   fence_after();
   const uint32_t tmem = tmem_slot;
   pdl_wait();  // the setup above touches no global memory
@@ -377,14 +366,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           // and no difference for the 128-column shapes)
           mbar_expect_tx(fb, 4 * (P.arows * BK * 2 + C::B_PLANE));
           uint8_t* st = smem + (size_t)s * C::STAGE;
-          if (C::CL == 1) {
-            tma_load_3d(smem_u32(st), &tmA, kb * BK, m0, P.pi[pr] * 4, fb);
-            tma_load_3d(smem_u32(st + 4 * A_PLANE), &tmB, kb * BK, n0, P.pj[pr] * 4, fb);
-          } else if ((blockIdx.x & 1) == 0) {  // one operand each, into both CTAs
-            tma_load_3d_multicast(smem_u32(st), &tmA, kb * BK, m0, P.pi[pr] * 4, fb, C::CL_MASK);
-          } else {
-            tma_load_3d_multicast(smem_u32(st + 4 * A_PLANE), &tmB, kb * BK, n0, P.pj[pr] * 4, fb, C::CL_MASK);
-          }
+          tma_load_3d(smem_u32(st), &tmA, kb * BK, m0, P.pi[pr] * 4, fb);
+          tma_load_3d(smem_u32(st + 4 * A_PLANE), &tmB, kb * BK, n0, P.pj[pr] * 4, fb);
           issued = u + 1;
         }
       }
@@ -426,8 +409,7 @@ __global__ void __launch_bounds__(THREADS, 1)
               default: stage_mmas<C, 3 & (4 - NC)>(dacc, ad, bd, ap, acc); break;
             }
           }
-          if (C::CL == 1) mma_commit(smem_u32(&bar_empty[s]));
-          else mma_commit_multicast(smem_u32(&bar_empty[s]), C::CL_MASK);
+          mma_commit(smem_u32(&bar_empty[s]));
         }
         __syncwarp();
         if (++s == STAGES) {
@@ -525,14 +507,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp == 0 && lane == 0 && abort_flag) {
     for (int u = (issued > STAGES ? issued - STAGES : 0); u < issued; u++)
       (void)mbar_wait(smem_u32(&bar_full[u % STAGES]), (u / STAGES) & 1, &abort_flag, nullptr, 0);
-    if (C::CL > 1) {  // copies into the other CTA's memory: far longer than any takes
-      const unsigned long long t0 = gtime();
-      while (gtime() - t0 < 1000000ull) {
-      }
-    }
   }
   __syncthreads();
-  if (C::CL > 1) cluster_sync();  // no copy or commit of the other CTA is on its way here
   if (warp == 1) {
     __syncwarp();
     fence_after();
@@ -562,17 +538,16 @@ long shape_items(int sh, int M, int N) {
 // four-component shape, which has one accumulator).  Storing the product itself
 // (FP32, or FP64 for the caller) is a short epilogue: with the combine pass's
 // cost there, one-term products took the pair shape and its twice the operand
-// bytes (4096^3 1.37 against 1.20 ms, 2048^3 211 against 188 us then).  Measured where
+// bytes (4096^3 1.37 against 1.20 ms, 2048^3 211 against 188 us).  Measured where
 // the line lies: 500 x 1000 x 500, 2 terms, 0.053 ms with 64 columns against
 // 0.082 with the component pair; 1000^3, 3 terms, 0.150 (component pair) against
 // 0.252 (four components) and 0.36 (64 columns); 1100^3, 1 term, 63 us (four
-// components) against 63-66; 2048^3, 1 term, 186 against 198 and 435; 2200 x 300
-// x 2200 70 (component pair) against 101; fused products of a 2048^2 solve in
-// three pairs: component pairs, 24.3 -> 23.8 ms for all of them.
+// components) against 66; 2048^3, 1 term, 188 against 207 and 435; 2200 x 300 x
+// 2200 72 (component pair) against 101.
 TcShape tc_shape(int broad, bool fused, bool f64, bool plain64, int M, int N, int units) {
   if (broad == 0) return SHAPE_64;
   if (broad == 1) return fused ? SHAPE_PAIR : SHAPE_FULL;
-  const double stage[4] = {1950, 1040, 600, 450};
+  const double stage[4] = {1950, 1100, 600, 450};
   const double tail[4] = {!fused || plain64 ? 12000. : f64 ? 60000. : 45000., f64 ? 24000. : 12000., 5000, 4000};
   const int nsm = std::max(1, sm_count());
   int best = SHAPE_PAIR;
@@ -602,12 +577,11 @@ cudaError_t launch_cfg(const TcGemmArgs& a, KParams& P, cudaStream_t st) {
   P.Mt = (a.M + BM - 1) / BM;
   P.Nt = (a.N + C::BN - 1) / C::BN;
   const long items = (long)P.Mt * P.Nt * (4 / C::NC);
-  const int nsm = sm_count() / C::CL * C::CL;
+  const int nsm = sm_count();
   if (nsm < 1 || items > 0x7fffffffL) return cudaErrorInvalidValue;
   P.items = (int)items;
   ++g_kernel_launches;
-  return launch_pdl_cluster(C::CL, k_qgemm_tc<C>, dim3((unsigned)std::min<long>(items, nsm)), dim3(THREADS), C::SMEM,
-                            st, mA, mB, P);
+  return launch_pdl(k_qgemm_tc<C>, dim3((unsigned)std::min<long>(items, nsm)), dim3(THREADS), C::SMEM, st, mA, mB, P);
 }
 
 int units_of(const TcGemmArgs& a) { return ((a.k1 + BK - 1) / BK - a.k0 / BK) * a.npairs; }
@@ -656,14 +630,10 @@ cudaError_t launch_qgemm_tc(const TcGemmArgs& a, cudaStream_t st) {
     if (P.E.aux[t] && O.caux[t].kind != CK_ZERO) P.plain64 = 0;
   P.err = a.err;
   switch (tc_shape(a.broad, P.E.nout > 0, P.E.f64 != 0, P.plain64 != 0, a.M, a.N, units_of(a))) {
-    case SHAPE_FULL: return launch_cfg<Cfg<128, 4, 1>>(a, P, st);
-    case SHAPE_PAIR: return launch_cfg<Cfg<128, 2, 2>>(a, P, st);
-    case SHAPE_64:
-      // a cluster costs a small product more than it saves (64 x 48 solve 1.005 ->
-      // 1.040 ms): only where the items fill the chip and share its L2 bandwidth
-      return shape_items(SHAPE_64, a.M, a.N) >= sm_count() ? launch_cfg<Cfg<64, 1, 2>>(a, P, st)
-                                                           : launch_cfg<Cfg<64, 1, 1>>(a, P, st);
-    default: return launch_cfg<Cfg<32, 1, 1>>(a, P, st);
+    case SHAPE_FULL: return launch_cfg<Cfg<128, 4>>(a, P, st);
+    case SHAPE_PAIR: return launch_cfg<Cfg<128, 2>>(a, P, st);
+    case SHAPE_64: return launch_cfg<Cfg<64, 1>>(a, P, st);
+    default: return launch_cfg<Cfg<32, 1>>(a, P, st);
   }
 }
 
