@@ -399,20 +399,20 @@ __device__ __noinline__ void TcGemm::products(int M, int N, int K, int u0, int w
         for (int d = TS - 1; d >= 0 && ok; d--) {
           for (int k0 = 0; k0 < K && ok; k0 += kc[d], w++) {
             const int b = w & 1;  // FP32 buffer of this chunk, free once chunk w - 2 was drained
-            if (w >= 2 && !mbar_wait(smem_u32(&ts->acc_empty[b]), ((w >> 1) - 1) & 1, &ts->abort_flag, err, 22)) {
-              ok = false;
-              break;
+            if (w >= 2) {
+              (void)mbar_wait(smem_u32(&ts->acc_empty[b]), ((w >> 1) - 1) & 1, &ts->abort_flag, err, 22);
+              if (warp_aborted(&ts->abort_flag)) {
+                ok = false;
+                break;
+              }
             }
             fence_after();
             const uint32_t dacc = ts->tmem + b * 256;
             const int kb0 = k0 / TBK, kb1 = (min(K, k0 + kc[d]) + TBK - 1) / TBK;
             uint32_t acc = 0u;
-            for (int kb = kb0; kb < kb1 && ok; kb++) {
+            for (int kb = kb0; kb < kb1; kb++) {
               for (int s = 0; s <= d; s++) {
-                if (!mbar_wait(smem_u32(&ts->full[st]), ph, &ts->abort_flag, err, 23)) {
-                  ok = false;
-                  break;
-                }
+                (void)mbar_wait(smem_u32(&ts->full[st]), ph, &ts->abort_flag, err, 23);
                 fence_after();
                 const uint32_t ad = a_lo + st * (TSTAGE >> 4), bd = b_lo + st * (TSTAGE >> 4);
                 if (elect_one()) {
@@ -428,7 +428,7 @@ __device__ __noinline__ void TcGemm::products(int M, int N, int K, int u0, int w
                 }
               }
             }
-            if (ok && elect_one()) mma_commit(smem_u32(&ts->acc_full[b]));
+            if (elect_one()) mma_commit(smem_u32(&ts->acc_full[b]));
             __syncwarp();
           }
         }

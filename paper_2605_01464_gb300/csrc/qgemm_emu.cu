@@ -225,18 +225,18 @@ __global__ void __launch_bounds__(ETHREADS, 1)
         const int h = P.h[it.g][li], kc = P.kc[it.g][li];
         for (int c0 = it.k0; c0 < it.k1 && ok; c0 += kc, w++) {
           const int b = w & 1, c1 = min(it.k1, c0 + kc);
-          if (w >= 2 && !mbar_wait(smem_u32(&bar_acc_empty[b]), ((w >> 1) - 1) & 1, &abort_flag, P.err, 12)) {
-            ok = false;
-            break;
-          }
-          fence_after();
-          const uint32_t dlo = tmem + b * C::BUF, dhi = dlo + BN;
-          for (int k = c0; k < c1 && ok; k += EBK) {
-            const int nkk = min(EBK / 16, (c1 - k + 15) / 16);
-            if (!mbar_wait(smem_u32(&bar_full[st]), ph, &abort_flag, P.err, 13)) {
+          if (w >= 2) {
+            (void)mbar_wait(smem_u32(&bar_acc_empty[b]), ((w >> 1) - 1) & 1, &abort_flag, P.err, 12);
+            if (warp_aborted(&abort_flag)) {
               ok = false;
               break;
             }
+          }
+          fence_after();
+          const uint32_t dlo = tmem + b * C::BUF, dhi = dlo + BN;
+          for (int k = c0; k < c1; k += EBK) {
+            const int nkk = min(EBK / 16, (c1 - k + 15) / 16);
+            (void)mbar_wait(smem_u32(&bar_full[st]), ph, &abort_flag, P.err, 13);
             for (int s = 0; s <= h; s++) {
               const int sn = st + 1 == STAGES ? 0 : st + 1;
               const uint32_t phn = st + 1 == STAGES ? ph ^ 1 : ph;
@@ -244,10 +244,7 @@ __global__ void __launch_bounds__(ETHREADS, 1)
               const uint32_t bh = b_lo + (STAGES - 1 - st) * (C::B_TILE >> 4);
               const uint32_t bl = b_lo + (STAGES - 1 - sn) * (C::B_TILE >> 4);
               const uint32_t acc = (k > c0 || s > 0) ? 1u : 0u;
-              if (s < h && !mbar_wait(smem_u32(&bar_full[sn]), phn, &abort_flag, P.err, 13)) {
-                ok = false;
-                break;
-              }
+              if (s < h) (void)mbar_wait(smem_u32(&bar_full[sn]), phn, &abort_flag, P.err, 13);
               fence_after();
               if (elect_one()) {
                 if (s < h && sn != 0) mma_steps<C::IDESC2>(dlo, ad, bl, nkk, acc);
@@ -262,7 +259,7 @@ __global__ void __launch_bounds__(ETHREADS, 1)
               ph = phn;
             }
           }
-          if (ok && elect_one()) mma_commit(smem_u32(&bar_acc_full[b]));
+          if (elect_one()) mma_commit(smem_u32(&bar_acc_full[b]));
           __syncwarp();
         }
       }

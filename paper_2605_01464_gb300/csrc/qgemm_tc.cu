@@ -378,22 +378,18 @@ __global__ void __launch_bounds__(THREADS, 1)
     const uint32_t ap = (uint32_t)(P.arows * BK * 2) >> 4;
     int s = 0, w = 0;
     uint32_t ph = 0;
-    bool ok = true;
-    for (int item = blockIdx.x; item < P.items && ok; item += gridDim.x, w++) {
+    for (int item = blockIdx.x; item < P.items; item += gridDim.x, w++) {
       int m0, n0, c0;
       item_origin(item, m0, n0, c0);
       const int b = w % NBUF;
-      if (w >= NBUF && !mbar_wait(smem_u32(&bar_acc_empty[b]), ((w / NBUF) - 1) & 1, &abort_flag, P.err, 42)) {
-        ok = false;
-        break;
+      if (w >= NBUF) {
+        (void)mbar_wait(smem_u32(&bar_acc_empty[b]), ((w / NBUF) - 1) & 1, &abort_flag, P.err, 42);
+        if (warp_aborted(&abort_flag)) break;
       }
       fence_after();
       const uint32_t dacc = tmem + b * C::ACC;
       for (int x = 0; x < units; x++) {
-        if (!mbar_wait(smem_u32(&bar_full[s]), ph, &abort_flag, P.err, 43)) {
-          ok = false;
-          break;
-        }
+        (void)mbar_wait(smem_u32(&bar_full[s]), ph, &abort_flag, P.err, 43);
         fence_after();
         const uint32_t ad = a_lo + s * (C::STAGE >> 4), bd = b_lo + s * (C::STAGE >> 4), acc = x > 0 ? 1u : 0u;
         if (elect_one()) {
@@ -417,7 +413,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           ph ^= 1;
         }
       }
-      if (ok && elect_one()) mma_commit(smem_u32(&bar_acc_full[b]));
+      if (elect_one()) mma_commit(smem_u32(&bar_acc_full[b]));
       __syncwarp();
     }
   } else {

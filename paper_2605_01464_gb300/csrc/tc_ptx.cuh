@@ -57,6 +57,14 @@ __device__ __forceinline__ bool elect_one() {
 }
 // Bounded wait: false if the abort flag is raised or WAIT_NS elapses (then
 // raises the flag and records `code` in *err).
+//
+// The issuing warps wait with all lanes (one lane's wait in front of the MMAs
+// moves their operands out of the uniform registers, see elect_one: 2048^3 3.5 ->
+// 3.9 ms).  Lanes see the barrier, the flag and the clock at different times, so
+// they must not branch on the answer: those that gave up would leave the others
+// in elect.sync or __syncwarp without limit.  They discard it, go on -- after an
+// abort on operands that may not have arrived, for a result that the host throws
+// away -- and leave together at the next warp_aborted().
 __device__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int code) {
   if (mbar_try(bar, parity)) return true;
   const unsigned long long t0 = gtime();
@@ -71,6 +79,10 @@ __device__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_fla
       }
     }
   }
+}
+// Whether the abort flag is raised: one answer for a converged warp.
+__device__ __forceinline__ bool warp_aborted(const volatile int* abort_flag) {
+  return __any_sync(0xffffffffu, *abort_flag != 0);
 }
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2,
                                             uint32_t bar) {

@@ -21,3 +21,37 @@ def test_no_multicast_loads(name):
     # into several CTAs' shared memory is not to be used
     for line in re.findall(r"cp\.async\.bulk[^;]*;", _code(os.path.join(CSRC, name))):
         assert "multicast" not in line, line
+
+
+def _guards(code, pos):
+    """Heads of the blocks and the statement head that enclose position pos."""
+    heads, depth = [], 0
+    for i in range(pos - 1, -1, -1):
+        if code[i] == "}":
+            depth += 1
+        elif code[i] == "{":
+            if depth == 0:
+                heads.append(code[max(code.rfind(c, 0, i) for c in ";{}") + 1:i])
+            else:
+                depth -= 1
+    return heads + [code[max(code.rfind(c, 0, pos) for c in ";{}") + 1:pos]]
+
+
+@pytest.mark.parametrize("name", ["qgemm_tc.cu", "qgemm_emu.cu", "batched_tc.cu"])
+def test_no_lane_leaves_its_warp_after_a_wait(name):
+    # The answer of a bounded wait is one lane's: lanes that wait together can part
+    # over it (one sees the abort flag, another the barrier), and those that go on
+    # would stay in elect.sync or __syncwarp for ever.  A wait is a single lane's,
+    # or its answer is discarded and the warp asks warp_aborted.
+    code = _code(os.path.join(CSRC, name))
+    waits = [m.start() for m in re.finditer(r"mbar_wait\(", code)]
+    assert len(waits) >= 5
+    for pos in waits:
+        guards = " ".join(_guards(code, pos))
+        single = re.search(r"elect_one\(\)|lane == 0|threadIdx\.x == 0", guards)
+        assert single or code[:pos].rstrip().endswith("(void)"), code[pos:pos + 60]
+    issuer = open(os.path.join(CSRC, name)).read()
+    issuer = issuer[issuer.index("// ---------------- MMA issuer"):]
+    assert "if (warp_aborted(" in issuer[:issuer.index("// ---------------- epilogue")]
+    assert re.search(r"bool warp_aborted\([^)]*\) \{\s*return __any_sync\(0xffffffffu,",
+                     _code(os.path.join(CSRC, "tc_ptx.cuh")))
