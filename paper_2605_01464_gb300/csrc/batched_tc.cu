@@ -74,7 +74,7 @@ constexpr size_t TC_LVL_BYTES = (size_t)TS * 4 * MAXD * MAXD * sizeof(int);
 constexpr size_t TC_SLOT_BYTES = 2 * TC_SLICE_BYTES + TC_LVL_BYTES;
 
 struct TcShared {
-  uint64_t full[TSTAGES], empty[TSTAGES], acc_full[2], acc_empty[2];
+  uint64_t full[TSTAGES], empty[TSTAGES], acc_full[2], acc_empty[2], drain;
   uint32_t tmem;
   int abort_flag;
   int u, w, issued;  // stage uses and chunks so far (mbarrier phases); loads issued
@@ -573,6 +573,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_batched_tc(BatchParams P) {
       mbar_init(smem_u32(&ts.acc_full[b]), TMMA_WARPS);
       mbar_init(smem_u32(&ts.acc_empty[b]), 8);  // one arrival per epilogue warp
     }
+    mbar_init(smem_u32(&ts.drain), TMMA_WARPS);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -615,7 +616,8 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_batched_tc(BatchParams P) {
 
   fence_before();
   __syncthreads();
-  // after an abort: wait (bounded) for the copies this CTA still has in flight
+  // after an abort: wait (bounded) for the MMAs and copies this CTA still has in flight
+  if (warp > 0 && warp < TEPI0 && ts.abort_flag) drain_mmas(smem_u32(&ts.drain));
   if (threadIdx.x == 0 && ts.abort_flag) {
     for (int u = (ts.issued > TSTAGES ? ts.issued - TSTAGES : 0); u < ts.issued; u++)
       (void)mbar_wait(smem_u32(&ts.full[u % TSTAGES]), (u / TSTAGES) & 1, &ts.abort_flag, nullptr, 0);

@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(ETHREADS, 1)
   using C = ECfg<BN>;
   constexpr int STAGES = C::STAGES, CW = C::CW;
   extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t bar_full[STAGES], bar_empty[STAGES], bar_acc_full[2], bar_acc_empty[2];
+  __shared__ uint64_t bar_full[STAGES], bar_empty[STAGES], bar_acc_full[2], bar_acc_empty[2], bar_drain;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
 
@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(ETHREADS, 1)
       mbar_init(smem_u32(&bar_acc_full[b]), 1);
       mbar_init(smem_u32(&bar_acc_empty[b]), EEPI_WARPS);
     }
+    mbar_init(smem_u32(&bar_drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -338,6 +339,7 @@ __global__ void __launch_bounds__(ETHREADS, 1)
 
   fence_before();
   __syncthreads();
+  if (warp == 1 && abort_flag) drain_mmas(smem_u32(&bar_drain));
   if (warp == 0 && lane == 0 && abort_flag) {
     for (int u = (issued > STAGES ? issued - STAGES : 0); u < issued; u++)
       (void)mbar_wait(smem_u32(&bar_full[u % STAGES]), (u / STAGES) & 1, &abort_flag, nullptr, 0);

@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                const __grid_constant__ KParams P) {
   constexpr int STAGES = C::STAGES, BN = C::BN, NC = C::NC, NBUF = C::NBUF;
   extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t bar_full[STAGES], bar_empty[STAGES], bar_acc_full[NBUF], bar_acc_empty[NBUF];
+  __shared__ uint64_t bar_full[STAGES], bar_empty[STAGES], bar_acc_full[NBUF], bar_acc_empty[NBUF], bar_drain;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
   __shared__ double red_sh[32];
@@ -316,6 +316,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       mbar_init(smem_u32(&bar_acc_full[b]), 1);
       mbar_init(smem_u32(&bar_acc_empty[b]), EPI_WARPS);  // one arrival per epilogue warp
     }
+    mbar_init(smem_u32(&bar_drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -500,6 +501,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   fence_before();
   __syncthreads();
   if (P.E.red.partials) reduce_last_block<3>(P.E.red, (long)gridDim.x * EPI_WARPS, red_sh);
+  if (warp == 1 && abort_flag) drain_mmas(smem_u32(&bar_drain));
   if (warp == 0 && lane == 0 && abort_flag) {
     for (int u = (issued > STAGES ? issued - STAGES : 0); u < issued; u++)
       (void)mbar_wait(smem_u32(&bar_full[u % STAGES]), (u / STAGES) & 1, &abort_flag, nullptr, 0);

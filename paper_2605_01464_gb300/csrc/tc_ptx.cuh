@@ -118,6 +118,17 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                : "memory");
 }
+// After an abort, by every issuing warp before TMEM is freed: the MMAs that the
+// warp's elected lane issued have completed (normally the epilogue has seen that).
+// `bar` counts one arrival per issuing warp and is used for nothing else; bounded.
+__device__ __forceinline__ void drain_mmas(uint32_t bar) {
+  if (elect_one()) {
+    mma_commit(bar);
+    for (const unsigned long long t0 = gtime(); !mbar_try(bar, 0) && gtime() - t0 < WAIT_NS;) {
+    }
+  }
+  __syncwarp();
+}
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 

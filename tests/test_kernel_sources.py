@@ -55,3 +55,15 @@ def test_no_lane_leaves_its_warp_after_a_wait(name):
     assert "if (warp_aborted(" in issuer[:issuer.index("// ---------------- epilogue")]
     assert re.search(r"bool warp_aborted\([^)]*\) \{\s*return __any_sync\(0xffffffffu,",
                      _code(os.path.join(CSRC, "tc_ptx.cuh")))
+
+
+@pytest.mark.parametrize("name", ["qgemm_tc.cu", "qgemm_emu.cu", "batched_tc.cu"])
+def test_tmem_is_freed_after_the_mmas(name):
+    # A CTA that gives up may still have MMAs in flight, and their TMEM columns go
+    # to the SM's next CTA: between the last block barrier of the roles and the
+    # deallocation, the issuing warps wait for them.
+    code = _code(os.path.join(CSRC, name))
+    end = code[:code.index("tcgen05.dealloc")]
+    m = re.search(r"abort_flag\) drain_mmas\(", end)
+    assert m and "__syncthreads();" in end[m.end():]
+    assert end[:m.start()].rfind("__syncthreads();") > end.rfind("tcgen05.alloc")
