@@ -92,6 +92,12 @@ struct qpinv_ctx {
   unsigned int* d_count = nullptr;  // in the status block
   double* d_red = nullptr;          // in the status block: kRedSums sums
   double* h_pin = nullptr;  // pinned host scalars
+  // Exact slices of all eight products of an operand take twice the memory of four:
+  // when an allocation of a call fails, what it holds of them is given back and the
+  // rest of the call works on four products at a time.
+  bool narrow_slices = false;  // of the current call
+  bool slices_pinned = false;  // SlicePin
+  unsigned slices_epoch = 0;   // counts the times they were given back
   cudaStream_t st = nullptr;
   bool trace = false;
   std::vector<float> alpha_w;  // learned-alpha network (empty: untrained)
@@ -128,14 +134,44 @@ void ck(qpinv_ctx* c, cudaError_t e, const char* what) {
   if (e != cudaSuccess) throw QpError{QPINV_E_CUDA, std::string(what) + ": " + cudaGetErrorString(e)};
 }
 
+// Gives back the slice buffers of exact-slice products (they hold nothing that a
+// later product needs; the slices kept of A are made again).
+bool drop_slices(qpinv_ctx* c) {
+  bool any = false;
+  for (const char* name : {"emu.za", "emu.zb", "emu.cacheA.z"}) {
+    const auto it = c->bufs.find(name);
+    if (it == c->bufs.end() || !it->second.p) continue;
+    cudaFree(it->second.p);  // waits for the kernels that read it
+    it->second = DevBuf();
+    any = true;
+  }
+  c->narrow_slices = true;
+  ++c->slices_epoch;
+  return any;
+}
+
+// While the slice buffers are being asked for: another one's failure must not
+// give back the first.
+struct SlicePin {
+  qpinv_ctx* c;
+  explicit SlicePin(qpinv_ctx* ctx) : c(ctx) { c->slices_pinned = true; }
+  ~SlicePin() { c->slices_pinned = false; }
+};
+
+bool try_alloc(DevBuf& b, size_t bytes) {
+  if (cudaMalloc(&b.p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  b.p = nullptr;
+  return false;
+}
+
 void* buf(qpinv_ctx* c, const std::string& name, size_t bytes) {
   DevBuf& b = c->bufs[name];
   if (b.bytes < bytes) {
     if (b.p) cudaFree(b.p);
     b.p = nullptr;
     b.bytes = 0;
-    if (cudaMalloc(&b.p, bytes) != cudaSuccess) {
-      cudaGetLastError();
+    if (!try_alloc(b, bytes) && (c->slices_pinned || !drop_slices(c) || !try_alloc(b, bytes))) {
       throw QpError{QPINV_E_NOMEM, "cudaMalloc of " + std::to_string(bytes) + " bytes for " + name + " failed"};
     }
     b.bytes = bytes;
@@ -314,6 +350,7 @@ struct Solver {
   // precision they were made for (form -1: none yet).
   int acache_form = -1, acache_S = 0;
   bool acache_dbl = false;
+  unsigned acache_epoch = 0;  // of the slice buffers (qpinv_ctx::slices_epoch)
   long long gemms = 0;
   QMat A, X[2];
   int cur = 0;
@@ -479,7 +516,6 @@ struct Solver {
     int* eP = (int*)buf(c, pA ? "emu.cacheA.e" : "emu.eP", sizeof(int) * (size_t)M + 64);
     int* eQ = (int*)buf(c, qA ? "emu.cacheA.e" : "emu.eQ", sizeof(int) * (size_t)N + 64);
     int* eS = (int*)buf(c, "emu.eS", sizeof(int) * (size_t)COL_SCRATCH(N) + 64);
-    const char* zname[2] = {pA ? "emu.cacheA.z" : "emu.za", qA ? "emu.cacheA.z" : "emu.zb"};
     EmuGemmArgs g;
     g.M = M;
     g.N = N;
@@ -495,18 +531,26 @@ struct Solver {
     za.lda = zb.ldb = rup64(K);
     za.psa = (long)M * za.lda;
     zb.psb = (long)N * zb.ldb;
-    // all eight combinations at once; four at a time when they do not fit
-    int np = 8;
-    try {
-      za.a = (bf16*)buf(c, zname[0], sizeof(bf16) * 8 * S * (size_t)za.psa + 64);
-      zb.b = (bf16*)buf(c, zname[1], sizeof(bf16) * 8 * S * (size_t)zb.psb + 64);
-    } catch (const QpError&) {
-      np = 4;
-      acache_form = -1;
-      za.a = (bf16*)buf(c, zname[0], sizeof(bf16) * 4 * S * (size_t)za.psa + 64);
-      zb.b = (bf16*)buf(c, zname[1], sizeof(bf16) * 4 * S * (size_t)zb.psb + 64);
+    // All eight combinations at once, A's kept; four at a time, none kept, when they
+    // do not fit.
+    auto slices = [&](int count, bool keep) {
+      za.a = (bf16*)buf(c, keep && pA ? "emu.cacheA.z" : "emu.za", sizeof(bf16) * count * S * (size_t)za.psa + 64);
+      zb.b = (bf16*)buf(c, keep && qA ? "emu.cacheA.z" : "emu.zb", sizeof(bf16) * count * S * (size_t)zb.psb + 64);
+    };
+    int np = c->narrow_slices ? 4 : 8;
+    {
+      const SlicePin pin(c);
+      try {
+        slices(np, np == 8);
+      } catch (const QpError&) {
+        if (np == 4) throw;
+        drop_slices(c);
+        np = 4;
+        slices(np, false);
+      }
     }
-    const bool hit = np == 8 && (pA || qA) && acache_form == (pA ? 0 : 1) && acache_S == S && acache_dbl == dbl;
+    const bool hit = np == 8 && (pA || qA) && acache_form == (pA ? 0 : 1) && acache_S == S && acache_dbl == dbl &&
+                     acache_epoch == c->slices_epoch;
     const bool skipP = pA && hit, skipQ = qA && hit;
     g.A = &za;
     g.B = &zb;
@@ -538,6 +582,7 @@ struct Solver {
       acache_form = np == 8 ? (pA ? 0 : 1) : -1;
       acache_S = S;
       acache_dbl = dbl;
+      acache_epoch = c->slices_epoch;
     }
     return Acc{g.C64, ACC_Q8, g.ld64, g.ps64, eP, eQ, plan.F + 1, plan.nparts};
   }
@@ -1294,6 +1339,7 @@ int qpinv_solve(qpinv_ctx* c, void* stream, int m, int n, const double* const A[
   const auto t_start = std::chrono::steady_clock::now();
   DeviceGuard g(c->device);
   c->st = (cudaStream_t)stream;
+  c->narrow_slices = false;
   const qpinv_options& o = c->opt;
   qpinv_result res;
   memset(&res, 0, sizeof(res));
@@ -1677,6 +1723,7 @@ int qpinv_qgemm(qpinv_ctx* c, void* stream, int m, int k, int n, const double* c
     return fail(c, QPINV_E_INVALID, "invalid argument");
   DeviceGuard g(c->device);
   c->st = (cudaStream_t)stream;
+  c->narrow_slices = false;
   try {
     if (precision != QPINV_PREC_FP64 && !tc_supported())
       return fail(c, QPINV_E_UNSUPPORTED, "tcgen05 path needs an sm_103 device");
@@ -1738,6 +1785,7 @@ int qpinv_penrose(qpinv_ctx* c, void* stream, int m, int n, const double* const 
     return fail(c, QPINV_E_INVALID, "invalid argument");
   DeviceGuard g(c->device);
   c->st = (cudaStream_t)stream;
+  c->narrow_slices = false;
   try {
     const int mode = c->opt.precision == QPINV_PREC_FP64 ? PM_F64 : PM_EMU;
     if (mode == PM_EMU && !tc_supported()) return fail(c, QPINV_E_UNSUPPORTED, "tcgen05 path needs an sm_103 device");
@@ -2161,6 +2209,7 @@ int qpinv_solve_batched(qpinv_ctx* c, void* stream, int batch, const int* m, con
   const auto t_start = std::chrono::steady_clock::now();
   DeviceGuard g(c->device);
   c->st = (cudaStream_t)stream;
+  c->narrow_slices = false;
   try {
     int nsm = 0;
     ck(c, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device), "device attribute");
@@ -2302,6 +2351,7 @@ int qpinv_alpha_features(qpinv_ctx* c, void* stream, int m, int n, const double*
   if (m <= 0 || n <= 0 || lda < n || !planes_ok(A) || !feat) return fail(c, QPINV_E_INVALID, "invalid argument");
   DeviceGuard g(c->device);
   c->st = (cudaStream_t)stream;
+  c->narrow_slices = false;
   try {
     QMat a = mat(c, "A", m, n, MST_F, false, false);
     a.d = input_planes(c, A, lda, m, n, "A");
@@ -2337,6 +2387,7 @@ int qpinv_alpha_gradient(qpinv_ctx* c, void* stream, int count, const float* fea
     return c ? fail(c, QPINV_E_INVALID, "invalid argument or untrained network") : QPINV_E_INVALID;
   DeviceGuard g(c->device);
   c->st = (cudaStream_t)stream;
+  c->narrow_slices = false;
   try {
     const int NW = alpha_nweights(), NT = alpha_ntrain();
     float* dW = (float*)buf(c, "alpha.W", sizeof(float) * NW);
@@ -2366,6 +2417,7 @@ int qpinv_alpha_train(qpinv_ctx* c, void* stream, int count, const float* feat, 
     return c ? fail(c, QPINV_E_INVALID, "invalid argument") : QPINV_E_INVALID;
   DeviceGuard g(c->device);
   c->st = (cudaStream_t)stream;
+  c->narrow_slices = false;
   try {
     const int NW = alpha_nweights(), NT = alpha_ntrain();
     std::vector<float> W(NW);
@@ -2438,6 +2490,7 @@ int qpinv_alpha_predict(qpinv_ctx* c, void* stream, const float* feat, double* y
     return c ? fail(c, QPINV_E_INVALID, "invalid argument or untrained network") : QPINV_E_INVALID;
   DeviceGuard g(c->device);
   c->st = (cudaStream_t)stream;
+  c->narrow_slices = false;
   try {
     *y = predict_one(c, feat);
   } catch (const QpError& e) {
