@@ -11,6 +11,8 @@
 // of the 152 SMs (1.1 ms, 0.36 at the pipe's rate) and a 1000-row one padded
 // 2.4 % per side.  The tiles' operand traffic (512 bytes per k) stays far below
 // what L2 delivers in the 2048 cycles their FMAs take.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace qp {
@@ -65,16 +67,17 @@ __global__ void __launch_bounds__(BM * BN) k_qgemm_f64(int M, int K, int N, Plan
 cudaError_t launch_qgemm_f64(int M, int K, int N, const Planes<const double>& A, const Planes<const double>& B,
                              const Planes<double>& C, cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  // rows in slabs: the grid's y extent is limited to 65535 blocks
-  dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
+  // rows in slabs: the grid's y extent is limited to 65535 blocks (64-bit row
+  // counter: the last slab may end at the largest int)
+  const dim3 grid((unsigned)(((long)N + BN - 1) / BN), (unsigned)(((long)M + BM - 1) / BM));
   if (grid.y > 65535) {
-    constexpr int slab = 65535 * BM;
-    for (int i = 0; i < M; i += slab) {
+    constexpr long slab = 65535L * BM;
+    for (long i = 0; i < M; i += slab) {
       Planes<const double> a = A;
       Planes<double> c = C;
-      a.p += (long)i * A.ld;
-      c.p += (long)i * C.ld;
-      const cudaError_t e = launch_qgemm_f64(M - i < slab ? M - i : slab, K, N, a, B, c, st);
+      a.p += i * A.ld;
+      c.p += i * C.ld;
+      const cudaError_t e = launch_qgemm_f64((int)std::min(M - i, slab), K, N, a, B, c, st);
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
