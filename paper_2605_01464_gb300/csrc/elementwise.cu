@@ -642,7 +642,9 @@ __global__ void __launch_bounds__(256) k_matrix_norms(Planes<const double> A, in
   __shared__ double mod[MN_ROWS][MN_COLS + 1];
   __shared__ double sh[256];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int j = blockIdx.x * MN_COLS + tx, r0 = blockIdx.y * MN_ROWS;
+  // tiles in one dimension, the columns' first: a grid's y extent is limited to 65535
+  const int cb = (n + MN_COLS - 1) / MN_COLS, bx = blockIdx.x % cb, by = blockIdx.x / cb;
+  const int j = bx * MN_COLS + tx, r0 = by * MN_ROWS;
   double s = 0.0, col = 0.0;
   int bad = 0;
 #pragma unroll 2
@@ -664,7 +666,7 @@ __global__ void __launch_bounds__(256) k_matrix_norms(Planes<const double> A, in
   const double t0 = block_sum(s, sh);
   const double t1 = block_count(bad, sh);
   if (threadIdx.x == 0) {
-    double* p = r.partials + 2 * ((long)blockIdx.y * gridDim.x + blockIdx.x);
+    double* p = r.partials + 2 * (long)blockIdx.x;
     p[0] = t0;
     p[1] = t1;
   }
@@ -674,15 +676,15 @@ __global__ void __launch_bounds__(256) k_matrix_norms(Planes<const double> A, in
   if (ty == 0 && j < n) {
 #pragma unroll
     for (int k = 1; k < 8; k++) col += sh[tx + 32 * k];
-    colpart[(long)blockIdx.y * n + j] = col;
+    colpart[(long)by * n + j] = col;
   }
   if (threadIdx.x >= 64 && threadIdx.x < 64 + MN_ROWS) {
     const int il = threadIdx.x - 64;
     double t = 0.0;
     for (int k = 0; k < MN_COLS; k++) t += mod[il][k];
-    if (r0 + il < m) rowpart[(long)blockIdx.x * m + r0 + il] = t;
+    if (r0 + il < m) rowpart[(long)bx * m + r0 + il] = t;
   }
-  reduce_last_block<2>(r, (long)gridDim.x * gridDim.y, sh);
+  reduce_last_block<2>(r, gridDim.x, sh);
 }
 
 // The largest row sum and column sum from the partials (summed in block
@@ -936,10 +938,10 @@ long norms_scratch(int m, int n) {  // row and column partials, block partials o
 cudaError_t launch_matrix_norms(const Planes<const double>& A, int m, int n, double* scratch, double* out,
                                 unsigned int* count, cudaStream_t st) {
   const int cb = (n + MN_COLS - 1) / MN_COLS, rb = (m + MN_ROWS - 1) / MN_ROWS;
-  if (rb > 65535) return cudaErrorInvalidValue;  // 4 million rows
+  if ((long)cb * rb > 0x7fffffffL) return cudaErrorInvalidValue;  // 2^42 entries
   double *rowpart = scratch, *colpart = scratch + (long)cb * m;
   const Reduce r{colpart + (long)rb * n, out, count};
-  QP_LAUNCH(k_matrix_norms, dim3(cb, rb), dim3(256), 0, st, A, m, n, rowpart, colpart, r);
+  QP_LAUNCH(k_matrix_norms, dim3(cb * rb), dim3(256), 0, st, A, m, n, rowpart, colpart, r);
   const int row_blocks = (m + 255) / 256;
   QP_LAUNCH(k_norms_finish, dim3(row_blocks + (n + 255) / 256), dim3(256), 0, st, rowpart, cb, m, colpart, rb, n,
             row_blocks, r);
