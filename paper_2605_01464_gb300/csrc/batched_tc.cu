@@ -154,12 +154,10 @@ __device__ __forceinline__ void slice8(bf16* base, long lstride, const dfv* v, f
 }
 
 // The 16 signed MMAs of one stage (BK / 16 steps) into components C0, C0 + 1.
-constexpr uint32_t TDESC_HI = ((8 * TSWB) >> 4) | (1u << 14) | (4u << 29);
-__device__ __forceinline__ uint32_t tdesc_lo(uint32_t addr) { return ((addr & 0x3FFFFu) >> 4) | (1u << 16); }
 template <int C0>
 __device__ __forceinline__ void tstage_mmas(uint32_t d, uint32_t ad, uint32_t bd, uint32_t acc) {
   constexpr uint32_t NEG_A = 1u << 13;
-  const uint64_t hi = (uint64_t)TDESC_HI << 32;
+  constexpr uint64_t hi = desc_hi(TSWB);
 #pragma unroll
   for (int kk = 0; kk < TBK / 16; kk++)
 #pragma unroll
@@ -391,7 +389,7 @@ __device__ __noinline__ void TcGemm::products(int M, int N, int K, int u0, int w
       // ---------------- MMA issuers: warp 1 components 0, 1; warp 2 components 2, 3 ----------------
       // warp-uniform loops, one elected lane issues (see elect_one)
       const bool lo = warp == 1;
-      const uint32_t a_lo = tdesc_lo(smem_u32(smem)), b_lo = tdesc_lo(smem_u32(smem + 4 * TA_PLANE));
+      const uint32_t a_lo = desc_lo(smem_u32(smem)), b_lo = desc_lo(smem_u32(smem + 4 * TA_PLANE));
       int w = w0, st = u0 % TSTAGES;
       uint32_t ph = (uint32_t)(u0 / TSTAGES) & 1u;
       bool ok = true;

@@ -120,15 +120,11 @@ __device__ __forceinline__ EItem item_of(const EParams& P, int item) {
   return it;
 }
 
-// Descriptors of 128-byte-swizzled K-major tiles: the upper word is the same
-// for all, the lower one holds the address / 16 (see smem_desc_sw).
-__device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return ((addr & 0x3FFFFu) >> 4) | (1u << 16); }
-constexpr uint32_t DESC_HI = ((8 * 128) >> 4) | (1u << 14) | (2u << 29);
 // nkk MMAs of K = 16 along one stage (32 bytes of the swizzle row each); the
 // first accumulates if acc, the others always.
 template <uint32_t IDESC>
 __device__ __forceinline__ void mma_steps(uint32_t d, uint32_t ad, uint32_t bd, int nkk, uint32_t acc) {
-  const uint64_t hi = (uint64_t)DESC_HI << 32;
+  constexpr uint64_t hi = desc_hi(2 * EBK);
   if (nkk == EBK / 16) {
 #pragma unroll
     for (int kk = 0; kk < EBK / 16; kk++)

@@ -86,8 +86,6 @@ struct KParams {
   int* err;
 };
 
-__device__ __forceinline__ bool al16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
-
 // Two adjacent entries (x, y) of a row; `two`: y is inside the matrix.
 __device__ __forceinline__ void load2(const float* p, bool two, float* u) {
   if (two && (reinterpret_cast<uintptr_t>(p) & 7) == 0) {
@@ -272,12 +270,10 @@ __device__ __forceinline__ void epi_piece(const EpiArgs& E, int c, int r0, int M
 // the upper word is the same for all tiles, the lower one is an address / 16;
 // ap = distance of the A planes / 16.  With fewer than 128 rows of A the MMAs
 // read on into the next plane: those accumulator rows are not used.
-constexpr uint32_t DESC_HI = ((8 * 64) >> 4) | (1u << 14) | (4u << 29);
-__device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return ((addr & 0x3FFFFu) >> 4) | (1u << 16); }
 template <class C, int C0>
 __device__ __forceinline__ void stage_mmas(uint32_t d, uint32_t ad, uint32_t bd, uint32_t ap, uint32_t acc) {
   constexpr uint32_t NEG_A = 1u << 13;
-  const uint64_t hi = (uint64_t)DESC_HI << 32;
+  constexpr uint64_t hi = desc_hi(2 * BK);
 #pragma unroll
   for (int kk = 0; kk < BK / 16; kk++)
 #pragma unroll

@@ -92,13 +92,12 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 // Shared-memory matrix descriptor: K-major, rows of `swb` swizzled bytes
-// (64 or 128), 8-row groups 8 * swb bytes apart.
-template <int SWB>
-__device__ __forceinline__ uint64_t smem_desc_sw(uint32_t addr) {
-  constexpr unsigned long long layout = SWB == 128 ? 2ull : 4ull;
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)((8 * SWB) >> 4) << 32) |
-         ((uint64_t)1 << 46) | (layout << 61);
+// (64 or 128), 8-row groups 8 * swb bytes apart.  The upper word is the same for
+// every tile of a layout, the lower one holds the address / 16.
+__host__ __device__ constexpr uint64_t desc_hi(int swb) {
+  return (uint64_t)(((8 * swb) >> 4) | (1u << 14) | ((swb == 128 ? 2u : 4u) << 29)) << 32;
 }
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return ((addr & 0x3FFFFu) >> 4) | (1u << 16); }
 
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate) {
@@ -132,35 +131,7 @@ __device__ __forceinline__ void drain_mmas(uint32_t bar) {
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int t = 0; t < 32; t++) v[t] = __uint_as_float(r[t]);
-}
-
 // 32 lanes x 16 consecutive columns (one row of 16 values per thread).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int t = 0; t < 16; t++) v[t] = __uint_as_float(r[t]);
-}
 __device__ __forceinline__ void tmem_ld16u(uint32_t taddr, uint32_t* r) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
@@ -200,19 +171,6 @@ __device__ __forceinline__ uint4 ld_shared16(uint32_t addr) {
   return v;
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// Epilogue row writer: lane j handles column j of up to 32 consecutive rows
-// (stride ld) of a transposed 32 x 33 shared-memory block `st` (already offset
-// by the lane).  All loads are issued before any store so that the 32 row
-// accesses of a lane are in flight together.
-__device__ __forceinline__ void store_rows32(float* __restrict__ dst, long ld, int nrow,
-                                             const float* __restrict__ st) {
-  float g[32];
-#pragma unroll
-  for (int r = 0; r < 32; r++) g[r] = st[r * 33];
-#pragma unroll
-  for (int r = 0; r < 32; r++)
-    if (r < nrow) dst[(long)r * ld] = g[r];
-}
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
