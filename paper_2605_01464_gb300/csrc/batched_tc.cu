@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_batched_tc(BatchParams P) {
   if (warp > 0 && warp < TEPI0 && ts.abort_flag) drain_mmas(smem_u32(&ts.drain));
   if (threadIdx.x == 0 && ts.abort_flag) {
     for (int u = (ts.issued > TSTAGES ? ts.issued - TSTAGES : 0); u < ts.issued; u++)
-      (void)mbar_wait(smem_u32(&ts.full[u % TSTAGES]), (u / TSTAGES) & 1, &ts.abort_flag, nullptr, 0);
+      drain_wait(smem_u32(&ts.full[u % TSTAGES]), (u / TSTAGES) & 1);
   }
   __syncthreads();
   if (warp == 1) {

@@ -215,20 +215,13 @@ __global__ void __launch_bounds__(ETHREADS, 1)
     const uint32_t a_lo = desc_lo(smem_u32(smem)), b_lo = desc_lo(smem_u32(smemB));
     int w = 0, st = 0;
     uint32_t ph = 0;  // parity of stage st's current fill
-    bool ok = true;
-    for (int item = blockIdx.x; item < P.items && ok; item += gridDim.x) {
+    for (int item = blockIdx.x; item < P.items; item += gridDim.x) {
       const EItem it = item_of<BN>(P, item);
-      for (int li = 0; li < P.np[it.g] && ok; li++) {
+      for (int li = 0; li < P.np[it.g]; li++) {
         const int h = P.h[it.g][li], kc = P.kc[it.g][li];
-        for (int c0 = it.k0; c0 < it.k1 && ok; c0 += kc, w++) {
+        for (int c0 = it.k0; c0 < it.k1; c0 += kc, w++) {
           const int b = w & 1, c1 = min(it.k1, c0 + kc);
-          if (w >= 2) {
-            (void)mbar_wait(smem_u32(&bar_acc_empty[b]), ((w >> 1) - 1) & 1, &abort_flag, P.err, 12);
-            if (warp_aborted(&abort_flag)) {
-              ok = false;
-              break;
-            }
-          }
+          if (w >= 2) (void)mbar_wait(smem_u32(&bar_acc_empty[b]), ((w >> 1) - 1) & 1, &abort_flag, P.err, 12);
           fence_after();
           const uint32_t dlo = tmem + b * C::BUF, dhi = dlo + BN;
           for (int k = c0; k < c1; k += EBK) {
@@ -260,6 +253,8 @@ __global__ void __launch_bounds__(ETHREADS, 1)
           __syncwarp();
         }
       }
+      // here: at every chunk 2048^3 takes 2.94 ms for 2.92, at the item's start 2.97
+      if (warp_aborted(&abort_flag)) break;
     }
   } else {
     // ---------------- epilogue: exact FP32 chunk sums -> 64-bit integers in registers ----------------
@@ -338,7 +333,7 @@ __global__ void __launch_bounds__(ETHREADS, 1)
   if (warp == 1 && abort_flag) drain_mmas(smem_u32(&bar_drain));
   if (warp == 0 && lane == 0 && abort_flag) {
     for (int u = (issued > STAGES ? issued - STAGES : 0); u < issued; u++)
-      (void)mbar_wait(smem_u32(&bar_full[u % STAGES]), (u / STAGES) & 1, &abort_flag, nullptr, 0);
+      drain_wait(smem_u32(&bar_full[u % STAGES]), (u / STAGES) & 1);
   }
   __syncthreads();
   if (warp == 1) {

@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp == 1 && abort_flag) drain_mmas(smem_u32(&bar_drain));
   if (warp == 0 && lane == 0 && abort_flag) {
     for (int u = (issued > STAGES ? issued - STAGES : 0); u < issued; u++)
-      (void)mbar_wait(smem_u32(&bar_full[u % STAGES]), (u / STAGES) & 1, &abort_flag, nullptr, 0);
+      drain_wait(smem_u32(&bar_full[u % STAGES]), (u / STAGES) & 1);
   }
   __syncthreads();
   if (warp == 1) {

@@ -70,9 +70,9 @@ __device__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_fla
   const unsigned long long t0 = gtime();
   for (unsigned it = 1;; ++it) {
     if (mbar_try(bar, parity)) return true;
-    if ((it & 255u) == 0) {
+    if ((it & 15u) == 0) {
       if (*abort_flag) return false;
-      if (gtime() - t0 > WAIT_NS) {
+      if ((it & 255u) == 0 && gtime() - t0 > WAIT_NS) {
         *abort_flag = 1;
         if (err) atomicCAS(err, 0, code);
         return false;
@@ -117,14 +117,20 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                : "memory");
 }
-// After an abort, by every issuing warp before TMEM is freed: the MMAs that the
-// warp's elected lane issued have completed (normally the epilogue has seen that).
-// `bar` counts one arrival per issuing warp and is used for nothing else; bounded.
+// After an abort: what the CTA started has to end before it frees TMEM and leaves
+// (normally the later roles have seen that).  One lane; bounded by the clock alone,
+// far longer than a copy or an MMA takes.
+constexpr unsigned long long DRAIN_NS = 100000000ull;
+__device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity) {
+  for (const unsigned long long t0 = gtime(); !mbar_try(bar, parity) && gtime() - t0 < DRAIN_NS;) {
+  }
+}
+// The MMAs that this warp's elected lane issued, by every issuing warp.  `bar` counts
+// one arrival per issuing warp and is used for nothing else.
 __device__ __forceinline__ void drain_mmas(uint32_t bar) {
   if (elect_one()) {
     mma_commit(bar);
-    for (const unsigned long long t0 = gtime(); !mbar_try(bar, 0) && gtime() - t0 < WAIT_NS;) {
-    }
+    drain_wait(bar, 0);
   }
   __syncwarp();
 }
