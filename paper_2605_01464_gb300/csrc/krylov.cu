@@ -373,8 +373,14 @@ cudaError_t launch_givens(double* H, long hstride, double* cs, double* sn, doubl
   return cudaGetLastError();
 }
 
-// Blocks of up to 64 KB: one block per basis vector is enough parallelism and
-// a phase is shorter than a launch.  Larger ones take a launch per phase.
+// Blocks of up to 64 KB in the cooperative kernel, larger ones a launch per phase.
+// Measured on both sides (times of whole unrestarted solves, launch per phase
+// divided by cooperative): 1.08 to 1.45 for 1 to 4 columns at 8192 numbers (2048 x
+// 1 to 512 x 4), 1.02 to 1.2 for 5 to 8 columns; even at 8192 numbers of 8 columns
+// and 8568 of 9; 0.95 at 238 x 12 (11424 numbers).  The line is a compromise: 12 to
+// 16 columns of 80 to 150 rows, where one block of 128 threads per row holds the
+// product in one wave, lose in the cooperative kernel (0.85 to 0.93), and 1 to 4
+// columns gain beyond the line too (1024 x 4 1.36, 2048 x 2 1.11).
 bool arnoldi_ok(long L, int m) { return skinny_ok(m) && L <= 8192; }
 
 cudaError_t launch_arnoldi(const Planes<const double>& A, int n, int m, double* V, double* W, double* h, long hlen,

@@ -47,9 +47,9 @@
 // pairs and K range over up to 16 parts, each with its own set of planes
 // (combined with the eight products, exactly).
 //
-// Measured (GB300): the 8-slice 2048^3 product 2.92 ms against 5.31 ms of the
-// 16-product kernel it replaced (1696 TFLOP/s issued of 1876 measured burst),
-// 4096^3 22.9 against 44.9 ms, 60 x 512 x 60 14 against 155 us.  What is left
+// Measured (GB300): the 8-slice 2048^3 product 2.89 ms against 5.31 ms of the
+// 16-product kernel it replaced (1710 TFLOP/s issued of 1957 measured burst),
+// 4096^3 23.9-24.3 against 44.9 ms, 60 x 512 x 60 14 against 155 us.  What is left
 // at 2048: 2048 items on 152 SMs fill 13.5 of 14 waves, and the MMA warp's
 // barrier waits between stages.
 #include <cuda.h>

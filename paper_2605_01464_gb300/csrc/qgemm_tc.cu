@@ -34,7 +34,7 @@
 // the component pair's operand traffic (64 bytes per cycle and SM at full rate)
 // and the last item's epilogue are what is left.
 // Every wait is bounded (2 s of globaltimer); on expiry the kernel records
-// an error code, stops issuing work, drains what it started and frees TMEM.
+// an error code, stops at its next work item, drains what it started and frees TMEM.
 #include <cuda.h>
 
 #include <algorithm>
